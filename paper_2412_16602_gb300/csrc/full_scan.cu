@@ -2007,11 +2007,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     auto info = [&](int sh, KernelInfo* ki, long long* resident) -> vmb_status {
         *ki = pick(a.dtype, np, sh, zoh);
         if (!ki->fn) return VMB_ERR_CUDA;
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ki->fn, ki->threads, ki->smem) != cudaSuccess)
-            return VMB_ERR_CUDA;
-        *resident = (long long)(per_sm < 1 ? 1 : per_sm) * sms;
-        return VMB_OK;
+        *resident = resident_ctas(ki->fn, ki->threads, ki->smem);
+        return *resident > 0 ? VMB_OK : VMB_ERR_CUDA;
     };
     // Rules measured on GB300 over the benchmark workloads: 16 states, L >= 128 and
     // at least 128 channel rows per SM -> the warp-specialised kernel when the tensors

@@ -776,11 +776,8 @@ vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
         if (forced && cand != forced) continue;
         KInfo ki = mpick(a.dtype, np, cand, zoh);
         if (!ki.fn) return VMB_ERR_CUDA;
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ki.fn, kThreads, a.D > 256 ? ki.smem2 : ki.smem) !=
-            cudaSuccess)
-            return VMB_ERR_CUDA;
-        const long long resident = (long long)(per_sm < 1 ? 1 : per_sm) * device_sm_count();
+        const long long resident = resident_ctas(ki.fn, kThreads, a.D > 256 ? ki.smem2 : ki.smem);
+        if (resident < 1) return VMB_ERR_CUDA;
         const long long ctas = seqs * ((a.L + cand - 1) / cand);
         const bool fills = a.D <= 256 ? 5 * ctas >= 4 * resident : ctas >= 2 * resident;
         if (forced || fills || cand == 32) {

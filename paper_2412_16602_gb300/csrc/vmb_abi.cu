@@ -34,6 +34,35 @@ int device_sm_count() {
     return n;
 }
 
+long long resident_ctas(const void* fn, int threads, size_t smem) {
+    struct Entry {
+        const void* fn;
+        size_t smem;
+        int dev, threads, per_sm;
+    };
+    constexpr int kMaxEntries = 512;  // above the number of kernel instances; a full table only stops keeping answers
+    static std::mutex mu;
+    static Entry table[kMaxEntries];
+    static int used = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    int per_sm = 0;
+    {
+        std::lock_guard<std::mutex> g(mu);
+        for (int i = 0; i < used && per_sm == 0; ++i) {
+            const Entry& e = table[i];
+            if (e.fn == fn && e.smem == smem && e.dev == dev && e.threads == threads) per_sm = e.per_sm;
+        }
+    }
+    if (per_sm == 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess) return 0;
+        if (per_sm < 1) per_sm = 1;
+        std::lock_guard<std::mutex> g(mu);
+        if (used < kMaxEntries) table[used++] = {fn, smem, dev, threads, per_sm};
+    }
+    return (long long)per_sm * device_sm_count();
+}
+
 namespace {
 
 bool mul_ok(long long a, long long b, long long* out) {

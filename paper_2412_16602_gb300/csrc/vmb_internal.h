@@ -137,6 +137,13 @@ struct MeanBwdArgs {
 
 int device_sm_count();
 
+// CTAs of a kernel that fit on the current device at once (at least one per
+// SM); 0 when the occupancy query fails.  The query costs about 2 us of host
+// time and its answer is fixed for a kernel, block size and shared-memory size,
+// so the answers are kept per device (a plan asks for up to eight, and a call
+// makes up to three plans: 25 of a small call's 48 us were these queries).
+long long resident_ctas(const void* fn, int threads, size_t smem);
+
 // The argument checks of the scan entry points (shapes, flags, pointers,
 // alignment); *empty is set for a problem with no elements.
 vmb_status validate_scan(const ScanArgs& a, bool mean, bool* empty);

@@ -124,7 +124,7 @@ def _dtype_code(t: torch.dtype) -> int:
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def _dev(t: torch.Tensor, name: str):
@@ -135,9 +135,9 @@ def _dev(t: torch.Tensor, name: str):
     return t
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 # ---------------------------------------------------------------- cross-scan / merge
