@@ -1919,7 +1919,7 @@ bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows
 
 // Tile shapes per padded state count, in order of preference (fewest lanes
 // per channel first).  The zero-order-hold variant uses the first shape.
-int shape_count(int np) { return np <= 4 ? 1 : np == 8 ? 2 : 20; }
+int shape_count(int np) { return np <= 4 ? 1 : np == 8 ? 2 : 23; }
 constexpr int kLanesShape = 7;   // index of the lane-per-state variant (N <= 16 padded to 16)
 constexpr int kChunkShape = 8;   // first index of the three-launch chunked variant (shapes 8 to 11)
 bool is_chunk_shape(int np, int shape) { return np == 16 && shape >= kChunkShape && shape < kChunkShape + 4; }
@@ -1929,6 +1929,11 @@ constexpr int kPackedShape = 16;  // first index of the packed streaming variant
 bool is_packed_shape(int np, int shape) { return np == 16 && shape >= kPackedShape && shape < kPackedShape + 3; }
 constexpr int kWsShape = 19;  // the warp-specialised variant (tensor copies; 16-byte rows and aligned tensors)
 bool is_ws_shape(int np, int shape) { return np == 16 && shape == kWsShape; }
+constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of an SM (a CTA also takes 1 KB of its own)
+constexpr int kSmallShape = 20;  // whole short sequences in shared memory (shapes 20 to 22: G = 1, 4, 16; small_map.cu)
+int small_lanes(int np, int shape) {
+    return np == 16 && shape >= kSmallShape && shape < kSmallShape + 3 ? 1 << (2 * (shape - kSmallShape)) : 0;
+}
 
 template <typename T, bool ZOH>
 KernelInfo pick_t(int np, int shape) {
@@ -1998,6 +2003,36 @@ ShapeRoles roles(int np) {
     return {0, 0, 0, 0};
 }
 
+// Lanes per channel with which short sequences take the whole-sequence kernel
+// (small_map.cu), 0 where another kernel is better.  `map`: the call is the
+// block from the map; `tma_ok`: the warp-specialised kernel can read the
+// tensors.  Measured on GB300 (fp32, us, block from the map unless said):
+//  - few rows: 16 lanes while the CTAs number at most two per SM (one 14x14 map
+//    of 192 channels 11.2, against 24.3 as cross-scan, lane-per-state scan and
+//    merge; 768 channels: 27.6, and 18.1 with 4 lanes), then 4 lanes up to three
+//    per SM, either only if they are all resident at once (batch 4 of 14x14x768,
+//    one CTA per SM and three waves: 51.8, warp-specialised 38.9);
+//  - many rows: one lane, where a warp's rows fit.  Rows that tensor copies
+//    cannot read: 7x7x768 at batch 32 38.1 against 130.5, the scan alone 39.0
+//    against 78.5; 11x11 137.8 against 283.6.  Rows that they can: the block
+//    while two CTAs fit an SM (8x8 47.7 against 72.6; 12x12, one CTA, 159
+//    against 111), the scan alone never (8x8 54.4 against 31.0).
+// One lane, the warp-specialised and the packed streaming kernel share their
+// arithmetic, so the block is bit-identical to the separate calls either way;
+// 4 and 16 lanes (other sums over the states) are taken by both or by neither.
+int small_rule(const ScanArgs& a, bool map, bool tma_ok, int sms) {
+    if (a.L > 256) return 0;
+    for (const int G : {16, 4}) {
+        const long long ctas = ((long long)a.B * a.K * ((a.D + 32 / G - 1) / (32 / G)) + 3) / 4;
+        const long long fit = (long long)(kSmemPerSm / (small_scan_smem(G, a.L, false) + 1024)) * sms;
+        const long long most = (G == 16 ? 2LL : 3LL) * sms;
+        if (ctas <= fit && ctas <= most) return G;
+    }
+    if (small_scan_smem(1, a.L, false) > kSmallMaxSmem) return 0;
+    if (!tma_ok) return 1;
+    return map && 2 * (small_scan_smem(1, a.L, true) + 1024) <= kSmemPerSm ? 1 : 0;
+}
+
 vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     if (a.N < 1 || a.N > 16) return VMB_ERR_UNSUPPORTED;
     const int np = pad_states(a.N);
@@ -2010,9 +2045,10 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         *resident = resident_ctas(ki->fn, ki->threads, ki->smem);
         return *resident > 0 ? VMB_OK : VMB_ERR_CUDA;
     };
-    // Rules measured on GB300 over the benchmark workloads: 16 states, L >= 128 and
-    // at least 128 channel rows per SM -> the warp-specialised kernel when the tensors
-    // allow tensor copies, else (at least 256 rows per SM) the packed streaming kernel; otherwise plenty of
+    // Rules measured on GB300 over the benchmark workloads: 16 states and short
+    // sequences -> the whole-sequence kernel (small_rule); at least 128 channel rows
+    // per SM (64 up to L = 1024) -> the warp-specialised kernel when the tensors
+    // allow tensor copies, else (at least 256 rows per SM and L >= 128) the packed streaming kernel; otherwise plenty of
     // rows -> one lane per channel; a fair number -> two lanes; too few -> cut L into
     // chunks: the three-launch variant (two lanes per channel, 32-step chunks)
     // while a grid of 64-step one-lane chunks would fit in two waves, else
@@ -2032,7 +2068,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     if (!zoh && forced_plan(&forced_shape, &forced_chunks)) {
         shape = forced_shape % shape_count(np);
         if (is_ws_shape(np, shape) && !tma_ok) shape = kPackedShape;
-        if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+        if (small_lanes(np, shape) && small_scan_smem(small_lanes(np, shape), a.L, false) > kSmallMaxSmem) shape = 0;
+        if (!small_lanes(np, shape) && (st = info(shape, &ki, &res)) != VMB_OK) return st;
         n_chunks = forced_chunks > 1 ? forced_chunks : 1;
     } else if (zoh) {
         if ((st = info(0, &ki, &res)) != VMB_OK) return st;
@@ -2041,10 +2078,15 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             const long long want = (res + tiles - 1) / tiles, mx = (a.L + 255) / 256;
             n_chunks = (int)(want < mx ? want : mx);
         }
-    } else if (tma_ok && rows >= 128LL * sms && a.L >= 128) {
+    } else if (const int G = np == 16 ? small_rule(a, a.gather_h > 0, tma_ok, sms) : 0) {
+        shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
+    } else if (tma_ok && rows >= (a.L <= 1024 ? 64LL : 128LL) * sms) {
         // a fair number of rows and tensors the tensor copies can read: the
         // warp-specialised kernel, one pass over L (measured on GB300: fastest
-        // from the batch-32 56x56 map, under a third of a wave of its tiles, up)
+        // from the batch-32 56x56 map, under a third of a wave of its tiles, up;
+        // of shorter sequences from half of that, where the alternatives are one
+        // lane per state or no tensor copies: 14x14x768 at batch 4 22.8 us
+        // against 34.4, 10x10x768 at batch 8 18.5 against 25.4)
         shape = kWsShape;
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
     } else if (np == 16 && rows >= 256LL * sms && a.L >= 128) {
@@ -2117,6 +2159,13 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             }
         }
     }
+    if (const int G = small_lanes(np, shape)) {
+        ki = KernelInfo{};
+        ki.G = G;
+        ki.DT = 32 / G;
+        ki.ts = a.L;
+        n_chunks = 1;
+    }
     if (is_chunk_shape(np, shape)) n_chunks = (a.L + ki.ts - 1) / ki.ts;  // chunks of exactly ts steps
     if (is_stream_shape(np, shape) || is_packed_shape(np, shape) || is_ws_shape(np, shape))
         n_chunks = 1;  // one pass over L
@@ -2143,6 +2192,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     *plan = p;
     return VMB_OK;
 }
+
+int full_plan_small(const ScanPlan& plan) { return small_lanes(plan.np, plan.split); }
 
 bool full_plan_gathers(const ScanPlan& plan) { return is_ws_shape(plan.np, plan.split); }
 
@@ -2189,6 +2240,7 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     const bool lowrank = a.R > 0;
     if ((lowrank || a.gather_h > 0) && !is_ws_shape(plan.np, plan.split)) return VMB_ERR_UNSUPPORTED;
     if (lowrank && a.gather_h > 0) return VMB_ERR_UNSUPPORTED;
+    if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream);
     KernelInfo ki = lowrank ? ws_lowrank_info(a.dtype, a.R)
                     : a.gather_h > 0 ? ws_gather_info(a.dtype)
                                      : pick(a.dtype, plan.np, plan.split, (a.flags & VMB_FLAG_B_ZOH) != 0);

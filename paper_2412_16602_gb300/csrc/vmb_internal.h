@@ -162,6 +162,13 @@ bool full_plan_gathers(const ScanPlan& plan);
 // out [B,K,D,L] (dtype) = Wup z, the raw Deltas of the low-rank form.
 vmb_status launch_lowrank_expand(const float* z, const float* Wup, void* out, int B, int K, int D, int R, int L,
                                  vmb_dtype dt, cudaStream_t stream);
+// Short sequences held whole in shared memory (small_map.cu): lanes per channel
+// of a plan that takes this kernel, 0 for the others; `map`: as the whole block.
+int full_plan_small(const ScanPlan& plan);
+constexpr size_t kSmallMaxSmem = 227 * 1024;
+size_t small_scan_smem(int G, int L, bool map);
+// out = null: the scan alone (a.u the sequences); else a.u is the map [B][D][H][W] and K = 4.
+vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream);
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
 vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W, vmb_dtype dt,
                              cudaStream_t stream);

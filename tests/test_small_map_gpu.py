@@ -1,0 +1,54 @@
+"""The whole-sequence kernel of short sequences (full-scan shapes 20 to 22: 1, 4
+and 16 lanes a channel), alone and as the one-launch block, against the fp64
+oracle; the block bit for bit against the three separate calls.  Sizes sit at
+the edges of its tiles: one step, lengths around the step blocks (4 and 16),
+the longest sequence of each rule, ragged channel tiles, padded states, bf16,
+odd rows and a plane one pixel wide."""
+import pytest
+
+import oracle
+import workloads
+from tests.parity import check, to_device, to_numpy
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU, skipped by marker
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import paper_2412_16602_gb300 as vmb  # noqa: E402
+
+DEV = torch.device("cuda", 0)
+
+SHAPES = [
+    # (B, D, N, H, W, dtype)
+    (1, 5, 16, 1, 1, "f32"),
+    (2, 33, 16, 1, 7, "f32"),
+    (1, 9, 16, 5, 3, "bf16"),
+    (3, 70, 16, 7, 7, "f32"),
+    (2, 40, 13, 4, 4, "bf16"),
+    (1, 34, 16, 17, 1, "f32"),
+    (2, 32, 9, 8, 12, "f32"),
+    (1, 19, 16, 16, 16, "f32"),
+    (8, 512, 16, 4, 4, "f32"),   # planner: the block with one lane a channel, the scan alone warp-specialised
+    (8, 500, 16, 3, 5, "bf16"),  # planner: one lane a channel for both
+]
+
+
+@pytest.mark.parametrize("plan", ["20", "21", "22", ""])
+@pytest.mark.parametrize("shape", SHAPES, ids=[f"B{s[0]}_D{s[1]}_N{s[2]}_{s[3]}x{s[4]}_{s[5]}" for s in SHAPES])
+def test_short_sequences(shape, plan, force_plan):
+    B, D, N, H, W, dt = shape
+    if plan:
+        force_plan.full(plan)
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=300 + D + N)
+    inp = workloads.make_inputs(wl, params="random")
+    g = to_device(inp, DEV)
+    args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+    y = vmb.vmb_selective_scan_fwd(vmb.vmb_cross_scan(g["x"]), *args, H, W)
+    out, ym = vmb.vmb_ss2d_full_fwd(g["x"], *args)
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    _, y_ref, out_ref = oracle.ss2d_full(inp)
+    check(to_numpy(y), y_ref, dt, "full y")
+    assert torch.equal(ym, y) and torch.equal(out, vmb.vmb_cross_merge(y, H, W))
+    check(to_numpy(out), out_ref, dt, "full out from the map")
