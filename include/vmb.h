@@ -116,8 +116,9 @@ vmb_status vmb_cross_merge(const void* ys, void* out, int B, int D, int H, int W
  * vmb_scan_workspace_bytes - bytes of zero-initialised device workspace that
  * vmb_selective_scan_fwd (path VMB_PATH_FULL) or vmb_mean_scan_fwd
  * (VMB_PATH_MEAN) needs for this problem on the current device, under any
- * flags (the larger of the plans of the two Bbar forms, which differ in tile
- * shape and chunking).  Always >= 256 (the status header).  The workspace
+ * flags and for any alignment of the tensors (the largest of the plans of the two
+ * Bbar forms and of aligned and unaligned rows, which differ in tile shape and
+ * chunking).  Always >= 256 (the status header).  The workspace
  * holds the status word and the chunk-carry exchange of the L-chunked scans.
  *
  * The workspace must be zero-filled once before its first use (cudaMemset or
@@ -130,8 +131,8 @@ size_t vmb_scan_workspace_bytes(int path, int B, int K, int D, int N, int H, int
 /*
  * vmb_scan_kernel_count - number of kernels one vmb_selective_scan_fwd
  * (VMB_PATH_FULL) or vmb_mean_scan_fwd (VMB_PATH_MEAN) call launches for this
- * problem on the current device: 1, or 3 for the L-chunked full scan that
- * resolves the chunk carry in launches of its own.  0 for an empty problem or
+ * problem on the current device: 1, or 2 or 3 for the L-chunked full scans that
+ * hand the chunk carry from launch to launch.  0 for an empty problem or
  * invalid arguments.  (vmb_mean_scan_merge_fwd launches the mean scan's
  * kernels plus one merge kernel.)  Bookkeeping for timing tools; the paper
  * has no counterpart.

@@ -27,37 +27,11 @@
 #include <mutex>
 #include <type_traits>
 
-#include "vmb_common.cuh"
+#include "full_common.cuh"
 #include "vmb_internal.h"
 
 namespace vmb {
 namespace {
-
-struct FullParams {
-    const void* u;
-    const void* dl;
-    const float* A;
-    const void* Bs;
-    const void* Cs;
-    const float* Dskip;
-    const float* bias;
-    void* y;
-    int K, D, N, L;
-    int softplus_on;
-    int tiles_per_bk, n_tiles, n_chunks, chunk_len;
-    int vec;       // rows are 16-byte aligned: cp.async 16-byte path and vector stores
-    int suppress;  // test hook: chunk 0 does not publish
-    int gather_h;  // > 0: u is gathered from the map x and its transpose (warp-specialised variant only)
-    const float* Wup;  // low-rank Delta (warp-specialised variant only): dl is z [B*K][R][L] fp32 and
-    int R;             // delta_raw[b,k,d,l] = sum_r Wup[k,d,r] z[b,k,r,l]
-    WsHeader* hdr;
-    unsigned* flags;
-    float* aggP;   // per chunk: sum of delta per channel (DT floats, rest unused)
-    float* aggH;
-    float* incH;
-};
-
-__host__ __device__ constexpr size_t a16(size_t v) { return (v + 15) / 16 * 16; }
 
 // Tile shape: G lanes per channel, DT channels per CTA, TS steps per stage
 // (0: one 16-byte chunk per row), NSTG stages in the cp.async ring, and the
@@ -83,22 +57,6 @@ struct Layout {
     static_assert(bytes <= 100 * 1024, "full-scan tile must leave room for two CTAs per SM");
 };
 
-// Four consecutive elements of one row as fp32 (16-byte / 8-byte aligned reads).
-__device__ __forceinline__ void load4(const float* p, float (&v)[4]) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = q.z;
-    v[3] = q.w;
-}
-__device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4]) {
-    const uint2 q = *reinterpret_cast<const uint2*>(p);
-    v[0] = __uint_as_float(q.x << 16);
-    v[1] = __uint_as_float(q.x & 0xffff0000u);
-    v[2] = __uint_as_float(q.y << 16);
-    v[3] = __uint_as_float(q.y & 0xffff0000u);
-}
-
 // NG consecutive fp32 values from shared memory (16-byte aligned when NG >= 4).
 template <int NG>
 __device__ __forceinline__ void load_states(const float* p, float (&v)[NG]) {
@@ -119,32 +77,6 @@ __device__ __forceinline__ void load_states(const float* p, float (&v)[NG]) {
 
 __device__ __forceinline__ float sel4(const float (&v)[4], int j) {
     return j == 0 ? v[0] : j == 1 ? v[1] : j == 2 ? v[2] : v[3];
-}
-
-// Store n consecutive outputs of one row (n = 4, 2 or 1), vectorised when aligned.
-template <typename T, int NV>
-__device__ __forceinline__ void store_row(T* dst, const float (&v)[NV], int nvalid_here, bool vec) {
-    if (vec && nvalid_here >= NV) {
-        if constexpr (sizeof(T) == 4 && NV == 4) {
-            *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-            return;
-        } else if constexpr (sizeof(T) == 4 && NV == 2) {
-            *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
-            return;
-        } else if constexpr (sizeof(T) == 2 && NV == 4) {
-            const unsigned lo = __bfloat16_as_ushort(io<T>::to(v[0])) | ((unsigned)__bfloat16_as_ushort(io<T>::to(v[1])) << 16);
-            const unsigned hi = __bfloat16_as_ushort(io<T>::to(v[2])) | ((unsigned)__bfloat16_as_ushort(io<T>::to(v[3])) << 16);
-            *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
-            return;
-        } else if constexpr (sizeof(T) == 2 && NV == 2) {
-            *reinterpret_cast<unsigned*>(dst) =
-                __bfloat16_as_ushort(io<T>::to(v[0])) | ((unsigned)__bfloat16_as_ushort(io<T>::to(v[1])) << 16);
-            return;
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j)
-        if (j < nvalid_here) dst[j] = io<T>::to(v[j]);
 }
 
 // Copy kTS steps (from l0) of DT u and delta rows and of the NP B (and C) rows
@@ -1445,281 +1377,6 @@ __global__ void __launch_bounds__(PackedLayout<T, PS>::THREADS, PS::MINB) full_p
     cp_async_wait<0>();
 }
 
-// ------------------------------------- warp-specialised variant (tensor copies)
-// The packed state update of the streaming variant, with the tile movement
-// taken off the compute warps.  A CTA is CW consumer warps (one channel per
-// lane, all 16 states in registers) and one producer warp.  The producer
-// issues, per stage of TS steps, four tiled tensor copies (u and delta:
-// DT rows x TS steps, B and C: 16 rows x TS steps) into an NSTG-deep ring
-// and, once a stage has landed, converts its B and C rows into fp32
-// [t][B0..15, C0..15] rows for broadcast reads.  Stages are handed over with
-// mbarriers (landed / ready / released), so no barrier spans the CTA and the
-// copies of the next stages overlap the consumers' arithmetic.  Each
-// consumer lane computes delta = softplus(raw + bias) of its own row of the
-// stage, runs the packed update (the same operations, in the same order, as
-// full_packed_kernel: its y is bit-identical) and stores y from registers.
-// Requires rows of 16-byte multiples and 16-byte aligned tensors (the host
-// picks this variant only then); every wait is bounded.
-// Gathering from the map (p.gather_h > 0, App. A cross-scan without the
-// cross-scanned sequences): direction k's u rows are the (b, d) planes of x
-// (k = 0, 2) or of its transpose xt (k = 1, 3), and the reversed directions
-// (k = 2, 3) load the mirrored box, steps [L - (s+1) TS, L - s TS), and read
-// it from the end, so each step sees the value the cross-scan would have put
-// there (the same operations: y is bit-identical to the scan of xs).
-// Low-rank Delta (RP > 0, Eq. 6's s_Delta = Linear_D(Linear_R(u)) with the
-// rank-R expansion fused into the scan): the second box of a stage is z
-// (16 rows x TS steps, fp32, rows past R zero) instead of the raw Deltas, and
-// each consumer lane forms its channel's raw Delta per step as
-// sum_r Wup[k,d,r] z_r (r in order, as the selection kernel's epilogue does,
-// so fp32 results are bit-identical to selection -> raw Deltas -> scan), with
-// its Wup row (RP >= R values, zero-padded) in registers.
-template <int CW_, int TS_, int NSTG_, int MINB_, int RP_ = 0, bool GATHER_ = false>
-struct WsShape {
-    static constexpr int CW = CW_, TS = TS_, NSTG = NSTG_, MINB = MINB_, RP = RP_;
-    static constexpr bool GATHER = GATHER_;  // u gathered from the map (see above)
-};
-
-struct TensorMaps {
-    CUtensorMap u, dl, B, C;  // [B*K][D][L] (u, delta) and [B*K][N][L] (B, C)
-    CUtensorMap u2;           // gathering from the map: u is x [B][D][L] and u2 its transpose xt
-};
-
-template <typename T, class WS>
-struct WsTileLayout {
-    static constexpr int CW = WS::CW, DT = 32 * CW, NP = 16, TS = WS::TS, NSTG = WS::NSTG;
-    static constexpr int THREADS = DT + 32;
-    static constexpr int U_BYTES = DT * TS * (int)sizeof(T);   // one u (or delta) box
-    static constexpr int DL_BYTES = WS::RP ? NP * TS * 4 : U_BYTES;  // the delta box, or the z box (fp32)
-    static constexpr int BC_BYTES = NP * TS * (int)sizeof(T);  // one B (or C) box
-    static constexpr int B_OFF = U_BYTES + DL_BYTES;            // B box within a stage (C follows)
-    static constexpr int RAW_STAGE = U_BYTES + DL_BYTES + 2 * BC_BYTES;
-    static constexpr int BCT_STAGE = TS * 2 * NP * 4;           // fp32 [TS][B0..15, C0..15]
-    static constexpr size_t bct_off = (size_t)NSTG * RAW_STAGE;
-    static constexpr size_t wup_off = bct_off + (size_t)NSTG * BCT_STAGE;  // low rank: fp32 [DT][RP + 1] Wup rows
-    static constexpr size_t bar_off = wup_off + (WS::RP ? (size_t)DT * (WS::RP + 1) * 4 : 0);
-    static constexpr size_t bytes = bar_off + (size_t)3 * NSTG * 8;
-    static_assert(U_BYTES % 128 == 0 && BC_BYTES % 128 == 0 && TS % 4 == 0 && TS * sizeof(T) % 16 == 0,
-                  "tensor-copy boxes: 16-byte rows, 128-byte aligned boxes");
-};
-
-constexpr uint64_t kStageWaitNs = 1000000000ull;  // 1 s per stage hand-over
-
-template <typename T, class WS>
-__global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
-    full_ws_kernel(const FullParams p, const __grid_constant__ TensorMaps tm) {
-    pdl_wait();
-    pdl_launch_dependents();
-    using LY = WsTileLayout<T, WS>;
-    constexpr int DT = LY::DT, NP = 16, TS = LY::TS, NSTG = LY::NSTG, NPR = NP / 2;
-    extern __shared__ __align__(128) unsigned char smem_ws[];
-    unsigned char* smem = smem_ws;
-    const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar0 = sbase + (uint32_t)LY::bar_off;
-    // landed[i]: the four copies of the stage in slot i arrived; ready[i]: its
-    // B/C rows are converted; released[i]: every consumer warp is done with it
-    auto landed = [&](int i) { return bar0 + 8u * i; };
-    auto ready = [&](int i) { return bar0 + 8u * (NSTG + i); };
-    auto released = [&](int i) { return bar0 + 8u * (2 * NSTG + i); };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile = blockIdx.x;
-    const int bk = tile / p.tiles_per_bk;
-    const int d0 = (tile % p.tiles_per_bk) * DT;
-    const int k = bk % p.K;
-    const int L = p.L;
-    const int nst = (L + TS - 1) / TS;
-    const int cwarps = min(LY::CW, (p.D - d0 + 31) / 32);  // consumer warps with at least one channel
-    if (tid == 0) {
-        for (int i = 0; i < NSTG; ++i) {
-            mbarrier_init(landed(i), 1);
-            mbarrier_init(ready(i), 32);
-            mbarrier_init(released(i), cwarps);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    if (warp == LY::CW) {
-        // ------------------------------------------------------ producer warp
-        // u: the rows of (b, k), or gathered from x / xt (see above)
-        constexpr bool gather = WS::GATHER;
-        const CUtensorMap* um = (gather && (k & 1)) ? &tm.u2 : &tm.u;
-        const int uz = gather ? bk / p.K : bk;
-        const bool urev = gather && k >= 2;
-        int issued = 0;  // stages whose copies have been issued (0 .. issued-1)
-        auto issue = [&](int s) {
-            issued = s + 1;
-            const int slot = s % NSTG;
-            const uint32_t dst = sbase + (uint32_t)(slot * LY::RAW_STAGE);
-            mbarrier_expect_tx(landed(slot), (unsigned)LY::RAW_STAGE);
-            tma_load_3d(dst, um, urev ? L - (s + 1) * TS : s * TS, d0, uz, landed(slot));
-            tma_load_3d(dst + LY::U_BYTES, &tm.dl, s * TS, WS::RP ? 0 : d0, bk, landed(slot));
-            tma_load_3d(dst + LY::B_OFF, &tm.B, s * TS, 0, bk, landed(slot));
-            tma_load_3d(dst + LY::B_OFF + LY::BC_BYTES, &tm.C, s * TS, 0, bk, landed(slot));
-        };
-        if (lane == 0)
-            for (int s = 0; s < NSTG && s < nst; ++s) issue(s);
-        issued = __shfl_sync(0xffffffffu, issued, 0);
-        int seen = 0;  // stages whose copies this warp has seen land
-        bool ok = true;
-        // (every wait's outcome is made warp-uniform, so that no lane leaves a
-        // loop whose warp-wide operations the others still execute)
-        for (int s = 0; s < nst; ++s) {
-            const int slot = s % NSTG;
-            if (!(ok = __all_sync(0xffffffffu, mbarrier_wait(landed(slot), (s / NSTG) & 1, kStageWaitNs)))) break;
-            seen = s + 1;
-            // lane r converts row r of [B rows 0..15, C rows 0..15] into column r
-            const T* rb = reinterpret_cast<const T*>(smem + slot * LY::RAW_STAGE + LY::B_OFF) + lane * TS;
-            float* bo = reinterpret_cast<float*>(smem + LY::bct_off + slot * LY::BCT_STAGE);
-#pragma unroll
-            for (int t = 0; t < TS; ++t) bo[t * 2 * NP + lane] = io<T>::cvt(rb[t]);
-            __syncwarp();
-            // (test hook: the first stage is never handed over, so every wait on it runs out)
-            if (!(p.suppress && s == 0)) mbarrier_arrive(ready(slot));
-            // refill the slot of stage s - 1 once the consumers released it
-            if (s >= 1 && s - 1 + NSTG < nst) {
-                const int ps = (s - 1) % NSTG;
-                if (!(ok = __all_sync(0xffffffffu, mbarrier_wait(released(ps), ((s - 1) / NSTG) & 1, kStageWaitNs))))
-                    break;
-                if (lane == 0) issue(s - 1 + NSTG);
-                issued = __shfl_sync(0xffffffffu, issued, 0);
-            }
-        }
-        if (!ok) {
-            if (lane == 0) atomicOr(&p.hdr->err, kErrTimeout);
-            // every copy issued must land before the CTA exits
-            for (int s = seen; s < issued; ++s) mbarrier_wait(landed(s % NSTG), (s / NSTG) & 1, kStageWaitNs);
-        }
-        return;
-    }
-    if (warp >= cwarps) return;  // a tile's channels past D: no work, not counted by `released`
-    // -------------------------------------------------------- consumer warps
-    const bool urev = WS::GATHER && k >= 2;  // u arrives mirrored (see above)
-    const int c = tid;
-    const int d = d0 + c;
-    const bool cval = d < p.D;
-    const size_t row0 = (size_t)bk * p.D + d0;
-    const float bias = cval ? p.bias[(size_t)k * p.D + d] : 0.0f;
-    const float dsk = cval ? p.Dskip[(size_t)k * p.D + d] : 0.0f;
-    const float* Ad = p.A + ((size_t)k * p.D + d) * p.N;
-    float2 A2[NPR], h[NPR];
-#pragma unroll
-    for (int i = 0; i < NPR; ++i) {
-        const int n = 2 * i;
-        A2[i] = make_float2((cval && n < p.N) ? Ad[n] * kLog2e : 0.0f, (cval && n + 1 < p.N) ? Ad[n + 1] * kLog2e : 0.0f);
-        h[i] = make_float2(0.0f, 0.0f);
-    }
-    T* yrow = static_cast<T*>(p.y) + (row0 + c) * (size_t)L;
-    constexpr int RP = WS::RP > 0 ? WS::RP : 1;
-    // low rank: this channel's Wup row, in the lane's own shared-memory row (a
-    // padded stride: conflict-free) to leave the registers to the states
-    float* wr = reinterpret_cast<float*>(smem + LY::wup_off) + c * (RP + 1);
-    if constexpr (WS::RP > 0) {
-#pragma unroll
-        for (int r = 0; r < RP; ++r) wr[r] = (cval && r < p.R) ? p.Wup[((size_t)k * p.D + d) * p.R + r] : 0.0f;
-    }
-    for (int s = 0; s < nst; ++s) {
-        const int slot = s % NSTG;
-        if (!__all_sync(0xffffffffu, mbarrier_wait(ready(slot), (s / NSTG) & 1, kStageWaitNs))) {
-            if (lane == 0) atomicOr(&p.hdr->err, kErrTimeout);
-            return;
-        }
-        const int l0 = s * TS;
-        const int nvalid = min(TS, L - l0);
-        const T* ru = reinterpret_cast<const T*>(smem + slot * LY::RAW_STAGE) + c * TS;
-        const T* rd = reinterpret_cast<const T*>(smem + slot * LY::RAW_STAGE + LY::U_BYTES) + c * TS;
-        float uv[TS], dv[TS];
-#pragma unroll
-        for (int j = 0; j < TS; j += 4) {
-            float q[4], w[4];
-            if (urev) {
-                // the mirrored box, read from its end
-                load4(ru + TS - 4 - j, q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) uv[j + e] = q[3 - e];
-            } else {
-                load4(ru + j, q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) uv[j + e] = q[e];
-            }
-            if constexpr (WS::RP == 0) {
-                load4(rd + j, w);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) dv[j + e] = w[e] + bias;
-            }
-        }
-        if constexpr (WS::RP > 0) {
-            // raw Delta = sum_r Wup[r] z_r, r in order (the z rows are broadcast reads)
-            const float* zr = reinterpret_cast<const float*>(smem + slot * LY::RAW_STAGE + LY::U_BYTES);
-            // (packed: each lane of a pair is the same fused multiply-add as fmaf)
-            float2 raw[TS / 2];
-#pragma unroll
-            for (int j = 0; j < TS / 2; ++j) raw[j] = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int r = 0; r < RP; ++r) {
-                if (r < p.R) {
-                    const float2 w2 = make_float2(wr[r], wr[r]);
-#pragma unroll
-                    for (int j = 0; j < TS; j += 4) {
-                        const float4 z4 = *reinterpret_cast<const float4*>(zr + r * TS + j);
-                        raw[j / 2] = __ffma2_rn(w2, make_float2(z4.x, z4.y), raw[j / 2]);
-                        raw[j / 2 + 1] = __ffma2_rn(w2, make_float2(z4.z, z4.w), raw[j / 2 + 1]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < TS; j += 2) {
-                dv[j] = raw[j / 2].x + bias;
-                dv[j + 1] = raw[j / 2].y + bias;
-            }
-        }
-        if (p.softplus_on) {
-#pragma unroll
-            for (int j = 0; j < TS; j += 2) {
-                const float2 v = softplus2(make_float2(dv[j], dv[j + 1]));
-                dv[j] = v.x;
-                dv[j + 1] = v.y;
-            }
-        }
-        const float* bct = reinterpret_cast<const float*>(smem + LY::bct_off + slot * LY::BCT_STAGE);
-#pragma unroll
-        for (int t0 = 0; t0 < TS; t0 += 4) {
-            float yp[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 dd = make_float2(dv[t0 + j], dv[t0 + j]);
-                const float du = dv[t0 + j] * uv[t0 + j];
-                const float2 uu = make_float2(du, du);
-                const float* bt = bct + (t0 + j) * 2 * NP;
-                float2 ya = make_float2(0.0f, 0.0f);
-#pragma unroll
-                for (int q = 0; q < NP / 4; ++q) {
-                    const float4 b = *reinterpret_cast<const float4*>(bt + 4 * q);
-                    const float4 cc = *reinterpret_cast<const float4*>(bt + NP + 4 * q);
-                    {
-                        const float2 x = __fmul2_rn(dd, A2[2 * q]);
-                        const float2 a = make_float2(ex2(x.x), ex2(x.y));
-                        h[2 * q] = __ffma2_rn(a, h[2 * q], __fmul2_rn(uu, make_float2(b.x, b.y)));
-                        ya = __ffma2_rn(make_float2(cc.x, cc.y), h[2 * q], ya);
-                    }
-                    {
-                        const float2 x = __fmul2_rn(dd, A2[2 * q + 1]);
-                        const float2 a = make_float2(ex2(x.x), ex2(x.y));
-                        h[2 * q + 1] = __ffma2_rn(a, h[2 * q + 1], __fmul2_rn(uu, make_float2(b.z, b.w)));
-                        ya = __ffma2_rn(make_float2(cc.z, cc.w), h[2 * q + 1], ya);
-                    }
-                }
-                yp[j] = ya.x + ya.y;
-            }
-            float o[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) o[j] = fmaf(dsk, uv[t0 + j], yp[j]);
-            if (cval) store_row<T, 4>(yrow + l0 + t0, o, nvalid - t0, true);
-        }
-        __syncwarp();
-        if (lane == 0) mbarrier_arrive(released(slot));
-    }
-}
-
 // Launch 2 of the chunked variant: the inclusive state after every chunk,
 // inc_m = 2^(A_n log2 e S_m) inc_{m-1} + H_m from inc_{-1} = 0, for every
 // (channel, state) of a tile.  The chain is short in arithmetic but long in
@@ -1793,6 +1450,7 @@ struct KernelInfo {
     int G, DT, threads, ts;
     const void* agg = nullptr;  // chunked variant: the aggregate kernel (launch 1)
     bool tma = false;           // warp-specialised variant: takes the tensor maps of u, delta, B and C
+    int slot_bytes = 0;         // its shared memory per ring slot
 };
 
 template <typename T, int NP, class SH, bool ZOH>
@@ -1859,31 +1517,33 @@ KernelInfo packed_info() {
     return {attr_err == cudaSuccess ? fn : nullptr, LY::bytes, LY::G, LY::DT, LY::THREADS, LY::TS};
 }
 
-template <typename T, class WS>
-KernelInfo ws_info() {
-    using LY = WsTileLayout<T, WS>;
-    const void* fn = reinterpret_cast<const void*>(&full_ws_kernel<T, WS>);
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
-    });
-    KernelInfo ki{attr_err == cudaSuccess ? fn : nullptr, LY::bytes, 1, LY::DT, LY::THREADS, LY::TS};
+constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of an SM (a CTA also takes 1 KB of its own)
+
+// An instance of the warp-specialised kernel (full_ws.cuh) with kWsMinSlots ring
+// slots, the depth its occupancy is planned with.
+constexpr int kWsMinSlots = 4, kWsMaxSlots = 16;
+KernelInfo ws_info(vmb_dtype dt, int np, int variant, bool gather = false, int R = 0) {
+    const WsKernel w = dt == VMB_BF16 ? ws_kernel_bf16(np, variant, gather, R) : ws_kernel_f32(np, variant, gather, R);
+    KernelInfo ki{w.fn, (size_t)w.per_slot * kWsMinSlots + w.fixed, w.G, w.DT, w.threads, w.ts};
     ki.tma = true;
+    ki.slot_bytes = w.per_slot;
     return ki;
 }
 
-// The gathering instance of the warp-specialised kernel (u from the map).
-KernelInfo ws_gather_info(vmb_dtype dt) {
-    return dt == VMB_BF16 ? ws_info<__nv_bfloat16, WsShape<4, 8, 4, 4, 0, true>>()
-                          : ws_info<float, WsShape<4, 8, 4, 4, 0, true>>();
-}
-
-// The low-rank-Delta instance of the warp-specialised kernel for rank <= RP.
-KernelInfo ws_lowrank_info(vmb_dtype dt, int R) {
-    if (dt == VMB_BF16)
-        return R <= 8 ? ws_info<__nv_bfloat16, WsShape<4, 8, 4, 4, 8>>() : ws_info<__nv_bfloat16, WsShape<4, 8, 4, 4, 16>>();
-    return R <= 8 ? ws_info<float, WsShape<4, 8, 4, 4, 8>>() : ws_info<float, WsShape<4, 8, 4, 4, 16>>();
+// Ring slots of a launch of `grid` CTAs: what the shared memory of an SM holds
+// for the CTAs it gets.  With one or two CTAs on an SM four slots leave too few
+// bytes in flight (GB300, 8 maps of 56x56x512 fp32, one CTA per SM: 332 us with
+// four slots, the copies' latency; see the rule in plan_full).
+int ws_slots(const KernelInfo& ki, long long grid, int sms) {
+    const long long resident = resident_ctas(ki.fn, ki.threads, ki.smem);
+    long long per_sm = (grid + sms - 1) / sms;
+    if (resident > 0 && per_sm * sms > resident) per_sm = resident / sms;
+    if (per_sm < 1) per_sm = 1;
+    const long long fixed = (long long)ki.smem - (long long)ki.slot_bytes * kWsMinSlots;
+    long long cap = (long long)kSmemPerSm / per_sm - 1024;
+    if (cap > (long long)kSmallMaxSmem) cap = (long long)kSmallMaxSmem;
+    const long long n = (cap - fixed) / ki.slot_bytes;
+    return (int)(n < kWsMinSlots ? kWsMinSlots : n > kWsMaxSlots ? kWsMaxSlots : n);
 }
 
 // The driver's tensor-map encoder, looked up once (null when unavailable).
@@ -1903,8 +1563,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // Tensor map of `planes` row-major [rows][L] slabs of u, delta, B or C, read
 // in boxes of box_rows rows x box_ts steps (rows past `rows` and steps past L
 // read as zero).
+// `swizzled`: the 16-byte pieces of 32- and 64-byte rows swizzled (full_ws.cuh).
 bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows, long long planes, int box_ts,
-                 int box_rows) {
+                 int box_rows, bool swizzled = false) {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return false;
     const cuuint64_t es = dt == VMB_BF16 ? 2 : 4;
@@ -1913,13 +1574,16 @@ bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows
     const cuuint32_t box[3] = {(cuuint32_t)box_ts, (cuuint32_t)box_rows, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, dt == VMB_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
-               const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               swizzled && box_ts * es == 64   ? CU_TENSOR_MAP_SWIZZLE_64B
+               : swizzled && box_ts * es == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                               : CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Tile shapes per padded state count, in order of preference (fewest lanes
 // per channel first).  The zero-order-hold variant uses the first shape.
-int shape_count(int np) { return np <= 4 ? 1 : np == 8 ? 2 : 23; }
+int shape_count(int np) { return np <= 4 ? 2 : np == 8 ? 3 : 24; }
 constexpr int kLanesShape = 7;   // index of the lane-per-state variant (N <= 16 padded to 16)
 constexpr int kChunkShape = 8;   // first index of the three-launch chunked variant (shapes 8 to 11)
 bool is_chunk_shape(int np, int shape) { return np == 16 && shape >= kChunkShape && shape < kChunkShape + 4; }
@@ -1927,9 +1591,14 @@ constexpr int kStreamShape = 12;  // first index of the streaming one-lane varia
 bool is_stream_shape(int np, int shape) { return np == 16 && shape >= kStreamShape && shape < kStreamShape + 4; }
 constexpr int kPackedShape = 16;  // first index of the packed streaming variant (shapes 16 to 18: G = 1, 2, 4)
 bool is_packed_shape(int np, int shape) { return np == 16 && shape >= kPackedShape && shape < kPackedShape + 3; }
-constexpr int kWsShape = 19;  // the warp-specialised variant (tensor copies; 16-byte rows and aligned tensors)
-bool is_ws_shape(int np, int shape) { return np == 16 && shape == kWsShape; }
-constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of an SM (a CTA also takes 1 KB of its own)
+// The warp-specialised variant (tensor copies; 16-byte rows and aligned tensors): the
+// last shape of fewer states; 16 states: one lane per channel (19) or two (23).
+constexpr int kWsShape = 19, kWsTwoShape = 23;
+int ws_shape(int np) { return np <= 4 ? 1 : np == 8 ? 2 : kWsShape; }
+bool is_ws_shape(int np, int shape) {
+    return shape == ws_shape(np) || (np == 16 && shape == kWsTwoShape);
+}
+int ws_variant(int np, int shape) { return np == 16 && shape == kWsTwoShape ? kWsTwoLanes : kWsOneLane; }
 constexpr int kSmallShape = 20;  // whole short sequences in shared memory (shapes 20 to 22: G = 1, 4, 16; small_map.cu)
 int small_lanes(int np, int shape) {
     return np == 16 && shape >= kSmallShape && shape < kSmallShape + 3 ? 1 << (2 * (shape - kSmallShape)) : 0;
@@ -1965,13 +1634,13 @@ KernelInfo pick_t(int np, int shape) {
         case 16: return packed_info<T, PackedShape<1, 128, 5, 8, 3>>();
         case 17: return packed_info<T, PackedShape<2, 64, 5, 8, 3>>();
         case 18: return packed_info<T, PackedShape<4, 32, 5, 8, 3>>();
-        case 19: return ws_info<T, WsShape<4, 8, 4, 4>>();
         default: return info_for<T, 16, Shape<1, 128, 0, 3, 7>, ZOH>();
         }
     }
 }
 
 KernelInfo pick(vmb_dtype dt, int np, int shape, bool zoh) {
+    if (!zoh && is_ws_shape(np, shape)) return ws_info(dt, np, ws_variant(np, shape));
     if (dt == VMB_BF16) return zoh ? pick_t<__nv_bfloat16, true>(np, shape) : pick_t<__nv_bfloat16, false>(np, shape);
     return zoh ? pick_t<float, true>(np, shape) : pick_t<float, false>(np, shape);
 }
@@ -2018,8 +1687,10 @@ ShapeRoles roles(int np) {
 //    while two CTAs fit an SM (8x8 47.7 against 72.6; 12x12, one CTA, 159
 //    against 111), the scan alone never (8x8 54.4 against 31.0).
 // One lane, the warp-specialised and the packed streaming kernel share their
-// arithmetic, so the block is bit-identical to the separate calls either way;
-// 4 and 16 lanes (other sums over the states) are taken by both or by neither.
+// arithmetic, so the block is bit-identical to the separate calls either way
+// (where the block may take one lane the scan alone keeps to one lane and one
+// pass); 4 and 16 lanes (other sums over the states) are taken by both or by neither.
+bool small_map_one_lane(int L) { return 2 * (small_scan_smem(1, L, true) + 1024) <= kSmemPerSm; }
 int small_rule(const ScanArgs& a, bool map, bool tma_ok, int sms) {
     if (a.L > 256) return 0;
     for (const int G : {16, 4}) {
@@ -2030,7 +1701,32 @@ int small_rule(const ScanArgs& a, bool map, bool tma_ok, int sms) {
     }
     if (small_scan_smem(1, a.L, false) > kSmallMaxSmem) return 0;
     if (!tma_ok) return 1;
-    return map && 2 * (small_scan_smem(1, a.L, true) + 1024) <= kSmemPerSm ? 1 : 0;
+    return map && small_map_one_lane(a.L) ? 1 : 0;
+}
+
+// Estimated time (ns) of the warp-specialised kernel, and the number of chunks
+// it would take (1: one pass).  A CTA takes a fixed time per step that grows
+// with the CTAs that share an SM; cut into P + 1 chunks, P CTAs a tile run
+// concurrently and each passes over two chunks.  ns per step with one, two and
+// three CTAs per SM, measured on GB300 (fp32, 56x56 maps): 16 states, two lanes a
+// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8).
+double ws_estimate(int np, long long tiles, int L, int sms, int ts, int* chunks) {
+    const double per_step[4][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {51, 79, 111}};
+    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 : 3];
+    double best = 0.0;
+    for (int P = 1; P <= 24; ++P) {
+        if (P > 1 && L / (P + 1) < 4 * ts) break;
+        const long long per_sm = (tiles * P + sms - 1) / sms;
+        const long long waves = (per_sm + 2) / 3;
+        const double step = c[per_sm > 2 ? 2 : per_sm - 1] * waves;
+        // two launches, and the second one folds up to P - 1 aggregates
+        const double t = P == 1 ? L * step : 2.0 * L / (P + 1) * step + 6000.0 + 300.0 * P;
+        if (P == 1 || t < best) {
+            best = t;
+            *chunks = P == 1 ? 1 : P + 1;
+        }
+    }
+    return best;
 }
 
 vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
@@ -2045,29 +1741,47 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         *resident = resident_ctas(ki->fn, ki->threads, ki->smem);
         return *resident > 0 ? VMB_OK : VMB_ERR_CUDA;
     };
-    // Rules measured on GB300 over the benchmark workloads: 16 states and short
-    // sequences -> the whole-sequence kernel (small_rule); at least 128 channel rows
-    // per SM (64 up to L = 1024) -> the warp-specialised kernel when the tensors
-    // allow tensor copies, else (at least 256 rows per SM and L >= 128) the packed streaming kernel; otherwise plenty of
-    // rows -> one lane per channel; a fair number -> two lanes; too few -> cut L into
-    // chunks: the three-launch variant (two lanes per channel, 32-step chunks)
-    // while a grid of 64-step one-lane chunks would fit in two waves, else
-    // look-back chunks with one lane per channel when they stay long (>= 256
-    // steps) and the widest split otherwise (>= 128 steps).
+    // Rules measured on GB300.  16 states and short sequences -> the whole-sequence
+    // kernel (small_rule).  Tensors that tensor copies can read, at least two
+    // channel rows per SM -> the warp-specialised kernel: one lane per channel from
+    // 256 rows per SM on, two lanes below (16 states, fp32, us: 24576 rows of 56x56
+    // 350 with two lanes, 471 with one; 49152 rows of 28x28 168 and 163), L cut into
+    // chunks where ws_estimate expects a gain (6144 rows of 128x128 bf16 605, one
+    // pass 1126, look-back chunks 870; 3072 rows of 56x56 80, look-back 187; one state, 131072 rows
+    // of 56x56 779, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
+    // the three-launch chunked variant while a grid of 64-step one-lane chunks
+    // fits in two waves (768 rows of 56x56 30.2, chunked warp-specialised 34.8; at 1536
+    // rows 56.9 and 46.6).  Other tensors: at least 256 rows per SM and L >= 128 ->
+    // the packed streaming kernel; otherwise plenty of rows -> one lane per
+    // channel; a fair number -> two lanes; too few -> cut L into chunks: the
+    // three-launch variant as above, else look-back chunks with one lane per
+    // channel when they stay long (>= 256 steps) and the widest split otherwise
+    // (>= 128 steps).
     // the warp-specialised variant needs 16-byte rows and 16-byte aligned
     // tensors (tiled tensor copies) and the driver's tensor-map encoder
     const size_t es = a.dtype == VMB_BF16 ? 2 : 4;
     const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    const bool tma_ok = np == 16 && (size_t)a.L * es % 16 == 0 && al16(a.u) && al16(a.delta) && al16(a.Bs) &&
+    const bool tma_ok = !a.no_tma && (size_t)a.L * es % 16 == 0 && al16(a.u) && al16(a.delta) && al16(a.Bs) &&
                         al16(a.Cs) && al16(a.y) && (a.gather_h == 0 || al16(a.u_t)) &&
                         tensor_map_encoder() != nullptr;
+    // the three-launch variant: a grid of 64-step, one-lane chunks fits in two
+    // waves (beyond that its aggregate traffic outweighs the other plans).  It
+    // then runs as two lanes per channel over 32-step chunks, which measured fastest
+    // with the launches chained (stage-1 maps at batch 1 to 3: 5 to 6% shorter
+    // steps than the 64-step chunks)
+    auto chunk_grid_fits = [&]() -> bool {
+        KernelInfo kc{};
+        long long rc = 0;
+        if (info(kChunkShape + 2, &kc, &rc) != VMB_OK) return false;
+        return a.B * a.K * (long long)((a.D + kc.DT - 1) / kc.DT) * ((a.L + kc.ts - 1) / kc.ts) <= 2 * rc;
+    };
     int shape = 0, n_chunks = 1, forced_chunks = 0, forced_shape = 0;
     KernelInfo ki{};
     long long res = 0;
     vmb_status st;
     if (!zoh && forced_plan(&forced_shape, &forced_chunks)) {
         shape = forced_shape % shape_count(np);
-        if (is_ws_shape(np, shape) && !tma_ok) shape = kPackedShape;
+        if (is_ws_shape(np, shape) && !tma_ok) shape = np == 16 ? kPackedShape : 0;
         if (small_lanes(np, shape) && small_scan_smem(small_lanes(np, shape), a.L, false) > kSmallMaxSmem) shape = 0;
         if (!small_lanes(np, shape) && (st = info(shape, &ki, &res)) != VMB_OK) return st;
         n_chunks = forced_chunks > 1 ? forced_chunks : 1;
@@ -2080,15 +1794,15 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         }
     } else if (const int G = np == 16 ? small_rule(a, a.gather_h > 0, tma_ok, sms) : 0) {
         shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
-    } else if (tma_ok && rows >= (a.L <= 1024 ? 64LL : 128LL) * sms) {
-        // a fair number of rows and tensors the tensor copies can read: the
-        // warp-specialised kernel, one pass over L (measured on GB300: fastest
-        // from the batch-32 56x56 map, under a third of a wave of its tiles, up;
-        // of shorter sequences from half of that, where the alternatives are one
-        // lane per state or no tensor copies: 14x14x768 at batch 4 22.8 us
-        // against 34.4, 10x10x768 at batch 8 18.5 against 25.4)
-        shape = kWsShape;
+    } else if (np == 16 && tma_ok && rows < 6LL * sms && chunk_grid_fits()) {
+        shape = kChunkShape + 1;
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+    } else if (tma_ok && rows >= 2LL * sms) {
+        const bool few = rows < 256LL * sms && (np < 16 || !small_map_one_lane(a.L));
+        shape = np == 16 && few ? kWsTwoShape : ws_shape(np);
+        if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+        if (few)
+            ws_estimate(np, a.B * a.K * (long long)((a.D + ki.DT - 1) / ki.DT), a.L, sms, ki.ts, &n_chunks);
     } else if (np == 16 && rows >= 256LL * sms && a.L >= 128) {
         // many rows: the packed streaming one-lane kernel, one pass over L (on
         // very short sequences its stage prologue does not pay off)
@@ -2113,29 +1827,13 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             KernelInfo km{};
             long long rm = 0;
             if ((st = info(r.mid, &km, &rm)) != VMB_OK) return st;
-            KernelInfo kc{}, k9{};
-            long long rc = 0, r9 = 0;
-            long long chunk_ctas = 0;
-            if (np == 16) {
-                // few rows: the three-launch chunked variant while a grid of
-                // 64-step, one-lane chunks would fit in two waves (beyond that
-                // its aggregate traffic outweighs the look-back's second pass).
-                // It then runs as two lanes per channel over 32-step chunks,
-                // which measured fastest on GB300 with the launches chained
-                // (stage-1 maps at batch 1 to 3: 5 to 6% shorter steps than
-                // the 64-step chunks)
-                if ((st = info(kChunkShape + 2, &kc, &rc)) != VMB_OK) return st;
-                if ((st = info(kChunkShape + 1, &k9, &r9)) != VMB_OK) return st;
-                chunk_ctas = a.B * a.K * (long long)((a.D + kc.DT - 1) / kc.DT) * ((a.L + kc.ts - 1) / kc.ts);
-            }
             if (rows * km.G * 2 >= rm * km.threads) {
                 shape = r.mid;
                 ki = km;
                 res = rm;
-            } else if (np == 16 && chunk_ctas <= 2 * rc) {
+            } else if (np == 16 && chunk_grid_fits()) {
                 shape = kChunkShape + 1;
-                ki = k9;
-                res = r9;
+                if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
             } else {
                 KernelInfo kn{};
                 long long rn = 0;
@@ -2167,7 +1865,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         n_chunks = 1;
     }
     if (is_chunk_shape(np, shape)) n_chunks = (a.L + ki.ts - 1) / ki.ts;  // chunks of exactly ts steps
-    if (is_stream_shape(np, shape) || is_packed_shape(np, shape) || is_ws_shape(np, shape))
+    if (is_stream_shape(np, shape) || is_packed_shape(np, shape) ||
+        (is_ws_shape(np, shape) && n_chunks < 3))
         n_chunks = 1;  // one pass over L
     if (n_chunks < 1) n_chunks = 1;
     ScanPlan p{};
@@ -2196,6 +1895,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
 int full_plan_small(const ScanPlan& plan) { return small_lanes(plan.np, plan.split); }
 
 bool full_plan_gathers(const ScanPlan& plan) { return is_ws_shape(plan.np, plan.split); }
+
+bool full_plan_lowrank(const ScanPlan& plan) { return plan.np == 16 && is_ws_shape(plan.np, plan.split); }
 
 // Raw Deltas of the low-rank form written out (for plans whose kernels read
 // materialised Deltas): out[b,k,d,l] = sum_r Wup[k,d,r] z[b,k,r,l], r in order
@@ -2233,17 +1934,18 @@ vmb_status launch_lowrank_expand(const float* z, const float* Wup, void* out, in
 }
 
 int full_plan_launches(const ScanPlan& plan) {
+    if (plan.n_chunks > 1 && is_ws_shape(plan.np, plan.split)) return 2;
     return (is_chunk_shape(plan.np, plan.split) && plan.n_chunks > 1) ? 3 : 1;
 }
 
 vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream) {
     const bool lowrank = a.R > 0;
-    if ((lowrank || a.gather_h > 0) && !is_ws_shape(plan.np, plan.split)) return VMB_ERR_UNSUPPORTED;
+    const bool ws_plan = is_ws_shape(plan.np, plan.split);
+    if ((lowrank && !full_plan_lowrank(plan)) || (a.gather_h > 0 && !ws_plan)) return VMB_ERR_UNSUPPORTED;
     if (lowrank && a.gather_h > 0) return VMB_ERR_UNSUPPORTED;
     if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream);
-    KernelInfo ki = lowrank ? ws_lowrank_info(a.dtype, a.R)
-                    : a.gather_h > 0 ? ws_gather_info(a.dtype)
-                                     : pick(a.dtype, plan.np, plan.split, (a.flags & VMB_FLAG_B_ZOH) != 0);
+    KernelInfo ki = ws_plan ? ws_info(a.dtype, plan.np, ws_variant(plan.np, plan.split), a.gather_h > 0, a.R)
+                            : pick(a.dtype, plan.np, plan.split, (a.flags & VMB_FLAG_B_ZOH) != 0);
     if (!ki.fn) return VMB_ERR_CUDA;
     const size_t es = a.dtype == VMB_BF16 ? 2 : 4;
     FullParams p{};
@@ -2267,8 +1969,6 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     p.vec = ((size_t)a.L * es % 16 == 0) && al16(a.u) && al16(a.delta) && al16(a.Bs) && al16(a.Cs) && al16(a.y);
     p.suppress = (a.flags & VMB_FLAG_TEST_SUPPRESS_PUBLISH) ? 1 : 0;
-    p.gather_h = a.gather_h;
-    if (a.gather_h > 0 && !ki.tma) return VMB_ERR_UNSUPPORTED;  // only the warp-specialised kernel gathers
     p.Wup = a.Wup;
     p.R = a.R;
     const WsLayout w = ws_layout(plan);
@@ -2299,26 +1999,42 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
         TensorMaps tm;
         const long long planes = (long long)a.B * a.K;
         const bool gather = a.gather_h > 0;
+        const int box_np = plan.np;
         // gathering: u and u2 are the map x and its transpose, [B][D][L] each
-        bool ok = gather ? encode_rows(&tm.u, a.u, a.dtype, a.L, a.D, a.B, ki.ts, ki.DT) &&
-                               encode_rows(&tm.u2, a.u_t, a.dtype, a.L, a.D, a.B, ki.ts, ki.DT)
-                         : encode_rows(&tm.u, a.u, a.dtype, a.L, a.D, planes, ki.ts, ki.DT);
+        bool ok = gather ? encode_rows(&tm.u, a.u, a.dtype, a.L, a.D, a.B, ki.ts, ki.DT, true) &&
+                               encode_rows(&tm.u2, a.u_t, a.dtype, a.L, a.D, a.B, ki.ts, ki.DT, true)
+                         : encode_rows(&tm.u, a.u, a.dtype, a.L, a.D, planes, ki.ts, ki.DT, true);
         if (!gather) tm.u2 = tm.u;
         // the delta box: DT rows of raw Deltas, or (low rank) the 16 rows of z, fp32
         ok = ok && (lowrank ? encode_rows(&tm.dl, a.delta, VMB_F32, a.L, a.R, planes, ki.ts, 16)
-                            : encode_rows(&tm.dl, a.delta, a.dtype, a.L, a.D, planes, ki.ts, ki.DT));
-        if (ok &&
-            encode_rows(&tm.B, a.Bs, a.dtype, a.L, a.N, planes, ki.ts, 16) &&
-            encode_rows(&tm.C, a.Cs, a.dtype, a.L, a.N, planes, ki.ts, 16)) {
+                            : encode_rows(&tm.dl, a.delta, a.dtype, a.L, a.D, planes, ki.ts, ki.DT, true));
+        if (ok && encode_rows(&tm.B, a.Bs, a.dtype, a.L, a.N, planes, ki.ts, box_np) &&
+            encode_rows(&tm.C, a.Cs, a.dtype, a.L, a.N, planes, ki.ts, box_np)) {
             void* targs[] = {&p, &tm};
+            const long long ctas = (long long)plan.n_seq * (plan.n_chunks > 1 ? plan.n_chunks - 1 : 1);
+            // launched early, behind a kernel that still holds shared memory, a CTA that
+            // fills its share of the SM waits for it or lands elsewhere (128 maps of
+            // 56x56x256 as the block: four slots 1966 us, five 2081)
+            p.nstg = plan.early ? kWsMinSlots : ws_slots(ki, ctas, device_sm_count());
+            ki.smem += (size_t)(p.nstg - kWsMinSlots) * ki.slot_bytes;
+            if (plan.n_chunks > 1) {
+                // chunk 0 and the aggregates of chunks 1 .. P - 1, then chunks 1 .. P
+                const unsigned grid_p = (unsigned)(plan.n_seq * (plan.n_chunks - 1));
+                for (p.phase = 1; p.phase <= 2; ++p.phase)
+                    if (launch_kernel(ki.fn, dim3(grid_p), dim3(ki.threads), ki.smem, targs, stream, plan.early) !=
+                        cudaSuccess)
+                        return VMB_ERR_CUDA;
+                return VMB_OK;
+            }
             return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, targs, stream, plan.early) ==
                            cudaSuccess
                        ? VMB_OK
                        : VMB_ERR_CUDA;
         }
         // the encoder refused the tensors: the packed streaming variant (same tiles, same
-        // results), which reads materialised sequences only
-        if (gather || lowrank) return VMB_ERR_UNSUPPORTED;
+        // results), which reads materialised sequences only (no fallback of the other variants)
+        if (gather || lowrank || plan.np != 16 || ws_variant(plan.np, plan.split) == kWsTwoLanes)
+            return VMB_ERR_UNSUPPORTED;
         ki = pick(a.dtype, plan.np, kPackedShape, false);
         if (!ki.fn) return VMB_ERR_CUDA;
     }

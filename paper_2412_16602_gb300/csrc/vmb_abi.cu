@@ -190,6 +190,14 @@ size_t plan_bytes(int path, const unsigned* flag_sets, int nsets, int B, int K, 
         ScanPlan plan{};
         if ((path == VMB_PATH_MEAN ? plan_mean(a, &plan) : plan_full(a, &plan)) != VMB_OK) return 0;
         if (plan.ws_bytes > need) need = plan.ws_bytes;
+        if (path == VMB_PATH_FULL && !(a.flags & VMB_FLAG_B_ZOH)) {
+            // the alignment of the call's tensors, which the query does not see,
+            // decides between two plans: cover both
+            a.no_tma = true;
+            if (plan_full(a, &plan) != VMB_OK) return 0;
+            a.no_tma = false;
+            if (plan.ws_bytes > need) need = plan.ws_bytes;
+        }
     }
     return need;
 }
@@ -390,7 +398,7 @@ vmb_status vmb_selective_scan_lowrank_fwd(const void* u, const float* z, const f
     s = plan_full(a, &plan);
     if (s != VMB_OK) return s;
     if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
-    if (full_plan_gathers(plan)) return launch_full(a, plan, stream);
+    if (full_plan_lowrank(plan)) return launch_full(a, plan, stream);
     // a plan whose kernel reads materialised raw Deltas: they are written into
     // y and the scan runs in place (each of its CTAs reads the steps of its own
     // rows before it writes them, and no other CTA touches them)

@@ -35,6 +35,7 @@ struct ScanArgs {
     float* saved = nullptr;  // mean path: the group means kept for the backward, [B*K][N + 1][L] fp32
     const float* Wup = nullptr;  // full path, low-rank Delta: delta is z [B*K][R][L] fp32 and
     int R = 0;                   // delta_raw = Wup z (Wup [K][D][R]); warp-specialised plans only
+    bool no_tma = false;         // full path, workspace query: plan as for tensors that tensor copies cannot read
 };
 
 // Execution plan of an L-chunked scan: how the (sequence, chunk) grid is cut
@@ -52,6 +53,17 @@ struct ScanPlan {
     size_t ws_bytes;      // total workspace bytes
     bool early = true;    // may be launched before the previous kernel of the stream completes
 };
+
+// One instance of the warp-specialised full scan (full_ws.cuh): fn is null when
+// it could not be set up.
+struct WsKernel {
+    const void* fn;
+    int per_slot, fixed;  // shared memory: bytes per ring slot, and once
+    int G, DT, threads, ts;
+};
+constexpr int kWsOneLane = 0, kWsTwoLanes = 1;  // variants of the 16-state kernel: lanes per channel
+WsKernel ws_kernel_f32(int np, int variant, bool gather, int R);
+WsKernel ws_kernel_bf16(int np, int variant, bool gather, int R);
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -156,9 +168,10 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan);
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan);
 vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
 int full_plan_launches(const ScanPlan& plan);  // kernels launch_full starts for this plan
-// Whether launch_full can read the plan's u gathered from the map (ScanArgs::gather_h)
-// or expand a low-rank Delta (ScanArgs::R): the warp-specialised plans.
+// Whether launch_full can read the plan's u gathered from the map (ScanArgs::gather_h):
+// the warp-specialised plans; or expand a low-rank Delta (ScanArgs::R): those of 16 states.
 bool full_plan_gathers(const ScanPlan& plan);
+bool full_plan_lowrank(const ScanPlan& plan);
 // out [B,K,D,L] (dtype) = Wup z, the raw Deltas of the low-rank form.
 vmb_status launch_lowrank_expand(const float* z, const float* Wup, void* out, int B, int K, int D, int R, int L,
                                  vmb_dtype dt, cudaStream_t stream);

@@ -1,0 +1,81 @@
+"""The forms of the warp-specialised full scan beyond one lane per channel and 16
+states: two lanes per channel (shape 23), L cut into chunks by two launches
+(chunks of shapes 19 and 23 and of fewer states), and 1 to 8 states (the last
+shape of their padded count), against the fp64 oracle, deterministic, and as the
+block from the map bit for bit against the three separate calls.  Sizes: ragged
+last stages and chunks, ragged channel tiles, padded states, bf16."""
+import pytest
+
+import oracle
+import workloads
+from tests.parity import check, to_device, to_numpy
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU, skipped by marker
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import paper_2412_16602_gb300 as vmb  # noqa: E402
+
+DEV = torch.device("cuda", 0)
+
+CASES = [
+    # (plan, B, D, N, H, W, dtype)
+    ("23", 1, 72, 16, 9, 12, "f32"),     # L = 108: a ragged last 16-step stage; a tile with one of four warps short
+    ("23", 2, 40, 13, 16, 24, "bf16"),
+    ("23", 1, 65, 16, 56, 56, "f32"),    # one channel in the second tile
+    ("23,3", 1, 72, 16, 20, 30, "f32"),  # L = 600: chunks of 208 steps, the last one ragged
+    ("23,7", 2, 40, 16, 16, 24, "bf16"),
+    ("23,25", 1, 33, 16, 40, 40, "f32"),  # 24 aggregates to fold
+    ("19,4", 1, 130, 16, 20, 30, "f32"),
+    ("1", 2, 72, 1, 9, 12, "f32"),
+    ("1", 1, 130, 2, 16, 24, "bf16"),
+    ("1", 1, 40, 3, 20, 30, "f32"),      # padded to 4 states
+    ("2", 2, 72, 5, 9, 12, "f32"),       # padded to 8 states
+    ("2", 1, 40, 8, 16, 24, "bf16"),
+    ("1,4", 1, 130, 1, 20, 30, "f32"),
+    ("2,5", 1, 40, 8, 20, 30, "f32"),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=["plan{}_B{}_D{}_N{}_{}x{}_{}".format(*c) for c in CASES])
+def test_warp_specialised_forms(case, force_plan):
+    plan, B, D, N, H, W, dt = case
+    force_plan.full(plan)
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=500 + D + N)
+    inp = workloads.make_inputs(wl, params="random")
+    g = to_device(inp, DEV)
+    args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+    xs = vmb.vmb_cross_scan(g["x"])
+    y = vmb.vmb_selective_scan_fwd(xs, *args, H, W)
+    y2 = vmb.vmb_selective_scan_fwd(xs, *args, H, W)
+    out, ym = vmb.vmb_ss2d_full_fwd(g["x"], *args)
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    _, y_ref, out_ref = oracle.ss2d_full(inp)
+    check(to_numpy(y), y_ref, dt, "full y")
+    check(to_numpy(out), out_ref, dt, "full out from the map")
+    assert torch.equal(y, y2), "deterministic"
+    assert torch.equal(ym, y) and torch.equal(out, vmb.vmb_cross_merge(y, H, W))
+
+
+@pytest.mark.parametrize("N", [16, 4])
+def test_workspace_of_the_query_serves_any_alignment(N):
+    """A workspace of exactly the queried size: aligned tensors take the chunked
+    warp-specialised plan, the same tensors one element into an allocation
+    another one with another workspace."""
+    B, D, H, W = 4, 64, 33, 32
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, seed=77)
+    inp = workloads.make_inputs(wl, params="random")
+    g = to_device(inp, DEV)
+    xs = vmb.vmb_cross_scan(g["x"])
+    _, y_ref, _ = oracle.ss2d_full(inp)
+    for shift in (0, 1):
+        buf = torch.empty(xs.numel() + shift, device=DEV)
+        u = buf[shift:].view(xs.shape)
+        u.copy_(xs)
+        ws = torch.zeros(vmb.vmb_scan_workspace_bytes(vmb.VMB_PATH_FULL, B, 4, D, N, H, W), dtype=torch.uint8,
+                         device=DEV)
+        y = vmb.vmb_selective_scan_fwd(u, g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W, workspace=ws)
+        assert vmb.vmb_read_status(ws) == vmb.VMB_OK
+        check(to_numpy(y), y_ref, "f32", f"full y, shifted by {shift}")
