@@ -71,22 +71,29 @@ struct MeanParams {
     float* incH;
 };
 
-template <typename T, int NP, int TC, bool ZOH, bool LR = false>
+// SPT steps per thread: 2 (see mean_scan_kernel) or 1.
+template <typename T, int NP, int TC, bool ZOH, bool LR = false, int SPT = 1>
 struct MLayout {
-    static constexpr int S = kThreads / TC;  // channel groups
+    static constexpr int NT = kThreads / SPT;  // threads per CTA
+    static constexpr int S = NT * SPT / TC;    // channel groups
+    // Two steps per thread: Abar and Bbar u replace the partial sums of the first
+    // two channel groups in place (rows padded by one), which leaves room for
+    // four CTAs per SM
+    static constexpr bool INPLACE = SPT == 2;
+    static constexpr int RT = TC + (INPLACE ? 1 : 0);  // row stride of the partial sums
     static constexpr int NMC = TC / kMC;
     // channels whose A / bias / Dskip (and, low rank, Wup rows) are staged at a time
-    static constexpr int CG = LR ? 128 : 256;
+    static constexpr int CG = LR || SPT == 2 ? 128 : 256;
     static constexpr int WR = 8;             // low rank: staged Wup row length (ranks up to 8, zero-padded)
     static constexpr int BCS = TC + 16 / (int)sizeof(T);  // raw B / C row stride (elements), rows 16-byte aligned
     // shared memory, byte offsets
     static constexpr size_t red = 0;                                            // f32 [S][NP][TC] partial sums of Abar
-    static constexpr size_t redb = red + (size_t)S * TC * NP * 4;               // f32 [S][NP][TC] of Bbar u (ZOH)
+    static constexpr size_t redb = red + (size_t)S * RT * NP * 4;               // f32 [S][NP][TC] of Bbar u (ZOH)
     static constexpr size_t redu = redb + (ZOH ? (size_t)S * TC * NP * 4 : 0);  // f32 [S][TC] sums of delta u
     static constexpr size_t reds = redu + (size_t)S * TC * 4;                   // f32 [S][TC] sums of Dskip u
     static constexpr size_t abar = reds + (size_t)S * TC * 4;                   // f32 [TC][NP]
-    static constexpr size_t bubar = abar + (size_t)TC * NP * 4;                 // f32 [TC][NP]
-    static constexpr size_t mc = bubar + (size_t)TC * NP * 4;                   // f32 [4][NMC][NP]
+    static constexpr size_t bubar = abar + (INPLACE ? 0 : (size_t)TC * NP * 4); // f32 [TC][NP]
+    static constexpr size_t mc = bubar + (INPLACE ? 0 : (size_t)TC * NP * 4);   // f32 [4][NMC][NP]
     static constexpr size_t ybar = a16(mc + (size_t)4 * NMC * NP * 4);          // f32 [TC], 16-byte aligned
     static constexpr size_t dsu = ybar + (size_t)TC * 4;                        // f32 [TC]
     static constexpr size_t hin = dsu + (size_t)TC * 4;                         // f32 [NP]
@@ -95,20 +102,19 @@ struct MLayout {
     // in place unless ZOH), delta bias [CG], Dskip [CG]
     static constexpr size_t tab0 = a16(bc + (size_t)2 * NP * BCS * sizeof(T));
     static constexpr size_t tab_bytes = (size_t)CG * NP * 4 + 2 * (size_t)CG * 4 + (LR ? (size_t)CG * WR * 4 : 0);
-    static constexpr size_t bytes1 = tab0 + tab_bytes;
-    static constexpr size_t bytes2 = bytes1;
-    static_assert(kThreads % TC == 0 && TC % 32 == 0, "a warp covers 32 consecutive steps");
-    static_assert(NP * NMC <= kThreads, "local scan mapping");
-    static_assert(bytes2 <= 110 * 1024, "mean-scan tile must leave room for two CTAs per SM");
+    static constexpr size_t bytes = tab0 + tab_bytes;
+    static_assert(NT * SPT % TC == 0 && TC % (32 * SPT) == 0, "a warp covers 32 SPT consecutive steps");
+    static_assert(!INPLACE || (S >= 2 && !ZOH), "Abar and Bbar u replace two groups' partial sums");
+    static_assert(bytes <= 110 * 1024, "mean-scan tile must leave room for two CTAs per SM");
 };
 
 // Stage group g0 of the channel tables (raw A rows, delta bias, Dskip) into
 // buffer `tb`: 16-byte async copies where rows are aligned, element loads
 // otherwise; channels past the group are zero.
-template <typename T, int NP, int TC, bool ZOH, bool LR = false>
+template <typename T, int NP, int TC, bool ZOH, bool LR = false, int SPT = 1>
 __device__ __forceinline__ void stage_tables(const MeanParams& p, unsigned char* tb, int k, int g0, int gn) {
-    using LY = MLayout<T, NP, TC, ZOH, LR>;
-    constexpr int CG = LY::CG;
+    using LY = MLayout<T, NP, TC, ZOH, LR, SPT>;
+    constexpr int CG = LY::CG, NT = LY::NT;
     float* ta = reinterpret_cast<float*>(tb);
     float* tbias = ta + CG * NP;
     float* tdsk = tbias + CG;
@@ -117,7 +123,7 @@ __device__ __forceinline__ void stage_tables(const MeanParams& p, unsigned char*
     bool rows_done = false;
     if constexpr (NP % 4 == 0) {
         if (p.N == NP && p.tabvec) {
-            for (int i = tid; i < CG * NP / 4; i += kThreads) {
+            for (int i = tid; i < CG * NP / 4; i += NT) {
                 const int r = i / (NP / 4);
                 const bool ok = r < gn;
                 cp_async16(ta + 4 * i, ok ? Ag + 4 * i : p.A, ok ? 16 : 0);
@@ -126,7 +132,7 @@ __device__ __forceinline__ void stage_tables(const MeanParams& p, unsigned char*
         }
     }
     if (!rows_done) {
-        for (int i = tid; i < CG * NP; i += kThreads) {
+        for (int i = tid; i < CG * NP; i += NT) {
             const int r = i / NP, n = i % NP;
             ta[i] = (r < gn && n < p.N) ? __ldg(Ag + (size_t)r * p.N + n) : 0.0f;
         }
@@ -134,13 +140,13 @@ __device__ __forceinline__ void stage_tables(const MeanParams& p, unsigned char*
     const float* bg = p.bias + (size_t)k * p.D + g0;
     const float* dg = p.Dskip + (size_t)k * p.D + g0;
     if (p.tabvec && (((size_t)k * p.D + g0) & 3) == 0) {
-        for (int i = tid; i < 2 * CG / 4; i += kThreads) {
+        for (int i = tid; i < 2 * CG / 4; i += NT) {
             const int which = i / (CG / 4), r = 4 * (i % (CG / 4));
             const int nb = max(0, min(4, gn - r)) * 4;
             cp_async16((which ? tdsk : tbias) + r, nb ? (which ? dg : bg) + r : p.bias, nb);
         }
     } else {
-        for (int i = tid; i < CG; i += kThreads) {
+        for (int i = tid; i < CG; i += NT) {
             tbias[i] = i < gn ? __ldg(bg + i) : 0.0f;
             tdsk[i] = i < gn ? __ldg(dg + i) : 0.0f;
         }
@@ -149,7 +155,7 @@ __device__ __forceinline__ void stage_tables(const MeanParams& p, unsigned char*
         // Wup rows of the group, [CG][WR] fp32, zero past R and past the group
         float* tw = reinterpret_cast<float*>(tb) + CG * NP + 2 * CG;
         const float* wg = p.Wup + ((size_t)k * p.D + g0) * p.R;
-        for (int i = tid; i < CG * LY::WR; i += kThreads) {
+        for (int i = tid; i < CG * LY::WR; i += NT) {
             const int r = i / LY::WR, q = i % LY::WR;
             tw[i] = (r < gn && q < p.R) ? __ldg(wg + (size_t)r * p.R + q) : 0.0f;
         }
@@ -190,10 +196,32 @@ __device__ __forceinline__ void st4_hint(__nv_bfloat16* q, const float (&v)[4], 
 // row read through L1 (every lane of a warp has the same channel).
 constexpr int kLRMax = 8;  // ranks the LR kernels hold in registers
 
-template <typename T, int NP, int TC, bool ZOH, bool LR = false>
-__global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const MeanParams p) {
-    using LY = MLayout<T, NP, TC, ZOH, LR>;
-    constexpr int S = LY::S, NMC = LY::NMC, CG = LY::CG, BCS = LY::BCS;
+// SPT = 2: a thread reduces two consecutive steps (8-byte loads of delta and u),
+// so a channel's A row, bias and loop are read and run once for 2 N terms instead
+// of N: the reduction is bound by instruction dispatch (per term one product, one
+// ex2 and one sum, 3.1 of 4 slots a clock, plus the softplus, the A row's loads
+// and the loop), and 128 threads with twice the registers keep as many
+// independent chains in flight as 256.  The sums and their order are those of SPT = 1
+// (bit-identical results).
+constexpr int mean_min_blocks(bool zoh, int spt) { return spt == 2 ? 4 : zoh ? 2 : 3; }
+
+// Two consecutive elements with an L2 eviction policy (8 bytes fp32, 4 bytes bf16).
+__device__ __forceinline__ float2 ld2_hint(const float* q, uint64_t pol) {
+    float2 v;
+    asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(q), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float2 ld2_hint(const __nv_bfloat16* q, uint64_t pol) {
+    unsigned a;
+    asm volatile("ld.global.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(a) : "l"(q), "l"(pol));
+    return make_float2(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u));
+}
+
+template <typename T, int NP, int TC, bool ZOH, bool LR = false, int SPT = 1>
+__global__ void __launch_bounds__(MLayout<T, NP, TC, ZOH, LR, SPT>::NT, mean_min_blocks(ZOH, SPT))
+    mean_scan_kernel(const MeanParams p) {
+    using LY = MLayout<T, NP, TC, ZOH, LR, SPT>;
+    constexpr int S = LY::S, NMC = LY::NMC, CG = LY::CG, BCS = LY::BCS, NT = LY::NT, RT = LY::RT;
     extern __shared__ __align__(16) unsigned char smb[];
     float* red = reinterpret_cast<float*>(smb + LY::red);
     float* redb = reinterpret_cast<float*>(smb + LY::redb);
@@ -211,7 +239,16 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     T* sB = reinterpret_cast<T*>(smb + LY::bc);
     T* sC = sB + NP * BCS;
     __shared__ unsigned s_misc[2];
-    __shared__ unsigned s_scr[2 * kThreads / 32 + 2];
+    __shared__ unsigned s_scr[2 * NT / 32 + 2];
+    // Abar and Bbar u of state n at step t of the chunk
+    auto ab = [&](int n, int t) -> float& {
+        if constexpr (LY::INPLACE) return red[n * RT + t];
+        else return abar[t * NP + n];
+    };
+    auto bu = [&](int n, int t) -> float& {
+        if constexpr (LY::INPLACE) return red[(NP + n) * RT + t];
+        else return bubar[t * NP + n];
+    };
 
     pdl_wait();
     pdl_launch_dependents();
@@ -258,14 +295,14 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
         const T* Cs = static_cast<const T*>(p.Cs);
         if (p.bcvec) {
             constexpr int VE = 16 / (int)sizeof(T), CPR = TC / VE;
-            for (int i = tid; i < 2 * NP * CPR; i += kThreads) {
+            for (int i = tid; i < 2 * NP * CPR; i += NT) {
                 const int which = i / (NP * CPR), r = (i / CPR) % NP, ch = i % CPR;
                 const bool ok = r < N && ch * VE < nvalid;
                 const T* src = (which ? Cs : Bs) + (bcrow0 + r) * (size_t)L + l0 + ch * VE;
                 cp_async16((which ? sC : sB) + r * BCS + ch * VE, ok ? src : Bs, ok ? 16 : 0);
             }
         } else {
-            for (int i = tid; i < 2 * NP * TC; i += kThreads) {
+            for (int i = tid; i < 2 * NP * TC; i += NT) {
                 const int which = i / (NP * TC), r = (i / TC) % NP, t = i % TC;
                 T v = T(0.0f);
                 if (r < N && t < nvalid) v = (which ? Cs : Bs)[(bcrow0 + r) * (size_t)L + l0 + t];
@@ -273,21 +310,24 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
             }
         }
     }
-    const int ngroups = (D + CG - 1) / CG;
-    stage_tables<T, NP, TC, ZOH, LR>(p, smb + LY::tab0, k, 0, min(CG, D));
+    stage_tables<T, NP, TC, ZOH, LR, SPT>(p, smb + LY::tab0, k, 0, min(CG, D));
     cp_async_commit();
 
     // ---------------------------------------------------------------- phase A
-    const int rt = tid % TC;  // step of this thread
-    const int sg = tid / TC;  // channel group of this thread
-    const bool tv = rt < nvalid;
-    float acc[NP], accb[NP];
+    const int rt = SPT * (tid % (TC / SPT));  // first step of this thread
+    const int sg = tid / (TC / SPT);          // channel group of this thread
+    const bool tv = rt < nvalid;              // (two steps: L is even, both or neither)
+    const int ngroups = (D + CG - 1) / CG;
+    float acc[SPT][NP], accb[ZOH ? NP : 1];
 #pragma unroll
     for (int n = 0; n < NP; ++n) {
-        acc[n] = 0.0f;
-        accb[n] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < SPT; ++e) acc[e][n] = 0.0f;
+        if constexpr (ZOH) accb[n] = 0.0f;
     }
-    float sdu = 0.0f, sdsu = 0.0f;
+    float sdu[SPT], sdsu[SPT];
+#pragma unroll
+    for (int e = 0; e < SPT; ++e) sdu[e] = sdsu[e] = 0.0f;
     // Channel groups of CG: the group's A, bias and Dskip are in shared memory
     // (async copies, the first group's issued with the prologue), A is scaled by
     // log2 e in place once it lands, then every thread reduces its channels of
@@ -296,7 +336,8 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     // at batch 128 and on the batch-32 stage-1 map: 4-5% faster than 4 or 8,
     // and fewer spills at 80 registers), eight otherwise (7% faster than six
     // with one state).
-    constexpr int kPF = (NP >= 16 && TC >= 128) ? 6 : 8;
+    // Two steps per thread: eight, each replaced as it is used.
+    constexpr int kPF = SPT == 2 ? 8 : (NP >= 16 && TC >= 128) ? 6 : 8;
     const size_t col = (size_t)l0 + (tv ? rt : 0);
     const T* dcol = dlr + urow0 * (size_t)L + col;
     const T* ucol = u + urow0 * (size_t)L + col;
@@ -305,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
         // the (b, d) plane of x row by row, 1 column by column (the rows of its
         // transpose u_t), 2 and 3 the same in reverse; the planes have the same
         // channel stride L as the rows of u
-        const int lr = (k >= 2) ? L - 1 - (int)col : (int)col;
+        const int lr = (k >= 2) ? L - SPT - (int)col : (int)col;  // (two steps: loaded as a pair and swapped)
         ucol = ((k & 1) ? static_cast<const T*>(p.u_t) : u) + (size_t)(seq / p.K) * D * (size_t)L + lr;
     }
     // u is read again by the broadcast pass: keep it in L2; delta streams through
@@ -317,12 +358,42 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     // Offsets within the (b, k) slab are 32-bit (D * L < 2^31, checked by the
     // planner); a thread's consecutive channels are SL elements apart.
     const int SL = S * L;
-    float vd[kPF], vu[kPF];
-    float zr[LR ? kLRMax : 1];  // LR: z of this thread's step
+    // the steps of one channel as loaded
+    struct Vals {
+        float v[SPT];
+    };
+    const bool swapped = SPT == 2 && p.gather_h > 0 && k >= 2;  // u pairs arrive in reverse
+    auto load_d = [&](int o) {
+        Vals r;
+        if constexpr (SPT == 2) {
+            const float2 q = ld2_hint(dcol + o, stream);
+            r.v[0] = q.x;
+            r.v[SPT - 1] = q.y;
+        } else {
+            r.v[0] = ld_hint(dcol + o, stream);
+        }
+        return r;
+    };
+    auto load_u = [&](int o) {
+        Vals r;
+        if constexpr (SPT == 2) {
+            const float2 q = ld2_hint(ucol + o, keep);
+            r.v[0] = swapped ? q.y : q.x;
+            r.v[SPT - 1] = swapped ? q.x : q.y;
+        } else {
+            r.v[0] = ld_hint(ucol + o, keep);
+        }
+        return r;
+    };
+    const Vals none{};
+    Vals vd[kPF], vu[kPF];
+    float zr[SPT][LR ? kLRMax : 1];  // LR: z of this thread's steps
     if constexpr (LR) {
 #pragma unroll
         for (int r = 0; r < kLRMax; ++r)
-            zr[r] = (tv && r < p.R) ? __ldg(p.z + ((size_t)seq * p.R + r) * L + col) : 0.0f;
+#pragma unroll
+            for (int e = 0; e < SPT; ++e)
+                zr[e][r] = (tv && r < p.R) ? __ldg(p.z + ((size_t)seq * p.R + r) * L + col + e) : 0.0f;
     }
     static_assert(!LR || kLRMax == 8, "the staged Wup rows hold 8 ranks");
     {
@@ -332,107 +403,159 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
 #pragma unroll
         for (int q = 0; q < kPF; ++q, o += SL) {
             const int d = sg + q * S;
-            vd[q] = (!LR && tv && d < gn) ? ld_hint(dcol + o, stream) : 0.0f;
-            vu[q] = (tv && d < gn) ? ld_hint(ucol + o, keep) : 0.0f;
+            vd[q] = (!LR && tv && d < gn) ? load_d(o) : none;
+            vu[q] = (tv && d < gn) ? load_u(o) : none;
         }
     }
     // one channel's contribution: softplus, the N exponentials of Abar, delta u
-    auto reduce_one = [&](float vdq, float vuq, int d) {
+    auto reduce_one = [&](Vals vdq, const Vals& vuq, int d) {
         if constexpr (LR) {
             // the row is zero past R, as is zr: the padded terms add exact zeros
             const float4* w4 = reinterpret_cast<const float4*>(s_wup + d * LY::WR);
             const float4 wa = w4[0], wb = w4[1];
-            float rs = 0.0f;
-            rs = fmaf(wa.x, zr[0], rs);
-            rs = fmaf(wa.y, zr[1], rs);
-            rs = fmaf(wa.z, zr[2], rs);
-            rs = fmaf(wa.w, zr[3], rs);
-            rs = fmaf(wb.x, zr[4], rs);
-            rs = fmaf(wb.y, zr[5], rs);
-            rs = fmaf(wb.z, zr[6], rs);
-            rs = fmaf(wb.w, zr[7], rs);
-            vdq = rs;
+#pragma unroll
+            for (int e = 0; e < SPT; ++e) {
+                float rs = 0.0f;
+                rs = fmaf(wa.x, zr[e][0], rs);
+                rs = fmaf(wa.y, zr[e][1], rs);
+                rs = fmaf(wa.z, zr[e][2], rs);
+                rs = fmaf(wa.w, zr[e][3], rs);
+                rs = fmaf(wb.x, zr[e][4], rs);
+                rs = fmaf(wb.y, zr[e][5], rs);
+                rs = fmaf(wb.z, zr[e][6], rs);
+                rs = fmaf(wb.w, zr[e][7], rs);
+                vdq.v[e] = rs;
+            }
         }
-        const float v = vdq + s_bias[d];
-        const float dv = p.softplus_on ? softplus(v) : v;
+        float dv[SPT];
+        const float bias = s_bias[d];
+        if constexpr (SPT == 2) {
+            float2 v = make_float2(vdq.v[0] + bias, vdq.v[SPT - 1] + bias);
+            if (p.softplus_on) v = softplus2(v);
+            dv[0] = v.x;
+            dv[SPT - 1] = v.y;
+        } else {
+            const float v = vdq.v[0] + bias;
+            dv[0] = p.softplus_on ? softplus(v) : v;
+        }
         const float* a2 = s_a2 + d * NP;  // broadcast reads: every lane has the same d
         if constexpr (ZOH) {
 #pragma unroll
             for (int n = 0; n < NP; ++n) {
                 const float an = a2[n];
-                const float em1 = expm1f(dv * an);
-                acc[n] += 1.0f + em1;
-                accb[n] = fmaf(an != 0.0f ? em1 / an : dv, vuq, accb[n]);
+                const float em1 = expm1f(dv[0] * an);
+                acc[0][n] += 1.0f + em1;
+                accb[n] = fmaf(an != 0.0f ? em1 / an : dv[0], vuq.v[0], accb[n]);
             }
         } else if constexpr (NP % 4 == 0) {
 #pragma unroll
             for (int n = 0; n < NP; n += 4) {
                 const float4 qa = *reinterpret_cast<const float4*>(a2 + n);
-                if constexpr (TC >= 64) {
-                    // packed f32x2 products and sums: half the issue slots (measured
-                    // 4-5% faster on the large maps that take these chunk lengths)
-                    const float2 dv2 = make_float2(dv, dv);
-                    const float2 t01 = __fmul2_rn(dv2, make_float2(qa.x, qa.y));
-                    const float2 t23 = __fmul2_rn(dv2, make_float2(qa.z, qa.w));
-                    const float2 a01 = __fadd2_rn(make_float2(acc[n], acc[n + 1]), make_float2(ex2(t01.x), ex2(t01.y)));
-                    const float2 a23 = __fadd2_rn(make_float2(acc[n + 2], acc[n + 3]), make_float2(ex2(t23.x), ex2(t23.y)));
-                    acc[n] = a01.x;
-                    acc[n + 1] = a01.y;
-                    acc[n + 2] = a23.x;
-                    acc[n + 3] = a23.y;
-                } else {
-                    acc[n] += ex2(dv * qa.x);
-                    acc[n + 1] += ex2(dv * qa.y);
-                    acc[n + 2] += ex2(dv * qa.z);
-                    acc[n + 3] += ex2(dv * qa.w);
+#pragma unroll
+                for (int e = 0; e < SPT; ++e) {
+                    float(&ac)[NP] = acc[e];
+                    if constexpr (TC >= 64) {
+                        // packed f32x2 products and sums: half the issue slots (measured
+                        // 4-5% faster on the large maps that take these chunk lengths)
+                        const float2 dv2 = make_float2(dv[e], dv[e]);
+                        const float2 t01 = __fmul2_rn(dv2, make_float2(qa.x, qa.y));
+                        const float2 t23 = __fmul2_rn(dv2, make_float2(qa.z, qa.w));
+                        const float2 a01 = __fadd2_rn(make_float2(ac[n], ac[n + 1]), make_float2(ex2(t01.x), ex2(t01.y)));
+                        const float2 a23 =
+                            __fadd2_rn(make_float2(ac[n + 2], ac[n + 3]), make_float2(ex2(t23.x), ex2(t23.y)));
+                        ac[n] = a01.x;
+                        ac[n + 1] = a01.y;
+                        ac[n + 2] = a23.x;
+                        ac[n + 3] = a23.y;
+                    } else {
+                        ac[n] += ex2(dv[e] * qa.x);
+                        ac[n + 1] += ex2(dv[e] * qa.y);
+                        ac[n + 2] += ex2(dv[e] * qa.z);
+                        ac[n + 3] += ex2(dv[e] * qa.w);
+                    }
                 }
             }
         } else {
 #pragma unroll
-            for (int n = 0; n < NP; ++n) acc[n] += ex2(dv * a2[n]);
+            for (int n = 0; n < NP; ++n) {
+                const float an = a2[n];
+#pragma unroll
+                for (int e = 0; e < SPT; ++e) acc[e][n] += ex2(dv[e] * an);
+            }
         }
-        sdu = fmaf(dv, vuq, sdu);
-        if (p.skip_mean) sdsu = fmaf(s_dsk[d], vuq, sdsu);
+#pragma unroll
+        for (int e = 0; e < SPT; ++e) {
+            sdu[e] = fmaf(dv[e], vuq.v[e], sdu[e]);
+            if (p.skip_mean) sdsu[e] = fmaf(s_dsk[d], vuq.v[e], sdsu[e]);
+        }
     };
     for (int gi = 0; gi < ngroups; ++gi) {
         const int g0 = gi * CG, gn = min(CG, D - g0);
         if (gi > 0) {
+            if constexpr (SPT == 1) {
+                // the group's first channels are requested before its tables are waited on
+                int o = (g0 + sg) * L;
+#pragma unroll
+                for (int q = 0; q < kPF; ++q, o += SL) {
+                    const int d = sg + q * S;
+                    vd[q] = (!LR && tv && d < gn) ? load_d(o) : none;
+                    vu[q] = (tv && d < gn) ? load_u(o) : none;
+                }
+            }
             __syncthreads();  // the previous group's tables are no longer read
-            stage_tables<T, NP, TC, ZOH, LR>(p, smb + LY::tab0, k, g0, gn);
+            stage_tables<T, NP, TC, ZOH, LR, SPT>(p, smb + LY::tab0, k, g0, gn);
             cp_async_commit();
         }
         cp_async_wait<0>();
         __syncthreads();  // this group's tables have landed
         if constexpr (!ZOH) {
-            for (int i = tid; i < CG * NP; i += kThreads) s_a2[i] *= kLog2e;
+            for (int i = tid; i < CG * NP; i += NT) s_a2[i] *= kLog2e;
             __syncthreads();
         }
         if (!tv) continue;
-        if (gi > 0) {
-            int o = (g0 + sg) * L;
+        if constexpr (SPT == 2) {
+            static_assert(CG % (kPF * S) == 0, "a group is whole batches: the requests run on into the next group");
+            for (int d0 = sg; d0 < gn; d0 += kPF * S) {
+                const int nx = g0 + d0 + kPF * S;  // the channel that takes the first slot next
+                int o = nx * L;
+                if (nx + (kPF - 1) * S < D && d0 + (kPF - 1) * S < gn) {
+                    // this batch and the next are entirely in range: no per-channel checks
 #pragma unroll
-            for (int q = 0; q < kPF; ++q, o += SL) {
-                const int d = sg + q * S;
-                vd[q] = (!LR && d < gn) ? ld_hint(dcol + o, stream) : 0.0f;
-                vu[q] = d < gn ? ld_hint(ucol + o, keep) : 0.0f;
+                    for (int q = 0; q < kPF; ++q, o += SL) {
+                        const Vals cd = vd[q], cu = vu[q];
+                        vd[q] = LR ? none : load_d(o);
+                        vu[q] = load_u(o);
+                        reduce_one(cd, cu, d0 + q * S);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < kPF; ++q, o += SL) {
+                        const Vals cd = vd[q], cu = vu[q];
+                        const bool in = nx + q * S < D;
+                        vd[q] = (!LR && in) ? load_d(o) : none;
+                        vu[q] = in ? load_u(o) : none;
+                        if (d0 + q * S < gn) reduce_one(cd, cu, d0 + q * S);
+                    }
+                }
             }
+            continue;
         }
         for (int d0 = sg; d0 < gn; d0 += kPF * S) {
-            float nd[kPF], nu[kPF];
+            Vals nd[kPF], nu[kPF];
             int o = (g0 + d0 + kPF * S) * L;  // the next batch's first channel
             if (d0 + (2 * kPF - 1) * S < gn) {
                 // the next batch is entirely in range: no per-channel checks
 #pragma unroll
                 for (int q = 0; q < kPF; ++q, o += SL) {
-                    nd[q] = LR ? 0.0f : ld_hint(dcol + o, stream);
-                    nu[q] = ld_hint(ucol + o, keep);
+                    nd[q] = LR ? none : load_d(o);
+                    nu[q] = load_u(o);
                 }
             } else {
 #pragma unroll
                 for (int q = 0; q < kPF; ++q, o += SL) {
                     const int d = d0 + (q + kPF) * S;
-                    nd[q] = (!LR && d < gn) ? ld_hint(dcol + o, stream) : 0.0f;
-                    nu[q] = d < gn ? ld_hint(ucol + o, keep) : 0.0f;
+                    nd[q] = (!LR && d < gn) ? load_d(o) : none;
+                    nu[q] = d < gn ? load_u(o) : none;
                 }
             }
             if (d0 + (kPF - 1) * S < gn) {
@@ -456,37 +579,44 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     if (!tv) {
         // steps past the end of the sequence: identity (Abar = 1, Bbar u = 0)
 #pragma unroll
-        for (int n = 0; n < NP; ++n) acc[n] = sg == 0 ? (float)D : 0.0f;
+        for (int n = 0; n < NP; ++n)
+#pragma unroll
+            for (int e = 0; e < SPT; ++e) acc[e][n] = sg == 0 ? (float)D : 0.0f;
     }
 
     // ---------------------------------------------------------------- phase B
 #pragma unroll
     for (int n = 0; n < NP; ++n) {  // [S][NP][TC]: lanes (consecutive t) hit consecutive banks
-        red[(sg * NP + n) * TC + rt] = acc[n];
+#pragma unroll
+        for (int e = 0; e < SPT; ++e) red[(sg * NP + n) * RT + rt + e] = acc[e][n];
         if constexpr (ZOH) redb[(sg * NP + n) * TC + rt] = accb[n];
     }
-    redu[sg * TC + rt] = sdu;
-    reds[sg * TC + rt] = sdsu;
+#pragma unroll
+    for (int e = 0; e < SPT; ++e) {
+        redu[sg * TC + rt + e] = sdu[e];
+        reds[sg * TC + rt + e] = sdsu[e];
+    }
     __syncthreads();
     const float invD = 1.0f / (float)D;
-    for (int i = tid; i < TC * NP; i += kThreads) {
+    for (int i = tid; i < TC * NP; i += NT) {
         const int n = i / TC, t = i % TC;
         float sa = 0.0f, sb = 0.0f, su = 0.0f;
 #pragma unroll
         for (int s2 = 0; s2 < S; ++s2) {
-            sa += red[(s2 * NP + n) * TC + t];
+            sa += red[(s2 * NP + n) * RT + t];
             if constexpr (ZOH) sb += redb[(s2 * NP + n) * TC + t];
             su += redu[s2 * TC + t];
         }
-        abar[t * NP + n] = sa * invD;
-        bubar[t * NP + n] = io<T>::cvt(sB[n * BCS + t]) * (ZOH ? sb : su) * invD;
+        // (in place: this thread alone reads and writes these words)
+        ab(n, t) = sa * invD;
+        bu(n, t) = io<T>::cvt(sB[n * BCS + t]) * (ZOH ? sb : su) * invD;
         if (p.save && t < nvalid) {
             float* sv = p.save + (size_t)seq * (N + 1) * L + l0 + t;
             if (n < N) sv[(size_t)n * L] = sa * invD;
             if (n == 0) sv[(size_t)N * L] = su * invD;
         }
     }
-    for (int t = tid; t < TC; t += kThreads) {
+    for (int t = tid; t < TC; t += NT) {
         float sd = 0.0f;
 #pragma unroll
         for (int s2 = 0; s2 < S; ++s2) sd += reds[s2 * TC + t];
@@ -494,14 +624,14 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     }
     __syncthreads();
     // local scan of each micro-chunk (from h = 0)
-    if (tid < NP * NMC) {
-        const int n = tid % NP, m = tid / NP;
+    for (int i = tid; i < NP * NMC; i += NT) {
+        const int n = i % NP, m = i / NP;
         float P = 1.0f, H = 0.0f;
 #pragma unroll
         for (int j = 0; j < kMC; ++j) {
             const int t = m * kMC + j;
-            const float a = abar[t * NP + n];
-            H = fmaf(a, H, bubar[t * NP + n]);
+            const float a = ab(n, t);
+            H = fmaf(a, H, bu(n, t));
             P *= a;
         }
         mcP[m * NP + n] = P;
@@ -542,19 +672,20 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
             // Decoupled look-back (the whole block polls 256 predecessors per round)
             // with a left fold after the inclusive state found: the carry is
             // bit-identical whichever predecessor the walk stops at.
-            const int found = lookback_find_block<kThreads>(p.flags + (size_t)seq * p.n_chunks, chunk, gen, p.hdr,
+            const int found = lookback_find_block<NT>(p.flags + (size_t)seq * p.n_chunks, chunk, gen, p.hdr,
                                                             (unsigned)seq, s_scr);
             if (found >= 0) {
                 // Fold the aggregates after the inclusive state left to right.  They are
                 // staged into shared memory (the partial-sum area, free by now) in
                 // batches with all loads in flight at once, then folded from there.
-                constexpr int kFB = (S * TC * NP) / (2 * NP);  // aggregates per batch
-                float* sP = red;
-                float* sH = red + kFB * NP;
+                // (two steps per thread: the A table's area)
+                constexpr int kFB = LY::INPLACE ? CG / 2 : (S * TC * NP) / (2 * NP);  // aggregates per batch
+                float* sP = LY::INPLACE ? s_a2 : red;
+                float* sH = sP + kFB * NP;
                 if (tid < NP) RH = ld_cg(&p.incH[((size_t)seq * p.n_chunks + found) * NP + tid]);
                 for (int m0 = found + 1; m0 < chunk; m0 += kFB) {
                     const int nb = min(kFB, chunk - m0);
-                    for (int i = tid; i < nb * NP; i += kThreads) {
+                    for (int i = tid; i < nb * NP; i += NT) {
                         const size_t smi = (size_t)seq * p.n_chunks + m0 + i / NP;
                         sP[i] = ld_cg(&p.aggP[smi * NP + i % NP]);
                         sH[i] = ld_cg(&p.aggH[smi * NP + i % NP]);
@@ -581,21 +712,21 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     }
     __syncthreads();
     // exact states of each micro-chunk and C . h  (written into abar as scratch)
-    if (tid < NP * NMC) {
-        const int n = tid % NP, m = tid / NP;
+    for (int i = tid; i < NP * NMC; i += NT) {
+        const int n = i % NP, m = i / NP;
         float h = fmaf(exP[m * NP + n], s_hin[n], exH[m * NP + n]);
 #pragma unroll
         for (int j = 0; j < kMC; ++j) {
             const int t = m * kMC + j;
-            h = fmaf(abar[t * NP + n], h, bubar[t * NP + n]);
-            abar[t * NP + n] = io<T>::cvt(sC[n * BCS + t]) * h;
+            h = fmaf(ab(n, t), h, bu(n, t));
+            ab(n, t) = io<T>::cvt(sC[n * BCS + t]) * h;
         }
     }
     __syncthreads();
-    for (int t = tid; t < TC; t += kThreads) {
+    for (int t = tid; t < TC; t += NT) {
         float s2 = 0.0f;
 #pragma unroll
-        for (int n = 0; n < NP; ++n) s2 += abar[t * NP + n];
+        for (int n = 0; n < NP; ++n) s2 += ab(n, t);
         s_ybar[t] = s2;
         // fused with the merge, ybar carries the broadcast skip term (the same
         // fp32 add the broadcast below would do)
@@ -607,7 +738,7 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
     if (!p.no_bcast && p.cvec) {
         // thread (quad, channel group): four consecutive steps of every DG-th
         // channel, 128-bit (bf16: 64-bit) loads and stores
-        constexpr int Q = TC / 4, DG = kThreads / Q;
+        constexpr int Q = TC / 4, DG = NT / Q;
         const int t4 = 4 * (tid % Q), dg = tid / Q;
         if (t4 < nvalid) {
             const bool qfull = t4 + 4 <= nvalid;
@@ -665,13 +796,15 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
             }
         }
     } else if (tv && !p.no_bcast) {
-        T* yc = static_cast<T*>(p.y) + urow0 * (size_t)L + l0 + rt;
-        const T* uc = u + urow0 * (size_t)L + l0 + rt;
-        const float yb = s_ybar[rt];
+#pragma unroll 1
+        for (int e = 0; e < SPT; ++e) {
+        T* yc = static_cast<T*>(p.y) + urow0 * (size_t)L + l0 + rt + e;
+        const T* uc = u + urow0 * (size_t)L + l0 + rt + e;
+        const float yb = s_ybar[rt + e];
         const uint64_t ev = l2_evict_first();
         if (p.skip_mean) {
             // y = ybar + the mean skip term: one value for every channel
-            const float yv = yb + s_dsu[rt];
+            const float yv = yb + s_dsu[rt + e];
             int o = sg * L;
             for (int d = sg; d < D; d += S, o += SL) st_hint(yc + o, yv, ev);
         } else {
@@ -698,6 +831,7 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
                 }
             }
         }
+        }
     }
 
     if (chunked) {
@@ -710,21 +844,20 @@ __global__ void __launch_bounds__(kThreads, ZOH ? 2 : 3) mean_scan_kernel(const 
 
 struct KInfo {
     const void* fn;
-    size_t smem;   // D <= 256: one buffer of channel tables
-    size_t smem2;  // D > 256: two
+    size_t smem;
+    int threads;
 };
 
-template <typename T, int NP, int TC, bool ZOH, bool LR>
+template <typename T, int NP, int TC, bool ZOH, bool LR, int SPT = 1>
 KInfo minfo() {
-    using LY = MLayout<T, NP, TC, ZOH, LR>;
-    const void* fn = reinterpret_cast<const void*>(&mean_scan_kernel<T, NP, TC, ZOH, LR>);
+    using LY = MLayout<T, NP, TC, ZOH, LR, SPT>;
+    const void* fn = reinterpret_cast<const void*>(&mean_scan_kernel<T, NP, TC, ZOH, LR, SPT>);
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     std::call_once(once, [&] {
-        err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes2);
+        err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
     });
-    if (err != cudaSuccess) return {nullptr, 0, 0};
-    return {fn, LY::bytes1, LY::bytes2};
+    return {err == cudaSuccess ? fn : nullptr, LY::bytes, LY::NT};
 }
 
 template <typename T, int NP, bool ZOH, bool LR>
@@ -755,6 +888,16 @@ KInfo mpick(vmb_dtype dt, int np, int tc, bool zoh, bool lr = false) {
     return zoh ? pick_np<float, true, false>(np, tc) : pick_np<float, false, false>(np, tc);
 }
 
+// Two steps per thread: 8 or more states, 128-step chunks, Euler Bbar.
+template <typename T, bool LR>
+KInfo pick_pair(int np) {
+    return np == 8 ? minfo<T, 8, 128, false, LR, 2>() : minfo<T, 16, 128, false, LR, 2>();
+}
+KInfo mpick_pair(vmb_dtype dt, int np, bool lr) {
+    if (dt == VMB_BF16) return lr ? pick_pair<__nv_bfloat16, true>(np) : pick_pair<__nv_bfloat16, false>(np);
+    return pick_pair<float, false>(np);
+}
+
 }  // namespace
 
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
@@ -776,7 +919,7 @@ vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
         if (forced && cand != forced) continue;
         KInfo ki = mpick(a.dtype, np, cand, zoh);
         if (!ki.fn) return VMB_ERR_CUDA;
-        const long long resident = resident_ctas(ki.fn, kThreads, a.D > 256 ? ki.smem2 : ki.smem);
+        const long long resident = resident_ctas(ki.fn, ki.threads, ki.smem);
         if (resident < 1) return VMB_ERR_CUDA;
         const long long ctas = seqs * ((a.L + cand - 1) / cand);
         const bool fills = a.D <= 256 ? 5 * ctas >= 4 * resident : ctas >= 2 * resident;
@@ -801,7 +944,18 @@ vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream) {
     const bool lr = a.R > 0;
     if (lr && ((a.flags & VMB_FLAG_B_ZOH) || a.R > kLRMax || a.bc_group != 1)) return VMB_ERR_UNSUPPORTED;
-    KInfo ki = mpick(a.dtype, plan.np, plan.chunk_len, (a.flags & VMB_FLAG_B_ZOH) != 0, lr);
+    const bool zoh = (a.flags & VMB_FLAG_B_ZOH) != 0;
+    // Two steps per thread where every pair of steps can be loaded as one and, in
+    // fp32, no y is written: four CTAs of 128 threads broadcast slower than three
+    // of 256 (GB300, 128 maps of 56x56x256 fp32: the block from the map 1531 us
+    // with one step, 1408 with two, with y written 1449 and 1516; 8 maps of
+    // 128x128x192 bf16: 427 and 368, with y 452 and 436).
+    const size_t pair = a.dtype == VMB_BF16 ? 4 : 8;
+    const auto al2 = [&](const void* q) { return reinterpret_cast<uintptr_t>(q) % pair == 0; };
+    const bool two = plan.np >= 8 && plan.chunk_len == 128 && !zoh && a.L % 2 == 0 &&
+                     (a.no_bcast || a.dtype == VMB_BF16) && al2(a.u) && (lr || al2(a.delta)) &&
+                     (a.gather_h == 0 || al2(a.u_t));
+    KInfo ki = two ? mpick_pair(a.dtype, plan.np, lr) : mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
     if (!ki.fn) return VMB_ERR_CUDA;
     MeanParams p{};
     p.u = a.u;
@@ -846,7 +1000,7 @@ vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     p.incH = reinterpret_cast<float*>(ws + w.incH_off);
     const unsigned grid = (unsigned)(plan.n_seq * plan.n_chunks);
     void* args[] = {&p};
-    cudaError_t e = launch_kernel(ki.fn, dim3(grid), dim3(kThreads), a.D > 256 ? ki.smem2 : ki.smem, args, stream);
+    cudaError_t e = launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream);
     return e == cudaSuccess ? VMB_OK : VMB_ERR_CUDA;
 }
 
