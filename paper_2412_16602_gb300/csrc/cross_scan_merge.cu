@@ -19,6 +19,9 @@
 // Index arithmetic uses division by invariant integers via multiply-high
 // (Granlund & Montgomery, "Division by invariant integers using
 // multiplication", PLDI 1994, round-up variant), valid for dividends < 2^31.
+#include <algorithm>
+#include <type_traits>
+
 #include "vmb_common.cuh"
 #include "vmb_internal.h"
 
@@ -630,12 +633,93 @@ vmb_status launch_mean_merge_t(const void* x, const float* ybar, const float* Ds
 // ------------------------------------------------------------ map transpose
 // xt[b, d, w, h] = x[b, d, h, w]: the column-major order of every (b, d) plane,
 // which the column-major directions of the cross-scan (1 and 3) read as
-// contiguous rows.  32 x 32 tiles through shared memory (one padded column so
-// the transposed reads hit distinct banks), coalesced on both sides.
+// contiguous rows.  The scan that follows reads xt in half of its CTAs only (see
+// pdl_wait in the gathering scans), so this kernel is built to run beside the
+// other half: one CTA per SM, which starts, and lets the scan be launched, at
+// once, and walks over the planes with the next item's loads in flight while the
+// current one is written.  Both sides are contiguous runs of whole planes.  VEC
+// (W and H multiples of a 16-byte vector): the pieces of a transposed row are
+// permuted by the column's vector index, so that the element stores of a
+// vector's columns and the vector reads of a row both spread over the banks.
+constexpr int kTrThreads = 512;
+constexpr int kTrVals = 4;    // vectors (VEC) or 4-element groups a thread holds
+constexpr size_t kTrSmem = kTransposeSmem - 1024;
+
+struct TransposeParams {
+    const void* x;
+    void* xt;
+    int H, W, HP;      // HP: row stride of the transposed tile (elements)
+    int ppi;           // planes per item
+    long long planes, items;
+    FastDiv fP, fA, fB;  // units per plane, per row of x, per row of xt
+};
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kTrThreads) map_transpose_kernel(const TransposeParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* sp = reinterpret_cast<T*>(smem_raw);  // [ppi][W][HP]
+    constexpr int VE = VEC ? 16 / (int)sizeof(T) : 1;  // elements per unit
+    constexpr int NV = VEC ? kTrVals : 4 * kTrVals;    // units per thread and item
+    using U = typename std::conditional<VEC, uint4, T>::type;
+    pdl_wait();
+    pdl_launch_dependents();
+    const unsigned per_plane = p.fP.d;  // units per plane
+    const U* x = static_cast<const U*>(p.x);
+    U* xt = static_cast<U*>(p.xt);
+    U v[NV];
+    auto load = [&](long long item) {
+        const long long p0 = item * p.ppi;
+        const unsigned n = (unsigned)min((long long)p.ppi, p.planes - p0) * per_plane;
+        const U* src = x + p0 * per_plane;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const unsigned i = threadIdx.x + q * kTrThreads;
+            if (i < n) v[q] = src[i];
+        }
+    };
+    long long item = blockIdx.x;
+    if (item < p.items) load(item);
+    for (; item < p.items; item += gridDim.x) {
+        const long long p0 = item * p.ppi;
+        const unsigned n = (unsigned)min((long long)p.ppi, p.planes - p0) * per_plane;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const unsigned i = threadIdx.x + q * kTrThreads;
+            if (i >= n) break;
+            const unsigned j = fdiv(i, p.fP), r = i - j * per_plane;
+            const unsigned h = fdiv(r, p.fA), c = r - h * p.fA.d;  // row, unit within it
+            if constexpr (VEC) {
+                Vec<T> w;
+                w.v = v[q];
+                T* dst = sp + (size_t)(j * p.W + c * VE) * p.HP + (h ^ ((c & 7) * VE));
+#pragma unroll
+                for (int e = 0; e < VE; ++e) dst[e * p.HP] = w.e[e];
+            } else {
+                sp[(size_t)(j * p.W + c) * p.HP + h] = v[q];
+            }
+        }
+        __syncthreads();
+        if (item + gridDim.x < p.items) load(item + gridDim.x);
+        U* dst = xt + p0 * per_plane;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const unsigned i = threadIdx.x + q * kTrThreads;
+            if (i >= n) break;
+            const unsigned j = fdiv(i, p.fP), r = i - j * per_plane;
+            const unsigned w = fdiv(r, p.fB), u = r - w * p.fB.d;  // column, unit within it
+            const T* src = sp + (size_t)(j * p.W + w) * p.HP + (VEC ? (u ^ ((w / VE) & 7)) * VE : u);
+            dst[i] = *reinterpret_cast<const U*>(src);
+        }
+        __syncthreads();  // the tile is rewritten by the next item
+    }
+}
+
+// Maps that do not fit an item: 32 x 32 tiles through shared memory (one padded
+// column so the transposed reads hit distinct banks), coalesced on both sides.
 constexpr int kTT = 32, kTR = 8;  // tile edge, rows per thread pass
 
 template <typename T>
-__global__ void __launch_bounds__(kTT * kTR) map_transpose_kernel(const T* x, T* xt, int H, int W, int tiles_w,
+__global__ void __launch_bounds__(kTT * kTR) tile_transpose_kernel(const T* x, T* xt, int H, int W, int tiles_w,
                                                                   int tiles_per_plane) {
     __shared__ T tile[kTT][kTT + 1];
     pdl_wait();
@@ -659,17 +743,55 @@ __global__ void __launch_bounds__(kTT * kTR) map_transpose_kernel(const T* x, T*
     }
 }
 
+
+template <typename T>
+vmb_status launch_plane_transpose(const void* x, void* xt, long long planes, int H, int W, cudaStream_t stream, bool* done) {
+    constexpr int VE = 16 / (int)sizeof(T);
+    const auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    const bool vec = W % VE == 0 && H % VE == 0 && a16(x) && a16(xt);
+    const int ve = vec ? VE : 1, nv = vec ? kTrVals : 4 * kTrVals;
+    TransposeParams p{};
+    p.x = x;
+    p.xt = xt;
+    p.H = H;
+    p.W = W;
+    p.HP = vec ? (H + 8 * VE - 1) / (8 * VE) * (8 * VE) : H | 1;
+    const long long L = (long long)H * W;
+    const size_t plane_bytes = (size_t)W * p.HP * sizeof(T);
+    *done = L <= (long long)nv * kTrThreads * ve && plane_bytes <= kTrSmem;
+    if (!*done) return VMB_OK;
+    const long long fit = std::min<long long>((long long)nv * kTrThreads * ve / L, (long long)(kTrSmem / plane_bytes));
+    const int sms = device_sm_count();
+    p.ppi = (int)std::max<long long>(1, std::min(fit, (planes + sms - 1) / sms));
+    p.planes = planes;
+    p.items = (planes + p.ppi - 1) / p.ppi;
+    p.fP = make_fastdiv((unsigned)(L / ve));
+    p.fA = make_fastdiv((unsigned)(W / ve));
+    p.fB = make_fastdiv((unsigned)(H / ve));
+    void* args[] = {&p};
+    const void* fn = vec ? reinterpret_cast<const void*>(&map_transpose_kernel<T, true>)
+                         : reinterpret_cast<const void*>(&map_transpose_kernel<T, false>);
+    return launch_kernel(fn, dim3((unsigned)std::min<long long>(p.items, sms)), dim3(kTrThreads), p.ppi * plane_bytes,
+                         args, stream) == cudaSuccess
+               ? VMB_OK
+               : VMB_ERR_CUDA;
+}
+
 }  // namespace
 
 vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, cudaStream_t stream) {
+    bool done = false;
+    const vmb_status st = dt == VMB_BF16 ? launch_plane_transpose<__nv_bfloat16>(x, xt, (long long)B * D, H, W, stream, &done)
+                                         : launch_plane_transpose<float>(x, xt, (long long)B * D, H, W, stream, &done);
+    if (done) return st;
     const int tiles_h = (H + kTT - 1) / kTT, tiles_w = (W + kTT - 1) / kTT;
     const long long grid = (long long)B * D * tiles_h * tiles_w;
     if (grid > INT32_MAX) return VMB_ERR_UNSUPPORTED;
     int tpp = tiles_h * tiles_w, tw = tiles_w;
     const void* xp = x;
     void* args[] = {&xp, &xt, &H, &W, &tw, &tpp};
-    const void* fn = dt == VMB_BF16 ? reinterpret_cast<const void*>(&map_transpose_kernel<__nv_bfloat16>)
-                                    : reinterpret_cast<const void*>(&map_transpose_kernel<float>);
+    const void* fn = dt == VMB_BF16 ? reinterpret_cast<const void*>(&tile_transpose_kernel<__nv_bfloat16>)
+                                    : reinterpret_cast<const void*>(&tile_transpose_kernel<float>);
     return launch_kernel(fn, dim3((unsigned)grid), dim3(kTT * kTR), 0, args, stream) == cudaSuccess ? VMB_OK
                                                                                                   : VMB_ERR_CUDA;
 }

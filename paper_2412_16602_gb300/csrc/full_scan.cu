@@ -1534,13 +1534,14 @@ KernelInfo ws_info(vmb_dtype dt, int np, int variant, bool gather = false, int R
 // for the CTAs it gets.  With one or two CTAs on an SM four slots leave too few
 // bytes in flight (GB300, 8 maps of 56x56x512 fp32, one CTA per SM: 332 us with
 // four slots, the copies' latency; see the rule in plan_full).
-int ws_slots(const KernelInfo& ki, long long grid, int sms) {
+// `other`: shared memory per SM of a kernel that runs beside it.
+int ws_slots(const KernelInfo& ki, long long grid, int sms, size_t other) {
     const long long resident = resident_ctas(ki.fn, ki.threads, ki.smem);
     long long per_sm = (grid + sms - 1) / sms;
     if (resident > 0 && per_sm * sms > resident) per_sm = resident / sms;
     if (per_sm < 1) per_sm = 1;
     const long long fixed = (long long)ki.smem - (long long)ki.slot_bytes * kWsMinSlots;
-    long long cap = (long long)kSmemPerSm / per_sm - 1024;
+    long long cap = (long long)(kSmemPerSm - other) / per_sm - 1024;
     if (cap > (long long)kSmallMaxSmem) cap = (long long)kSmallMaxSmem;
     const long long n = (cap - fixed) / ki.slot_bytes;
     return (int)(n < kWsMinSlots ? kWsMinSlots : n > kWsMaxSlots ? kWsMaxSlots : n);
@@ -2012,21 +2013,29 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
             encode_rows(&tm.C, a.Cs, a.dtype, a.L, a.N, planes, ki.ts, box_np)) {
             void* targs[] = {&p, &tm};
             const long long ctas = (long long)plan.n_seq * (plan.n_chunks > 1 ? plan.n_chunks - 1 : 1);
+            const bool sub_wave = ctas <= resident_ctas(ki.fn, ki.threads, ki.smem);
             // launched early, behind a kernel that still holds shared memory, a CTA that
             // fills its share of the SM waits for it or lands elsewhere (128 maps of
             // 56x56x256 as the block: four slots 1966 us, five 2081)
-            p.nstg = plan.early ? kWsMinSlots : ws_slots(ki, ctas, device_sm_count());
+            // gathering, the kernel before is the one-CTA-per-SM transpose, beside which
+            // half of the grid runs: launched early at any size in one pass (24576 rows
+            // of 56x56: 436 us, 452 launched after it), but not chunked (6144 rows of
+            // 128x128 bf16: 747, 705)
+            const bool beside = gather && plan.n_chunks == 1;
+            p.nstg = plan.early && !sub_wave ? kWsMinSlots
+                                             : ws_slots(ki, ctas, device_sm_count(), beside ? kTransposeSmem : 0);
+            const bool early = plan.early || beside;
             ki.smem += (size_t)(p.nstg - kWsMinSlots) * ki.slot_bytes;
             if (plan.n_chunks > 1) {
                 // chunk 0 and the aggregates of chunks 1 .. P - 1, then chunks 1 .. P
                 const unsigned grid_p = (unsigned)(plan.n_seq * (plan.n_chunks - 1));
                 for (p.phase = 1; p.phase <= 2; ++p.phase)
-                    if (launch_kernel(ki.fn, dim3(grid_p), dim3(ki.threads), ki.smem, targs, stream, plan.early) !=
+                    if (launch_kernel(ki.fn, dim3(grid_p), dim3(ki.threads), ki.smem, targs, stream, early) !=
                         cudaSuccess)
                         return VMB_ERR_CUDA;
                 return VMB_OK;
             }
-            return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, targs, stream, plan.early) ==
+            return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, targs, stream, early) ==
                            cudaSuccess
                        ? VMB_OK
                        : VMB_ERR_CUDA;

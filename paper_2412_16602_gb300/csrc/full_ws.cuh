@@ -118,8 +118,22 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
     // inputs were complete before launch 1 passed its own wait.  Its consumers wait
     // for launch 1 before they read the carries or write.
     const bool late = p.phase == 2;
+    // Gathering, the kernel before this one writes xt, which only the column-major
+    // directions read: the CTAs of directions 0 and 2 (the first half of the grid)
+    // do not wait for it.  What they touch was complete before that kernel passed its
+    // own wait, and this grid's dependents are released by its waiting CTAs.
+    const int tiles = p.n_tiles;
+    int tile = blockIdx.x % tiles;
+    bool own = true;
+    if constexpr (WS::GATHER) {
+        // tiles of directions 0, 2 of every b, then of 1, 3
+        const int t2 = 2 * p.tiles_per_bk, half = tiles / 2, odd = tile >= half;
+        const int r = tile - odd * half, b = r / t2, w = r % t2;
+        tile = (b * 4 + 2 * (w / p.tiles_per_bk) + odd) * p.tiles_per_bk + w % p.tiles_per_bk;
+        own = odd;
+    }
     if (!late) {
-        pdl_wait();
+        if (own) pdl_wait();
         pdl_launch_dependents();
     }
     using LY = WsTileLayout<T, WS>;
@@ -136,8 +150,7 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
     auto ready = [&](int i) { return bar0 + 24u * i + 8u; };
     auto released = [&](int i) { return bar0 + 24u * i + 16u; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile = blockIdx.x % p.n_tiles;
-    const int chunk = (int)(blockIdx.x / p.n_tiles) + (p.phase == 2 ? 1 : 0);
+    const int chunk = (int)(blockIdx.x / tiles) + (p.phase == 2 ? 1 : 0);
     const bool agg = p.phase == 1 && chunk > 0;  // aggregate only: no y
     const int bk = tile / p.tiles_per_bk;
     const int d0 = (tile % p.tiles_per_bk) * DT;

@@ -250,8 +250,12 @@ __global__ void __launch_bounds__(MLayout<T, NP, TC, ZOH, LR, SPT>::NT, mean_min
         else return bubar[t * NP + n];
     };
 
-    pdl_wait();
-    pdl_launch_dependents();
+    // Gathering from the map, the kernel before this one writes u_t, which only the
+    // column-major directions read: the CTAs of directions 0 and 2 (the first half
+    // of the tickets) do not wait for it.  What else this kernel reads or writes,
+    // the workspace included, was last touched before that kernel passed its own wait.
+    const bool gather = p.gather_h > 0;
+    if (!gather) pdl_wait();
     const int tid = threadIdx.x;
     const bool chunked = p.n_chunks > 1;
     int seq, chunk;
@@ -265,19 +269,30 @@ __global__ void __launch_bounds__(MLayout<T, NP, TC, ZOH, LR, SPT>::NT, mean_min
         const unsigned t = s_misc[0];
         gen = s_misc[1];
         if (t >= (unsigned)(p.n_seq * p.n_chunks)) {  // workspace was not zero-filled
+            if (gather) pdl_wait();
             if (tid == 0) {
                 atomicOr(&p.hdr->err, kErrBounds);
                 finish_launch(p.hdr, (unsigned)(p.n_seq * p.n_chunks));
             }
             return;
         }
-        chunk = (int)(t / (unsigned)p.n_seq);
-        seq = (int)(t % (unsigned)p.n_seq);
+        const unsigned half = gather ? (unsigned)p.n_seq / 2 : (unsigned)p.n_seq;
+        const unsigned odd = t >= half * p.n_chunks;  // gathering: every chunk of directions 0, 2, then of 1, 3
+        const unsigned r = t - odd * half * p.n_chunks;
+        chunk = (int)(r / half);
+        seq = (int)(r % half);
+        if (gather) seq = 2 * seq + (int)odd;
     } else {
         seq = blockIdx.x;
         chunk = 0;
+        if (gather) {
+            const int half = p.n_seq / 2, odd = seq >= half;
+            seq = 2 * (seq - odd * half) + odd;
+        }
     }
     const int k = seq % p.K;
+    if (gather && (k & 1)) pdl_wait();
+    pdl_launch_dependents();
     const int D = p.D, L = p.L, N = p.N;
     const int l0 = chunk * p.chunk_len;
     const int nvalid = min(TC, L - l0);

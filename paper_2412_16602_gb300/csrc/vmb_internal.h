@@ -187,6 +187,8 @@ vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W
                              cudaStream_t stream);
 vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, int W, vmb_dtype dt,
                               cudaStream_t stream);
+// The transpose runs as one CTA per SM of at most this shared memory (1 KB of the CTA's own included).
+constexpr size_t kTransposeSmem = 33 * 1024;
 vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt,
                                 cudaStream_t stream);
 vmb_status launch_discretise(const DiscArgs& a, bool mean, cudaStream_t stream);
