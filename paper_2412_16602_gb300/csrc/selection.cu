@@ -107,13 +107,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase) {
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelParams p) {
+// NBUF operand buffers: with two, the tensor cores work on a chunk while the next
+// one is converted and stored, which takes the products' latency off the chain of
+// a CTA, and the next two chunks' loads are in flight, at twice the shared memory
+// and registers (two CTAs per SM instead of five): for grids
+// that leave SMs with one or two CTAs (see launch_selection).
+template <typename T, int NBUF>
+__global__ void __launch_bounds__(kSelThreads, NBUF == 1 ? 5 : 2) selection_kernel(const SelParams p) {
     using LY = SelLayout;
     constexpr bool F32 = sizeof(T) == 4;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar;
+    __shared__ __align__(8) uint64_t s_mbar[NBUF];
     pdl_wait();
     pdl_launch_dependents();
     const int tid = threadIdx.x, warp = tid / 32;
@@ -129,9 +134,10 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
                      "n"(kSelTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    const uint32_t mbar = smem_addr(&s_mbar);
+    const uint32_t mbar0 = smem_addr(s_mbar);  // MMA completion of each buffer's chunk
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar));
+#pragma unroll
+        for (int b = 0; b < NBUF; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar0 + 8u * b));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -139,17 +145,11 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
 
-    const uint32_t sbase = smem_addr(smem);
-    float* sAhi = reinterpret_cast<float*>(smem + LY::a_hi);
-    float* sAlo = reinterpret_cast<float*>(smem + LY::a_lo);
-    float* sBhi = reinterpret_cast<float*>(smem + LY::b_hi);
-    float* sBlo = reinterpret_cast<float*>(smem + LY::b_lo);
     const T* ucol = static_cast<const T*>(p.u) + (size_t)bk * D * L + (lv ? l : 0);
     // this thread's row of A (its step): row group tid / 8, row tid % 8
     const int arow = (tid / 8) * 128 + (tid % 8) * 16;  // bytes within a channel quad's block
     constexpr int AG = kSelThreads / 8, BG = kSelCols / 8;
     bool ok = true;
-    uint32_t phase = 0;
     // The tensor cores accumulate a run of kSelDrain chunks in TMEM; each run's
     // sums are then added to fp32 registers, which keeps the accumulation chain
     // inside the tensor cores short for wide maps (D up to 1536).
@@ -183,11 +183,14 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
     // together; the next chunk's loads are issued while the tensor cores work
     // on the current one
     constexpr int kWPT = kSelCols * kSelKC / kSelThreads;  // weights per thread and chunk
-    float v[kSelKC], wv[kWPT];
-    auto load_chunk = [&](int c0) {
+    // (u as stored: converted only when staged, so that no request is waited for
+    // where it is issued)
+    T v[NBUF][kSelKC];
+    float wv[NBUF][kWPT];
+    auto load_chunk = [&](int c0, T (&v)[kSelKC], float (&wv)[kWPT]) {
         const int cn = min(kSelKC, D - c0);
 #pragma unroll
-        for (int j = 0; j < kSelKC; ++j) v[j] = (lv && j < cn) ? io<T>::ld(ucol + (size_t)(c0 + j) * L) : 0.0f;
+        for (int j = 0; j < kSelKC; ++j) v[j] = (lv && j < cn) ? ucol[(size_t)(c0 + j) * L] : T(0.0f);
 #pragma unroll
         for (int q = 0; q < kWPT; ++q) {
             const int i = tid + q * kSelThreads, m = i / kSelKC, j = i % kSelKC;
@@ -198,17 +201,27 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
             wv[q] = in ? __ldg(src + c0 + j) : 0.0f;
         }
     };
-    load_chunk(0);
-    for (int chunk = 0; chunk < nchunks; ++chunk) {
+    auto run_chunk = [&](int chunk, T (&v)[kSelKC], float (&wv)[kWPT]) {
         const int d0 = chunk * kSelKC;
         const int dn = min(kSelKC, D - d0);
+        const int buf = chunk % NBUF;
+        const uint32_t mbar = mbar0 + 8u * buf;
+        const uint32_t sbase = smem_addr(smem) + (uint32_t)(buf * LY::bytes);
+        float* sAhi = reinterpret_cast<float*>(smem + buf * LY::bytes + LY::a_hi);
+        float* sAlo = reinterpret_cast<float*>(smem + buf * LY::bytes + LY::a_lo);
+        float* sBhi = reinterpret_cast<float*>(smem + buf * LY::bytes + LY::b_hi);
+        float* sBlo = reinterpret_cast<float*>(smem + buf * LY::bytes + LY::b_lo);
+        // the MMAs of the buffer's last chunk have read the operands before they are
+        // overwritten (after a wait that gave up, the rest of the tile is not waited for)
+        if (chunk >= NBUF && ok) ok = mbar_wait(mbar, (uint32_t)(chunk / NBUF - 1) & 1u);
 #pragma unroll
         for (int c = 0; c < kSelKC / 4; ++c) {
             float hi[4], lo[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                hi[e] = F32 ? to_tf32(v[4 * c + e]) : v[4 * c + e];  // bf16 values are exact in tf32
-                lo[e] = to_tf32(v[4 * c + e] - hi[e]);
+                const float x = io<T>::cvt(v[4 * c + e]);
+                hi[e] = F32 ? to_tf32(x) : x;  // bf16 values are exact in tf32
+                lo[e] = to_tf32(x - hi[e]);
             }
             const int off = (c * AG * 128 + arow) / 4;
             *reinterpret_cast<float4*>(sAhi + off) = make_float4(hi[0], hi[1], hi[2], hi[3]);
@@ -223,6 +236,8 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
             sBhi[off] = hi;
             sBlo[off] = to_tf32(wv[q] - hi);
         }
+        // the registers are free again: request the chunk that uses them next
+        if (chunk + NBUF < nchunks) load_chunk(d0 + NBUF * kSelKC, v, wv);
         // the generic-proxy stores become visible to the tensor cores' async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
@@ -245,13 +260,21 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                          : "memory");
         }
-        if (chunk + 1 < nchunks) load_chunk(d0 + kSelKC);
-        // the chunk's MMAs have read the operands before they are overwritten
-        // (after a wait that gave up, the rest of the tile is not waited for)
-        if (ok) ok = mbar_wait(mbar, phase);
-        phase ^= 1u;
-        // this step's sums of the run: warp w reads TMEM lanes 32 w .. 32 w + 31
-        if (chunk % kSelDrain == kSelDrain - 1 || chunk == nchunks - 1) drain();
+        // this step's sums of the run, once its last MMAs are done: warp w reads TMEM
+        // lanes 32 w .. 32 w + 31
+        if (chunk % kSelDrain == kSelDrain - 1 || chunk == nchunks - 1) {
+            if (ok) ok = mbar_wait(mbar, (uint32_t)(chunk / NBUF) & 1u);
+            drain();
+        }
+    };
+#pragma unroll
+    for (int b = 0; b < NBUF; ++b)
+        if (b < nchunks) load_chunk(b * kSelKC, v[b], wv[b]);
+#pragma unroll 1
+    for (int chunk = 0; chunk < nchunks; chunk += NBUF) {
+#pragma unroll
+        for (int b = 0; b < NBUF; ++b)
+            if (chunk + b < nchunks) run_chunk(chunk + b, v[b], wv[b]);
     }
     if (!ok) {
 #pragma unroll
@@ -314,13 +337,13 @@ __global__ void __launch_bounds__(kSelThreads, 5) selection_kernel(const SelPara
     }
 }
 
-template <typename T>
+template <typename T, int NBUF>
 const void* sel_fn() {
-    const void* fn = reinterpret_cast<const void*>(&selection_kernel<T>);
+    const void* fn = reinterpret_cast<const void*>(&selection_kernel<T, NBUF>);
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     std::call_once(once, [&] {
-        err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SelLayout::bytes);
+        err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(NBUF * SelLayout::bytes));
     });
     return err == cudaSuccess ? fn : nullptr;
 }
@@ -346,10 +369,17 @@ vmb_status launch_selection(const SelArgs& a, cudaStream_t stream) {
     p.nlb = (a.L + kSelThreads - 1) / kSelThreads;
     const long long grid = (long long)a.B * a.K * p.nlb;
     if (grid > INT32_MAX) return VMB_ERR_UNSUPPORTED;
-    const void* fn = a.dtype == VMB_BF16 ? sel_fn<__nv_bfloat16>() : sel_fn<float>();
+    // Two buffers while the grid is at most two CTAs per SM (GB300, low-rank form,
+    // 32 maps of 14x14x768, 256 CTAs: 57.0 us with two buffers, 60.7 with one, 50.9
+    // with two chunks' loads in flight as well); more CTAs hide a chunk's latencies
+    // behind one another better than a second buffer does.
+    const bool two = grid <= 2LL * device_sm_count();
+    const void* fn = a.dtype == VMB_BF16 ? (two ? sel_fn<__nv_bfloat16, 2>() : sel_fn<__nv_bfloat16, 1>())
+                                         : (two ? sel_fn<float, 2>() : sel_fn<float, 1>());
     if (!fn) return VMB_ERR_CUDA;
     void* args[] = {&p};
-    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSelThreads), SelLayout::bytes, args, stream) == cudaSuccess
+    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSelThreads), (two ? 2 : 1) * SelLayout::bytes,
+                         args, stream) == cudaSuccess
                ? VMB_OK
                : VMB_ERR_CUDA;
 }
