@@ -903,14 +903,15 @@ KInfo mpick(vmb_dtype dt, int np, int tc, bool zoh, bool lr = false) {
     return zoh ? pick_np<float, true, false>(np, tc) : pick_np<float, false, false>(np, tc);
 }
 
-// Two steps per thread: 8 or more states, 128-step chunks, Euler Bbar.
+// Two steps per thread: 8 or more states, chunks of 64 or 128 steps, Euler Bbar.
 template <typename T, bool LR>
-KInfo pick_pair(int np) {
+KInfo pick_pair(int np, int tc) {
+    if (tc == 64) return np == 8 ? minfo<T, 8, 64, false, LR, 2>() : minfo<T, 16, 64, false, LR, 2>();
     return np == 8 ? minfo<T, 8, 128, false, LR, 2>() : minfo<T, 16, 128, false, LR, 2>();
 }
-KInfo mpick_pair(vmb_dtype dt, int np, bool lr) {
-    if (dt == VMB_BF16) return lr ? pick_pair<__nv_bfloat16, true>(np) : pick_pair<__nv_bfloat16, false>(np);
-    return pick_pair<float, false>(np);
+KInfo mpick_pair(vmb_dtype dt, int np, int tc, bool lr) {
+    if (dt == VMB_BF16) return lr ? pick_pair<__nv_bfloat16, true>(np, tc) : pick_pair<__nv_bfloat16, false>(np, tc);
+    return pick_pair<float, false>(np, tc);
 }
 
 }  // namespace
@@ -964,13 +965,14 @@ vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     // fp32, no y is written: four CTAs of 128 threads broadcast slower than three
     // of 256 (GB300, 128 maps of 56x56x256 fp32: the block from the map 1531 us
     // with one step, 1408 with two, with y written 1449 and 1516; 8 maps of
-    // 128x128x192 bf16: 427 and 368, with y 452 and 436).
+    // 128x128x192 bf16: 427 and 368, with y 452 and 436; 64-step chunks, 32 maps of
+    // 28x28x384: 182 and 161).
     const size_t pair = a.dtype == VMB_BF16 ? 4 : 8;
     const auto al2 = [&](const void* q) { return reinterpret_cast<uintptr_t>(q) % pair == 0; };
-    const bool two = plan.np >= 8 && plan.chunk_len == 128 && !zoh && a.L % 2 == 0 &&
+    const bool two = plan.np >= 8 && plan.chunk_len >= 64 && !zoh && a.L % 2 == 0 &&
                      (a.no_bcast || a.dtype == VMB_BF16) && al2(a.u) && (lr || al2(a.delta)) &&
                      (a.gather_h == 0 || al2(a.u_t));
-    KInfo ki = two ? mpick_pair(a.dtype, plan.np, lr) : mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
+    KInfo ki = two ? mpick_pair(a.dtype, plan.np, plan.chunk_len, lr) : mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
     if (!ki.fn) return VMB_ERR_CUDA;
     MeanParams p{};
     p.u = a.u;

@@ -1,5 +1,5 @@
-"""The channel-mean scan with two steps per thread (128-step chunks, 8 or 16 padded
-states, even L): ybar and the merged map bit for bit against the one-step kernel
+"""The channel-mean scan with two steps per thread (chunks of 64 or 128 steps, 8 or
+16 padded states, even L): ybar and the merged map bit for bit against the one-step kernel
 (which the same call runs on tensors one element into an allocation, where pairs
 of steps cannot be loaded as one), and against the fp64 oracle.  Sizes: a ragged
 last chunk of two steps, one chunk, channels around the 16-channel request
@@ -32,10 +32,11 @@ CASES = [
 ]
 
 
+@pytest.mark.parametrize("tc", [64, 128])
 @pytest.mark.parametrize("case", CASES, ids=["B{}_D{}_N{}_{}x{}_{}_f{}".format(*c) for c in CASES])
-def test_two_steps_per_thread(case, force_plan):
+def test_two_steps_per_thread(case, tc, force_plan):
     B, D, N, H, W, dt, extra = case
-    force_plan.mean(128)
+    force_plan.mean(tc)
     wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=900 + D + N)
     inp = workloads.make_inputs(wl, params="random")
     g = to_device(inp, DEV)
