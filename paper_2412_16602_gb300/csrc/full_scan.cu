@@ -93,8 +93,8 @@ __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t ro
     const T* Bs = static_cast<const T*>(p.Bs);
     const T* Cs = static_cast<const T*>(p.Cs);
     const int L = p.L;
-    T* dB = dst + 2 * DT * RS;
     if (p.vec) {
+        T* dB = dst + 2 * DT * RS;
         // thread i copies 16-byte column i % CPR of rows i / CPR + k * RPP
         constexpr int RPP = kThreads / CPR;  // rows covered per pass of the CTA
         static_assert(kThreads % CPR == 0, "tile loader mapping");
@@ -124,23 +124,51 @@ __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t ro
             }
         }
     } else {
+        // element by element: fp32 as 4-byte asynchronous copies, in flight like the
+        // 16-byte ones; bf16 (2-byte elements) through registers, a batch of
+        // independent loads at a time
         constexpr int nU = DT * kTS, nB = NP * kTS;
         constexpr int total = 2 * nU + (WITH_B ? (WITH_C ? 2 : 1) * nB : 0);
-        for (int i = threadIdx.x; i < total; i += kThreads) {
-            T v = T(0.0f);
+        auto locate = [&](int i, const T** src, int* at) -> bool {  // source, offset in dst; false: zero
             if (i < 2 * nU) {
                 const int j = i < nU ? i : i - nU;
                 const int r = j / kTS, t = j % kTS;
-                const T* base = i < nU ? u : dl;
-                if (r < nrows && l0 + t < L) v = base[(row0 + r) * (size_t)L + l0 + t];
-                dst[(i < nU ? 0 : DT * RS) + r * RS + t] = v;
-            } else {
-                const int i2 = i - 2 * nU;
-                const int j = i2 < nB ? i2 : i2 - nB;
-                const int r = j / kTS, t = j % kTS;
-                const T* base = i2 < nB ? Bs : Cs;
-                if (r < p.N && l0 + t < L) v = base[(bcrow0 + r) * (size_t)L + l0 + t];
-                dB[(i2 < nB ? 0 : NP * RS) + r * RS + t] = v;
+                *at = (i < nU ? 0 : DT * RS) + r * RS + t;
+                *src = (i < nU ? u : dl) + (row0 + r) * (size_t)L + l0 + t;
+                return r < nrows && l0 + t < L;
+            }
+            const int i2 = i - 2 * nU;
+            const int j = i2 < nB ? i2 : i2 - nB;
+            const int r = j / kTS, t = j % kTS;
+            *at = 2 * DT * RS + (i2 < nB ? 0 : NP * RS) + r * RS + t;
+            *src = (i2 < nB ? Bs : Cs) + (bcrow0 + r) * (size_t)L + l0 + t;
+            return r < p.N && l0 + t < L;
+        };
+        if constexpr (sizeof(T) == 4) {
+            for (int i = threadIdx.x; i < total; i += kThreads) {
+                const T* src;
+                int at;
+                const bool ok = locate(i, &src, &at);
+                cp_async4(dst + at, ok ? src : u, ok ? 4 : 0);
+            }
+        } else {
+            constexpr int kBatch = 8;
+            for (int i0 = threadIdx.x; i0 < total; i0 += kBatch * kThreads) {
+                T v[kBatch];
+                int at[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q) {
+                    const int i = i0 + q * kThreads;
+                    v[q] = T(0.0f);
+                    at[q] = -1;
+                    if (i < total) {
+                        const T* src;
+                        if (locate(i, &src, &at[q])) v[q] = *src;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (at[q] >= 0) dst[at[q]] = v[q];
             }
         }
     }
