@@ -1,20 +1,14 @@
 // cross_scan_merge.cu - SS2D cross-scan and cross-merge (App. A, "VMamba") for sm_103a.
 //
-// cross-scan: x[B,D,H,W] -> xs[B,4,D,L].  A CTA stages ppc whole maps (planes)
-// in shared memory with a padded row stride, then writes the four direction
-// rows of every plane: 0 row-major, 1 column-major, 2 and 3 the reverses of 0
-// and 1.  Global loads and stores are 16-byte vectors when rows are 16-byte
-// aligned; the padding keeps the column-major reads free of bank conflicts.
-//
-// Maps of 1024 pixels or more use band kernels instead: one CTA per band of
-// rows of one map (eight for the scan, up to 32 for the merge; see below),
-// which keeps batch-1 problems parallel.
-//
-// cross-merge: ys[B,4,D,L] -> out[B,D,H,W], out = (ys0[p0] + ys2[p2]) +
-// (ys1[p1] + ys3[p3]) in fp32 in that order.  Directions 0 and 2 are read
-// straight from global memory in output order (2 reversed); directions 1 and
-// 3 are staged in shared memory keyed by (w, h) so the transposed reads are
-// conflict-free.
+// cross-scan: x[B,D,H,W] -> xs[B,4,D,L], direction 0 row-major, 1 column-major,
+// 2 and 3 the reverses of 0 and 1.  cross-merge: ys[B,4,D,L] -> out[B,D,H,W],
+// out = (ys0[p0] + ys2[p2]) + (ys1[p1] + ys3[p3]) in fp32 in that order.
+// Maps below 1024 pixels: a CTA stages ppc whole maps (planes) in shared memory
+// with a padded row stride, which keeps the column-major accesses free of bank
+// conflicts; global loads and stores are 16-byte vectors when rows are 16-byte
+// aligned.  Larger maps use band kernels: one CTA per band of rows of one map
+// (eight for the scan, up to 32 for the merge; see below), which keeps batch-1
+// problems parallel.
 //
 // Index arithmetic uses division by invariant integers via multiply-high
 // (Granlund & Montgomery, "Division by invariant integers using
@@ -48,6 +42,7 @@ struct CsmParams {
     int D, H, W, L;
     long long planes;  // B * D
     int ppc;           // planes per CTA
+    int tabn;          // entries of one index table, padded (8-byte multiple)
     int vec;
     FastDiv fL, fW, fH, fD;
 };
@@ -58,158 +53,164 @@ union Vec {
     T e[16 / sizeof(T)];
 };
 
+// Tile indices of a plane's positions, computed once per CTA (the planes of a CTA
+// share them; a division per element and plane was half of these kernels'
+// instructions): row[r] of pixel r in row-major order, col[m] of the m-th pixel in
+// column-major order.
+__device__ __forceinline__ void plane_tables(unsigned short* row, unsigned short* col, const CsmParams& p, bool by_col) {
+    for (int i = threadIdx.x; i < p.L; i += kThreads) {
+        const int h = (int)fdiv((unsigned)i, p.fW), w = i - h * p.W;
+        row[i] = (unsigned short)(by_col ? w * (p.H + 1) + h : h * (p.W + 1) + w);
+        const int w1 = (int)fdiv((unsigned)i, p.fH), h1 = i - w1 * p.H;
+        col[i] = (unsigned short)(by_col ? w1 * (p.H + 1) + h1 : h1 * (p.W + 1) + w1);
+    }
+}
+
+// Directions 0 and 2 are written straight from the loaded values, 1 and 3 (the same
+// values in opposite orders) from the staged planes.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = p.L, PS = p.H * (p.W + 1);
+    unsigned short* row = reinterpret_cast<unsigned short*>(smem_raw);  // [L]
+    unsigned short* col = row + p.tabn;                                 // [L]
+    T* sp = reinterpret_cast<T*>(col + p.tabn);                         // [ppc][H][W+1]
+    constexpr int VE = 16 / sizeof(T);
+    plane_tables(row, col, p, false);
     pdl_wait();
     pdl_launch_dependents();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sp = reinterpret_cast<T*>(smem_raw);  // [ppc][H][W+1]
-    constexpr int VE = 16 / sizeof(T);
+    __syncthreads();
     const T* x = static_cast<const T*>(p.in);
     T* xs = static_cast<T*>(p.out);
-    const int L = p.L, W = p.W, H = p.H, WP = p.W + 1;
     const long long p0 = (long long)blockIdx.x * p.ppc;
     const int np = (int)min((long long)p.ppc, p.planes - p0);
     const unsigned n = (unsigned)(np * L);
     const T* src = x + p0 * L;
-    // stage the planes
+    const size_t DL = (size_t)p.D * L;
+    // direction 0's row of a plane; direction k's is k DL further
+    auto base = [&](unsigned j) {
+        const unsigned pi = (unsigned)(p0 + j), b = fdiv(pi, p.fD);
+        return xs + ((size_t)pi + (size_t)3 * p.D * b) * L;
+    };
     if (p.vec) {
+#pragma unroll 2
         for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
-            Vec<T> v;
+            Vec<T> v, r;
             v.v = *reinterpret_cast<const uint4*>(src + i);
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
 #pragma unroll
             for (int q = 0; q < VE; ++q) {
-                const unsigned e = i + q;
-                const unsigned j = fdiv(e, p.fL), r = e - j * L;
-                const unsigned h = fdiv(r, p.fW), w = r - h * W;
-                sp[(j * H + h) * WP + w] = v.e[q];
+                sp[j * PS + row[l + q]] = v.e[q];
+                r.e[q] = v.e[VE - 1 - q];
             }
+            T* o = base(j);
+            *reinterpret_cast<uint4*>(o + l) = v.v;
+            *reinterpret_cast<uint4*>(o + 2 * DL + (L - VE - l)) = r.v;
         }
     } else {
-        for (unsigned e = threadIdx.x; e < n; e += kThreads) {
-            const unsigned j = fdiv(e, p.fL), r = e - j * L;
-            const unsigned h = fdiv(r, p.fW), w = r - h * W;
-            sp[(j * H + h) * WP + w] = src[e];
+#pragma unroll 2
+        for (unsigned i = threadIdx.x; i < n; i += kThreads) {
+            const T v = src[i];
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            sp[j * PS + row[l]] = v;
+            T* o = base(j);
+            o[l] = v;
+            o[2 * DL + (L - 1 - l)] = v;
         }
     }
     __syncthreads();
-    // write the four direction rows of every staged plane
-#pragma unroll 1
-    for (int kd = 0; kd < 4; ++kd) {
-        const bool rev = kd >= 2, colmajor = kd & 1;
-        if (p.vec) {
-            for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
-                const unsigned j = fdiv(i, p.fL), l = i - j * L;
-                const long long pi = p0 + j;
-                const unsigned b = fdiv((unsigned)pi, p.fD), d = (unsigned)pi - b * p.D;
-                Vec<T> v;
+    if (p.vec) {
+#pragma unroll 2
+        for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            Vec<T> v, r;
 #pragma unroll
-                for (int q = 0; q < VE; ++q) {
-                    const unsigned m = rev ? L - 1 - (l + q) : l + q;
-                    unsigned h, w;
-                    if (colmajor) {
-                        w = fdiv(m, p.fH);
-                        h = m - w * H;
-                    } else {
-                        h = fdiv(m, p.fW);
-                        w = m - h * W;
-                    }
-                    v.e[q] = sp[(j * H + h) * WP + w];
-                }
-                *reinterpret_cast<uint4*>(xs + (((long long)b * 4 + kd) * p.D + d) * L + l) = v.v;
+            for (int q = 0; q < VE; ++q) {
+                v.e[q] = sp[j * PS + col[l + q]];
+                r.e[VE - 1 - q] = v.e[q];
             }
-        } else {
-            for (unsigned i = threadIdx.x; i < n; i += kThreads) {
-                const unsigned j = fdiv(i, p.fL), l = i - j * L;
-                const long long pi = p0 + j;
-                const unsigned b = fdiv((unsigned)pi, p.fD), d = (unsigned)pi - b * p.D;
-                const unsigned m = rev ? L - 1 - l : l;
-                unsigned h, w;
-                if (colmajor) {
-                    w = fdiv(m, p.fH);
-                    h = m - w * H;
-                } else {
-                    h = fdiv(m, p.fW);
-                    w = m - h * W;
-                }
-                xs[(((long long)b * 4 + kd) * p.D + d) * L + l] = sp[(j * H + h) * WP + w];
-            }
+            T* o = base(j);
+            *reinterpret_cast<uint4*>(o + DL + l) = v.v;
+            *reinterpret_cast<uint4*>(o + 3 * DL + (L - VE - l)) = r.v;
+        }
+    } else {
+#pragma unroll 2
+        for (unsigned i = threadIdx.x; i < n; i += kThreads) {
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            const T v = sp[j * PS + col[l]];
+            T* o = base(j);
+            o[DL + l] = v;
+            o[3 * DL + (L - 1 - l)] = v;
         }
     }
 }
 
+// ys1 + ys3 of every pixel is formed in column-major order and staged in fp32,
+// then added to ys0 + ys2 in row order (the sums and their order as stated above).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = p.L, PS = p.W * (p.H + 1);
+    unsigned short* row = reinterpret_cast<unsigned short*>(smem_raw);  // [L]
+    unsigned short* col = row + p.tabn;                                 // [L]
+    float* sp = reinterpret_cast<float*>(col + p.tabn);                 // [ppc][W][H+1]
+    constexpr int VE = 16 / sizeof(T);
+    plane_tables(row, col, p, true);
     pdl_wait();
     pdl_launch_dependents();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int L = p.L, W = p.W, H = p.H, HP = p.H + 1;
+    __syncthreads();
     const long long p0 = (long long)blockIdx.x * p.ppc;
     const int np = (int)min((long long)p.ppc, p.planes - p0);
-    T* s1 = reinterpret_cast<T*>(smem_raw);  // [ppc][W][H+1], keyed by (w, h)
-    T* s3 = s1 + (size_t)p.ppc * W * HP;
-    constexpr int VE = 16 / sizeof(T);
     const T* ys = static_cast<const T*>(p.in);
-    T* out = static_cast<T*>(p.out);
+    T* out = static_cast<T*>(p.out) + p0 * L;
     const unsigned n = (unsigned)(np * L);
-    auto row = [&](long long pi, int kd) {
-        const unsigned b = fdiv((unsigned)pi, p.fD), d = (unsigned)pi - b * p.D;
-        return ys + (((long long)b * 4 + kd) * p.D + d) * L;
+    const size_t DL = (size_t)p.D * L;
+    auto base = [&](unsigned j) {
+        const unsigned pi = (unsigned)(p0 + j), b = fdiv(pi, p.fD);
+        return ys + ((size_t)pi + (size_t)3 * p.D * b) * L;
     };
-    // stage directions 1 and 3
-    for (int kd = 1; kd <= 3; kd += 2) {
-        T* dst = kd == 1 ? s1 : s3;
-        const bool rev = kd == 3;
-        if (p.vec) {
-            for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
-                const unsigned j = fdiv(i, p.fL), l = i - j * L;
-                Vec<T> v;
-                v.v = *reinterpret_cast<const uint4*>(row(p0 + j, kd) + l);
+    if (p.vec) {
+#pragma unroll 2
+        for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            const T* o = base(j);
+            Vec<T> v1, v3;
+            v1.v = *reinterpret_cast<const uint4*>(o + DL + l);
+            v3.v = *reinterpret_cast<const uint4*>(o + 3 * DL + (L - VE - l));  // reversed block
 #pragma unroll
-                for (int q = 0; q < VE; ++q) {
-                    const unsigned m = rev ? L - 1 - (l + q) : l + q;  // column-major position
-                    const unsigned w = fdiv(m, p.fH), h = m - w * H;
-                    dst[(j * W + w) * HP + h] = v.e[q];
-                }
-            }
-        } else {
-            for (unsigned i = threadIdx.x; i < n; i += kThreads) {
-                const unsigned j = fdiv(i, p.fL), l = i - j * L;
-                const unsigned m = rev ? L - 1 - l : l;
-                const unsigned w = fdiv(m, p.fH), h = m - w * H;
-                dst[(j * W + w) * HP + h] = row(p0 + j, kd)[l];
-            }
+            for (int q = 0; q < VE; ++q) sp[j * PS + col[l + q]] = io<T>::cvt(v1.e[q]) + io<T>::cvt(v3.e[VE - 1 - q]);
+        }
+    } else {
+#pragma unroll 2
+        for (unsigned i = threadIdx.x; i < n; i += kThreads) {
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            const T* o = base(j);
+            sp[j * PS + col[l]] = io<T>::cvt(o[DL + l]) + io<T>::cvt(o[3 * DL + (L - 1 - l)]);
         }
     }
     __syncthreads();
-    // out[h, w] = (ys0[hW+w] + ys2[L-1-(hW+w)]) + (ys1[wH+h] + ys3[L-1-(wH+h)])
     if (p.vec) {
+#pragma unroll 2
         for (unsigned i = threadIdx.x * VE; i < n; i += kThreads * VE) {
-            const unsigned j = fdiv(i, p.fL), pos = i - j * L;
-            const long long pi = p0 + j;
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            const T* y = base(j);
             Vec<T> v0, v2, o;
-            v0.v = *reinterpret_cast<const uint4*>(row(pi, 0) + pos);
-            v2.v = *reinterpret_cast<const uint4*>(row(pi, 2) + (L - VE - pos));  // reversed block
+            v0.v = *reinterpret_cast<const uint4*>(y + l);
+            v2.v = *reinterpret_cast<const uint4*>(y + 2 * DL + (L - VE - l));  // reversed block
 #pragma unroll
             for (int q = 0; q < VE; ++q) {
-                const unsigned pq = pos + q;
-                const unsigned h = fdiv(pq, p.fW), w = pq - h * W;
-                const unsigned si = (j * W + w) * HP + h;
                 const float a = io<T>::cvt(v0.e[q]) + io<T>::cvt(v2.e[VE - 1 - q]);
-                const float c = io<T>::cvt(s1[si]) + io<T>::cvt(s3[si]);
-                o.e[q] = io<T>::to(a + c);
+                o.e[q] = io<T>::to(a + sp[j * PS + row[l + q]]);
             }
-            *reinterpret_cast<uint4*>(out + pi * L + pos) = o.v;
+            *reinterpret_cast<uint4*>(out + i) = o.v;
         }
     } else {
+#pragma unroll 2
         for (unsigned i = threadIdx.x; i < n; i += kThreads) {
-            const unsigned j = fdiv(i, p.fL), pos = i - j * L;
-            const long long pi = p0 + j;
-            const unsigned h = fdiv(pos, p.fW), w = pos - h * W;
-            const unsigned si = (j * W + w) * HP + h;
-            const float a = io<T>::cvt(row(pi, 0)[pos]) + io<T>::cvt(row(pi, 2)[L - 1 - pos]);
-            const float c = io<T>::cvt(s1[si]) + io<T>::cvt(s3[si]);
-            out[pi * L + pos] = io<T>::to(a + c);
+            const unsigned j = fdiv(i, p.fL), l = i - j * L;
+            const T* y = base(j);
+            const float a = io<T>::cvt(y[l]) + io<T>::cvt(y[2 * DL + (L - 1 - l)]);
+            out[i] = io<T>::to(a + sp[j * PS + row[l]]);
         }
     }
 }
@@ -377,7 +378,7 @@ __global__ void __launch_bounds__(kBandThreads) cross_merge_band_kernel(const Ba
     }
 }
 
-// Planes too large for shared memory: one thread per element, plain gathers.
+// Rows too long for a band in shared memory: one thread per element, plain gathers.
 template <typename T>
 __global__ void cross_scan_direct(const T* x, T* xs, int D, int H, int W, long long total) {
     pdl_wait();
@@ -414,10 +415,10 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
     const int L = H * W;
     const long long planes = (long long)B * D;
     const size_t es = sizeof(T);
-    const size_t per_plane = merge ? 2 * (size_t)W * (H + 1) * es : (size_t)H * (W + 1) * es;
-    const bool small_enough = per_plane <= kMaxSmem && planes < (1ll << 31) &&
-                              (long long)L * 4 < (1ll << 31);
-    if (!small_enough) {
+    const bool small_enough = planes < (1ll << 31) && (long long)L * 4 < (1ll << 31);
+    const bool band = small_enough && L >= kBandMinL && (size_t)2 * kRB * (W + 1) * es <= kMaxSmem &&
+                      planes * ((H + kRB - 1) / kRB) < (1ll << 31);
+    if (!small_enough || (L >= kBandMinL && !band)) {
         const long long total = merge ? planes * L : planes * 4 * L;
         const int grid = (int)std::min<long long>((total + kThreads - 1) / kThreads, 152ll * 32);
         const void* fn = merge ? reinterpret_cast<const void*>(&cross_merge_direct<T>)
@@ -427,7 +428,7 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
         void* args[] = {&src, &dst, &D, &H, &W, const_cast<long long*>(&total)};
         return launch_kernel(fn, dim3(grid), dim3(kThreads), 0, args, stream) == cudaSuccess ? VMB_OK : VMB_ERR_CUDA;
     }
-    if (L >= kBandMinL && (size_t)2 * kRB * (W + 1) * es <= kMaxSmem && planes * ((H + kRB - 1) / kRB) < (1ll << 31)) {
+    if (band) {
         BandParams bp{};
         bp.in = in;
         bp.out = outp;
@@ -455,10 +456,13 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
         return launch_kernel(fn, dim3(nblk), dim3(kBandThreads), smem, args, stream) == cudaSuccess ? VMB_OK
                                                                                                      : VMB_ERR_CUDA;
     }
-    // about 8K elements per CTA, bounded by shared memory
-    int ppc = (int)std::max<long long>(1, 8192 / L);
-    while (ppc > 1 && (size_t)ppc * per_plane > kMaxSmem) --ppc;
-    if (ppc > planes) ppc = (int)planes;
+    // about 8K elements per CTA, bounded by shared memory, fewer while the grid would
+    // leave SMs idle
+    const int tabn = (L + 7) / 8 * 8;
+    const size_t tables = (size_t)2 * tabn * 2, plane = merge ? (size_t)W * (H + 1) * 4 : (size_t)H * (W + 1) * es;
+    long long want = std::max<long long>(1, std::min<long long>(8192 / L, planes / (4LL * device_sm_count())));
+    while (want > 1 && tables + (size_t)want * plane > kMaxSmem) --want;
+    const int ppc = (int)want;
     CsmParams p{};
     p.in = in;
     p.out = outp;
@@ -468,13 +472,14 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
     p.L = L;
     p.planes = planes;
     p.ppc = ppc;
+    p.tabn = tabn;
     const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     p.vec = ((size_t)L * es % 16 == 0) && al16(in) && al16(outp);
     p.fL = make_fastdiv((unsigned)L);
     p.fW = make_fastdiv((unsigned)W);
     p.fH = make_fastdiv((unsigned)H);
     p.fD = make_fastdiv((unsigned)D);
-    const size_t smem = (size_t)ppc * per_plane;
+    const size_t smem = tables + (size_t)ppc * plane;
     const void* fn = merge ? reinterpret_cast<const void*>(&cross_merge_kernel<T>)
                            : reinterpret_cast<const void*>(&cross_scan_kernel<T>);
     if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
