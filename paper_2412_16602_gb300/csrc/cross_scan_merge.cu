@@ -510,11 +510,13 @@ vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, in
 // from x and the four ybar rows of (b, .) without y ever being written.  The
 // fp32 operations and their order are those of the broadcast and of the
 // cross-merge, so fp32 results are bit-identical to the unfused path; bf16
-// rounds once, at the end.  A thread owns kMP consecutive positions and keeps
-// their four ybar values in registers across the CTA's channels.
+// rounds once, at the end.  A thread owns MP consecutive positions and keeps
+// their four ybar values in registers across the CTA's channels; MP is the most that 16-byte
+// accesses and the row length allow (GB300, with four channels in flight, block from the map: 8 maps of
+// 128x128x192 bf16 349 us with two positions, 328 with eight; 32 maps of 28x28x384 fp32 161 and 148).
 namespace {
 constexpr int kMMThreads = 128;
-constexpr int kMP = 2;  // positions per thread
+constexpr int kMMAhead = 4;  // channels whose loads a thread has in flight
 constexpr int kMMMaxDC = 64;
 
 struct MeanMergeParams {
@@ -524,11 +526,50 @@ struct MeanMergeParams {
     const float* Dskip;  // [4 D]
     int B, D, H, W;
     int per_channel;  // 0: skip already in ybar
-    int vec;          // kMP positions of a row vector-accessible (aligned rows, L % kMP == 0)
+    int vec;          // MP positions of a row vector-accessible (aligned rows, L % MP == 0)
     int dc;           // channels per CTA
 };
 
-template <typename T>
+// MP consecutive elements as fp32, and back (MP sizeof(T) bytes at once).
+template <typename T, int MP>
+struct MmVec {
+    static constexpr int W = MP * (int)sizeof(T) / 4;  // 32-bit words
+    static __device__ __forceinline__ void load(const T* q, unsigned (&r)[W]) {
+        if constexpr (W == 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(q);
+            r[0] = v.x, r[1] = v.y, r[2] = v.z, r[3] = v.w;
+        } else if constexpr (W == 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(q);
+            r[0] = v.x, r[1] = v.y;
+        } else {
+            r[0] = *reinterpret_cast<const unsigned*>(q);
+        }
+    }
+    static __device__ __forceinline__ float get(const unsigned (&r)[W], int j) {
+        if constexpr (sizeof(T) == 4) return __uint_as_float(r[j]);
+        else return __uint_as_float((j & 1) ? (r[j / 2] & 0xffff0000u) : (r[j / 2] << 16));
+    }
+    static __device__ __forceinline__ void store(T* q, const float (&o)[MP], uint64_t pol) {
+        unsigned r[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            if constexpr (sizeof(T) == 4) r[i] = __float_as_uint(o[i]);
+            else r[i] = __bfloat16_as_ushort(io<T>::to(o[2 * i])) |
+                        ((unsigned)__bfloat16_as_ushort(io<T>::to(o[2 * i + 1])) << 16);
+        }
+        if constexpr (W == 4)
+            asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(q), "r"(r[0]), "r"(r[1]),
+                         "r"(r[2]), "r"(r[3]), "l"(pol)
+                         : "memory");
+        else if constexpr (W == 2)
+            asm volatile("st.global.L2::cache_hint.v2.b32 [%0], {%1, %2}, %3;" ::"l"(q), "r"(r[0]), "r"(r[1]), "l"(pol)
+                         : "memory");
+        else
+            asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(q), "r"(r[0]), "l"(pol) : "memory");
+    }
+};
+
+template <typename T, int MP>
 __global__ void __launch_bounds__(kMMThreads) mean_merge_kernel(const MeanMergeParams p) {
     pdl_wait();
     pdl_launch_dependents();
@@ -540,11 +581,11 @@ __global__ void __launch_bounds__(kMMThreads) mean_merge_kernel(const MeanMergeP
         const int kd = i / kMMMaxDC, j = i % kMMMaxDC;
         sd[kd][j] = (p.per_channel && j < dn) ? __ldg(p.Dskip + (size_t)kd * p.D + dbeg + j) : 0.0f;
     }
-    const int pos0 = (blockIdx.x * kMMThreads + threadIdx.x) * kMP;
+    const int pos0 = (blockIdx.x * kMMThreads + threadIdx.x) * MP;
     const float* yb = p.ybar + (size_t)b * 4 * L;
-    float y0[kMP], y1[kMP], y2[kMP], y3[kMP];
+    float y0[MP], y1[MP], y2[MP], y3[MP];
 #pragma unroll
-    for (int j = 0; j < kMP; ++j) {
+    for (int j = 0; j < MP; ++j) {
         const int pos = pos0 + j;
         if (pos < L) {
             const int h = pos / W, w = pos - h * W, p1 = w * H + h;
@@ -558,56 +599,44 @@ __global__ void __launch_bounds__(kMMThreads) mean_merge_kernel(const MeanMergeP
     }
     __syncthreads();
     if (pos0 >= L) return;
-    const bool full = p.vec && pos0 + kMP <= L;
     const T* x = static_cast<const T*>(p.x) + ((size_t)b * p.D + dbeg) * L + pos0;
     T* out = static_cast<T*>(p.out) + ((size_t)b * p.D + dbeg) * L + pos0;
     const uint64_t ev = l2_evict_first();
+    auto merged = [&](int dd, int j, float xv) {
+        const float a = fmaf(sd[0][dd], xv, y0[j]) + fmaf(sd[2][dd], xv, y2[j]);
+        const float c = fmaf(sd[1][dd], xv, y1[j]) + fmaf(sd[3][dd], xv, y3[j]);
+        return a + c;
+    };
+    if (p.vec) {  // L is a multiple of MP: all of a thread's positions are in range
+        using V = MmVec<T, MP>;
+        for (int d0 = 0; d0 < dn; d0 += kMMAhead) {
+            unsigned r[kMMAhead][V::W];
+#pragma unroll
+            for (int q = 0; q < kMMAhead; ++q)
+                if (d0 + q < dn) V::load(x + (size_t)(d0 + q) * L, r[q]);
+#pragma unroll
+            for (int q = 0; q < kMMAhead; ++q) {
+                if (d0 + q >= dn) break;
+                float o[MP];
+#pragma unroll
+                for (int j = 0; j < MP; ++j) o[j] = merged(d0 + q, j, V::get(r[q], j));
+                V::store(out + (size_t)(d0 + q) * L, o, ev);
+            }
+        }
+        return;
+    }
     for (int dd = 0; dd < dn; ++dd, x += L, out += L) {
-        float xv[kMP], o[kMP];
-        if (full) {
-            if constexpr (sizeof(T) == 4) {
-                const float2 q = *reinterpret_cast<const float2*>(x);
-                xv[0] = q.x;
-                xv[1] = q.y;
-            } else {
-                const unsigned q = *reinterpret_cast<const unsigned*>(x);
-                xv[0] = __uint_as_float(q << 16);
-                xv[1] = __uint_as_float(q & 0xffff0000u);
-            }
-        } else {
 #pragma unroll
-            for (int j = 0; j < kMP; ++j) xv[j] = pos0 + j < L ? io<T>::cvt(x[j]) : 0.0f;
-        }
-        const float s0 = sd[0][dd], s1 = sd[1][dd], s2 = sd[2][dd], s3 = sd[3][dd];
-#pragma unroll
-        for (int j = 0; j < kMP; ++j) {
-            const float a = fmaf(s0, xv[j], y0[j]) + fmaf(s2, xv[j], y2[j]);
-            const float c = fmaf(s1, xv[j], y1[j]) + fmaf(s3, xv[j], y3[j]);
-            o[j] = a + c;
-        }
-        if (full) {
-            if constexpr (sizeof(T) == 4) {
-                asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(out), "f"(o[0]), "f"(o[1]),
-                             "l"(ev)
-                             : "memory");
-            } else {
-                const unsigned q = __bfloat16_as_ushort(io<T>::to(o[0])) |
-                                   ((unsigned)__bfloat16_as_ushort(io<T>::to(o[1])) << 16);
-                *reinterpret_cast<unsigned*>(out) = q;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < kMP; ++j)
-                if (pos0 + j < L) out[j] = io<T>::to(o[j]);
-        }
+        for (int j = 0; j < MP; ++j)
+            if (pos0 + j < L) out[j] = io<T>::to(merged(dd, j, io<T>::cvt(x[j])));
     }
 }
 
-template <typename T>
-vmb_status launch_mean_merge_t(const void* x, const float* ybar, const float* Dskip, void* out, int B, int D, int H,
-                               int W, bool per_channel, cudaStream_t stream) {
+template <typename T, int MP>
+vmb_status launch_mean_merge_mp(const void* x, const float* ybar, const float* Dskip, void* out, int B, int D, int H,
+                                int W, bool per_channel, cudaStream_t stream) {
     const long long L = (long long)H * W;
-    const unsigned nblk = (unsigned)((L + kMMThreads * kMP - 1) / (kMMThreads * kMP));
+    const unsigned nblk = (unsigned)((L + kMMThreads * MP - 1) / (kMMThreads * MP));
     // channels per CTA: enough CTAs for a few waves, each amortising its ybar
     // reads over as many channels as that leaves
     const long long per_ch = (long long)nblk * B;
@@ -625,15 +654,29 @@ vmb_status launch_mean_merge_t(const void* x, const float* ybar, const float* Ds
     p.H = H;
     p.W = W;
     p.per_channel = per_channel ? 1 : 0;
-    p.vec = (L % kMP == 0) && al(x, kMP * sizeof(T)) && al(out, kMP * sizeof(T));
+    p.vec = (L % MP == 0) && al(x, MP * sizeof(T)) && al(out, MP * sizeof(T));
     p.dc = (int)dc;
     const dim3 grid(nblk, (unsigned)B, (unsigned)((D + dc - 1) / dc));
     if (grid.y > 65535u || grid.z > 65535u) return VMB_ERR_UNSUPPORTED;
     void* args[] = {&p};
-    return launch_kernel(reinterpret_cast<const void*>(&mean_merge_kernel<T>), grid, dim3(kMMThreads), 0, args, stream) ==
-                   cudaSuccess
+    return launch_kernel(reinterpret_cast<const void*>(&mean_merge_kernel<T, MP>), grid, dim3(kMMThreads), 0, args,
+                         stream) == cudaSuccess
                ? VMB_OK
                : VMB_ERR_CUDA;
+}
+
+template <typename T>
+vmb_status launch_mean_merge_t(const void* x, const float* ybar, const float* Dskip, void* out, int B, int D, int H,
+                               int W, bool per_channel, cudaStream_t stream) {
+    const long long L = (long long)H * W;
+    const auto fits = [&](int mp) {
+        return L % mp == 0 && reinterpret_cast<uintptr_t>(x) % (mp * sizeof(T)) == 0 &&
+               reinterpret_cast<uintptr_t>(out) % (mp * sizeof(T)) == 0;
+    };
+    if (sizeof(T) == 2 && fits(8))
+        return launch_mean_merge_mp<T, sizeof(T) == 2 ? 8 : 4>(x, ybar, Dskip, out, B, D, H, W, per_channel, stream);
+    if (fits(4)) return launch_mean_merge_mp<T, 4>(x, ybar, Dskip, out, B, D, H, W, per_channel, stream);
+    return launch_mean_merge_mp<T, 2>(x, ybar, Dskip, out, B, D, H, W, per_channel, stream);
 }
 // ------------------------------------------------------------ map transpose
 // xt[b, d, w, h] = x[b, d, h, w]: the column-major order of every (b, d) plane,
