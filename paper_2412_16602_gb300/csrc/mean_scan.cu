@@ -972,7 +972,22 @@ vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     const bool two = plan.np >= 8 && plan.chunk_len >= 64 && !zoh && a.L % 2 == 0 &&
                      (a.no_bcast || a.dtype == VMB_BF16) && al2(a.u) && (lr || al2(a.delta)) &&
                      (a.gather_h == 0 || al2(a.u_t));
-    KInfo ki = two ? mpick_pair(a.dtype, plan.np, plan.chunk_len, lr) : mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
+    KInfo ki = mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
+    if (two) {
+        // ... and where its waves do not cost more than they save: four CTAs share an
+        // SM at 0.87 of the time each takes of it, but a last wave costs at least
+        // three quarters of a full one (4 maps of 62x117x384: 912 CTAs, two full waves
+        // of three per SM, 228 us, or one and a half of four, 238)
+        const KInfo k2 = mpick_pair(a.dtype, plan.np, plan.chunk_len, lr);
+        const long long sms = device_sm_count(), n = (long long)plan.n_seq * plan.n_chunks;
+        auto cost = [&](const KInfo& k) {
+            const long long res = k.fn ? resident_ctas(k.fn, k.threads, k.smem) : 0;
+            if (res < 1) return 1e30;
+            const double full = (double)res / sms, rest = (double)(n % res) / sms;
+            return (n / res) * full + (n % res ? (rest > 0.75 * full ? rest : 0.75 * full) : 0.0);
+        };
+        if (0.87 * cost(k2) <= cost(ki)) ki = k2;
+    }
     if (!ki.fn) return VMB_ERR_CUDA;
     MeanParams p{};
     p.u = a.u;
