@@ -46,7 +46,7 @@ METRIC = ("selective-scan HBM GB/s and (B·K·D·L)/s, full vs channel-mean, "
 DEFAULT_WORKLOAD = "batch128_d256_n16_56x56_sigma0.05_f32"
 FALLBACK_HBM_GBS = 6800.0
 KERNELS = ["cross_scan", "full_scan", "mean_scan", "cross_merge_full", "cross_merge_mean"]
-SOURCES = {"full_scan": "full_scan.cu", "mean_scan": "mean_scan.cu", "cross_scan": "cross_scan_merge.cu",
+SOURCES = {"full_scan": "full_ws.cuh", "mean_scan": "mean_scan.cu", "cross_scan": "cross_scan_merge.cu",
            "cross_merge_full": "cross_scan_merge.cu", "cross_merge_mean": "cross_scan_merge.cu"}
 
 

@@ -38,9 +38,12 @@
  *     (programmatic dependent launch): their blocks may be scheduled while
  *     the previous kernel of the stream is finishing, and each waits
  *     (griddepcontrol.wait) for that kernel to complete before it reads or
- *     writes global memory.  (The exception: a warp-specialised full scan
+ *     writes global memory.  (Two exceptions: a warp-specialised full scan
  *     whose grid is smaller than one wave is launched normally, so that its
- *     blocks spread over every SM.)  Stream order is therefore kept for any
+ *     blocks spread over every SM; and inside the calls that start from the map,
+ *     the scan's blocks that do not read the map's transpose run beside the
+ *     kernel that writes it, which has itself waited for everything before the
+ *     call.)  Stream order is therefore kept for any
  *     preceding work; a caller's own kernel launched after a vmb call with
  *     the same attribute must likewise wait before touching vmb outputs.
  */
@@ -240,8 +243,10 @@ vmb_status vmb_mean_scan_merge_fwd(const void* u, const void* delta, const float
  *   delta [B, 4, D, L], Bs, Cs [B, 4, N, L] (dtype); A [4*D, N], Dskip [4*D],
  *   delta_bias [4*D] (fp32); flags and workspace as vmb_selective_scan_fwd with
  *   K = 4 (vmb_scan_workspace_bytes(VMB_PATH_FULL, B, 4, D, N, H, W, dtype)).
- * Where the warp-specialised scan kernel runs (16 states, rows of 16-byte
- * multiples, 16-byte aligned tensors, enough channel rows) direction k's step
+ * Short maps of 9 to 16 states (up to 256 pixels, by the number of channel rows) take one
+ * launch that reads the map in every direction's order and merges on chip; xt
+ * is then left as it was.  Where the warp-specialised scan kernel runs (rows of
+ * 16-byte multiples, 16-byte aligned tensors, enough channel rows) direction k's step
  * l reads the value the cross-scan would have put there: directions 0 and 2
  * the (b, d) planes of x row by row (forward and reversed), directions 1 and 3
  * the rows of xt, the transpose of every plane (written by this call), so the
@@ -387,7 +392,7 @@ vmb_status vmb_selection_fwd(const void* u, const float* WB, const float* WC, co
  *   formed inside the scan from z [B,K,R,L] fp32 and Wup [K,D,R] fp32 (R in
  *   1..16; VMB_ERR_UNSUPPORTED above); every other argument, flag and the
  *   workspace (vmb_scan_workspace_bytes(VMB_PATH_FULL, ...)) as there; y must
- *   not alias u.  The warp-specialised scan (16 states, rows of 16-byte
+ *   not alias u.  The warp-specialised scan (9 to 16 states, rows of 16-byte
  *   multiples, 16-byte aligned tensors, enough channel rows, Euler Bbar) reads
  *   z instead of the raw Deltas, i.e. R instead of D values per step and
  *   direction; for other plans the raw Deltas are written into y (rounded to

@@ -20,6 +20,16 @@
 // copies swizzle their 16-byte pieces so that a quarter warp's 128-bit reads of
 // one piece of consecutive rows hit distinct banks.
 //
+// What bounds it: at 16 states the dispatch of the packed update (about 6.4
+// cycles of a scheduler per update: a packed FMA with three register operands takes
+// 3.3, a product 2.1, an ex2 1) and the softplus; at one state HBM (90% of it).  GB300,
+// fp32, us: 128 maps of 56x56x256, 16 states, one lane 1448, two 1535; 24576 rows of
+// 56x56 471 with one lane, 350 with two (a warp per scheduler leaves the step's
+// latency open, 106 ns a step with one lane and 51 with two); one state 1355 with
+// barrier-staged tiles, 795 here.  Eight steps are unrolled together with one lane, 16 with
+// two (4: 10% slower; 16 with one lane spill); starting the next stage's softplus
+// before this stage's updates was 20% slower.
+//
 // Requires rows of 16-byte multiples and 16-byte aligned tensors (the host
 // picks this variant only then); every wait is bounded.
 // Gathering from the map (GATHER, App. A cross-scan without the cross-scanned

@@ -17,8 +17,10 @@
 // Why: at these lengths the streaming kernels spend their time on stage
 // prologues and element-wise loads (rows of 49 steps are not 16-byte
 // multiples), and a block of three launches spends it on the launches.
-// Measured on GB300 against the kernels that took these sizes before: see the
-// rule in full_scan.cu (plan_full).
+// Bound by instruction dispatch (the update loop, and about as many again for
+// staging short rows): block of 32 maps of 7x7x1536 213 -> 69 us, of one 14x14x192 map 38.5
+// -> 11 us on the device.  Which lengths and row counts take it, with both
+// sides measured: small_rule in full_scan.cu.
 #include <mutex>
 
 #include "vmb_common.cuh"

@@ -16,9 +16,9 @@
 extern "C" {
 #endif
 
-/* Force the full scan's tile shape (0..15 for 16 states; taken modulo the
- * number of shapes of the padded state count) and, for the look-back shapes,
- * the number of L-chunks (<= 1: one chunk).  shape < 0 restores the planner.
+/* Force the full scan's tile shape (0..23 for 16 states; taken modulo the
+ * number of shapes of the padded state count) and, for the look-back and
+ * warp-specialised shapes, the number of L-chunks (<= 1: one chunk).  shape < 0 restores the planner.
  * Ignored under VMB_FLAG_B_ZOH, which has one shape.  Returns 0. */
 int vmb_testing_force_full_plan(int shape, int chunks);
 
