@@ -1718,9 +1718,10 @@ ShapeRoles roles(int np) {
 // One lane, the warp-specialised and the packed streaming kernel share their
 // arithmetic, so the block is bit-identical to the separate calls either way
 // (where the block may take one lane the scan alone keeps to one lane and one
-// pass); 4 and 16 lanes (other sums over the states) are taken by both or by neither.
+// pass, so the rule for both goes by the tensors of the scan alone: `seq_ok`); 4 and 16
+// lanes (other sums over the states) are taken by both or by neither.
 bool small_map_one_lane(int L) { return 2 * (small_scan_smem(1, L, true) + 1024) <= kSmemPerSm; }
-int small_rule(const ScanArgs& a, bool map, bool tma_ok, int sms) {
+int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (a.L > 256) return 0;
     for (const int G : {16, 4}) {
         const long long ctas = ((long long)a.B * a.K * ((a.D + 32 / G - 1) / (32 / G)) + 3) / 4;
@@ -1729,7 +1730,7 @@ int small_rule(const ScanArgs& a, bool map, bool tma_ok, int sms) {
         if (ctas <= fit && ctas <= most) return G;
     }
     if (small_scan_smem(1, a.L, false) > kSmallMaxSmem) return 0;
-    if (!tma_ok) return 1;
+    if (!seq_ok) return 1;
     return map && small_map_one_lane(a.L) ? 1 : 0;
 }
 
@@ -1790,9 +1791,12 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // tensors (tiled tensor copies) and the driver's tensor-map encoder
     const size_t es = a.dtype == VMB_BF16 ? 2 : 4;
     const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    const bool tma_ok = !a.no_tma && (size_t)a.L * es % 16 == 0 && al16(a.u) && al16(a.delta) && al16(a.Bs) &&
-                        al16(a.Cs) && al16(a.y) && (a.gather_h == 0 || al16(a.u_t)) &&
-                        tensor_map_encoder() != nullptr;
+    const bool map = a.gather_h > 0;
+    // seq_ok: the call on materialised sequences has them.  For a call from the map that is
+    // the scan it must equal bit for bit, whatever the alignment of x and xt
+    const bool seq_ok = !a.no_tma && (size_t)a.L * es % 16 == 0 && (map || al16(a.u)) && al16(a.delta) && al16(a.Bs) &&
+                        al16(a.Cs) && al16(a.y) && tensor_map_encoder() != nullptr;
+    const bool tma_ok = seq_ok && (!map || (al16(a.u) && al16(a.u_t)));
     // the three-launch variant: a grid of 64-step, one-lane chunks fits in two
     // waves (beyond that its aggregate traffic outweighs the other plans).  It
     // then runs as two lanes per channel over 32-step chunks, which measured fastest
@@ -1821,7 +1825,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             const long long want = (res + tiles - 1) / tiles, mx = (a.L + 255) / 256;
             n_chunks = (int)(want < mx ? want : mx);
         }
-    } else if (const int G = np == 16 ? small_rule(a, a.gather_h > 0, tma_ok, sms) : 0) {
+    } else if (const int G = np == 16 ? small_rule(a, map, seq_ok, sms) : 0) {
         shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
     } else if (np == 16 && tma_ok && rows < 6LL * sms && chunk_grid_fits()) {
         shape = kChunkShape + 1;

@@ -477,8 +477,9 @@ vmb_status vmb_ss2d_full_fwd(const void* x, void* xt, const void* delta, const f
     ScanPlan plan{};
     s = plan_full(a, &plan);
     if (s != VMB_OK) return s;
-    if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
-    if (const int G = full_plan_small(plan)) return launch_small(a, G, out, H, W, stream);
+    const int small = full_plan_small(plan);
+    if ((small || full_plan_gathers(plan)) && workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
+    if (small) return launch_small(a, small, out, H, W, stream);
     if (full_plan_gathers(plan)) {
         s = launch_map_transpose(x, xt, B, D, H, W, dtype, stream);
         if (s != VMB_OK) return s;

@@ -52,3 +52,28 @@ def test_short_sequences(shape, plan, force_plan):
     check(to_numpy(y), y_ref, dt, "full y")
     assert torch.equal(ym, y) and torch.equal(out, vmb.vmb_cross_merge(y, H, W))
     check(to_numpy(out), out_ref, dt, "full out from the map")
+
+
+@pytest.mark.parametrize("case", [(8, 512, 10, 12, "f32"), (8, 512, 8, 13, "bf16"), (3, 700, 9, 12, "f32"),
+                                  (8, 512, 8, 8, "f32"), (2, 40, 10, 12, "f32"), (8, 256, 12, 12, "f32"), (2, 64, 28, 28, "f32"),
+                                  (1, 40, 40, 42, "bf16")],
+                         ids=lambda c: "B{}_D{}_{}x{}_{}".format(*c))
+@pytest.mark.parametrize("which", ["x", "xt"])
+def test_block_of_an_unaligned_map(case, which):
+    """x or xt one element past 16-byte alignment: y and out are those of the three calls
+    on aligned sequences, bit for bit, with a workspace of the queried size."""
+    B, D, H, W, dt = case
+    wl = workloads.small_case(B=B, D=D, N=16, H=H, W=W, dtype=dt, seed=B + D)
+    g = workloads.make_device_inputs(wl, DEV, seed=3, params="random")
+    args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+    x = g["x"]
+    off = torch.empty(x.numel() + 1, dtype=x.dtype, device=DEV)[1:]
+    ws = torch.zeros(vmb.vmb_scan_workspace_bytes(vmb.VMB_PATH_FULL, B, 4, D, 16, H, W, x.dtype), dtype=torch.uint8,
+                     device=DEV)
+    if which == "x":
+        out, y = vmb.vmb_ss2d_full_fwd(off.view(x.shape).copy_(x), *args, workspace=ws)
+    else:
+        out, y = vmb.vmb_ss2d_full_fwd(x, *args, xt=off.view(B, D, W, H), workspace=ws)
+    y2 = vmb.vmb_selective_scan_fwd(vmb.vmb_cross_scan(x), *args, H, W)
+    assert vmb.vmb_read_status(ws) == vmb.VMB_OK
+    assert torch.equal(y, y2) and torch.equal(out, vmb.vmb_cross_merge(y2, H, W))
