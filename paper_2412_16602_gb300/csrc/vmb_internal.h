@@ -206,6 +206,7 @@ vmb_status launch_mean_bwd(const MeanBwdArgs& a, cudaStream_t stream);
 // Whether the channel-mean scan of this plan runs beside the transpose by planes.
 bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W);
 vmb_status launch_scan_only(const OnlyArgs& a, cudaStream_t stream);
+bool selection_two_buffers(long long grid, int D, int sms);
 vmb_status launch_mean_merge(const void* x, const float* ybar, const float* Dskip, void* out, int B, int D, int H,
                              int W, bool per_channel_skip, vmb_dtype dt, cudaStream_t stream);
 
