@@ -21,17 +21,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr size_t kMaxSmem = 200 * 1024;
 
-struct FastDiv {
-    unsigned d, m, s;
-};
-FastDiv make_fastdiv(unsigned d) {
-    unsigned s = 0;
-    while ((1ull << s) < d) ++s;
-    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
-    return {d, (unsigned)m, s};
-}
-__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
-
 struct CsmParams {
     const void* in;
     void* out;
@@ -51,6 +40,17 @@ union Vec {
 
 // Tile indices of a plane's positions, computed once per CTA (the planes of a CTA
 // share them; a division per element and plane was half of these kernels'
+// instructions): row[r] of pixel r in row-major order, col[m] of the m-th pixel in
+// column-major order.
+__device__ __forceinline__ void plane_tables(unsigned short* row, unsigned short* col, const CsmParams& p, bool by_col) {
+    for (int i = threadIdx.x; i < p.L; i += kThreads) {
+        const int h = (int)fdiv((unsigned)i, p.fW), w = i - h * p.W;
+        row[i] = (unsigned short)(by_col ? w * (p.H + 1) + h : h * (p.W + 1) + w);
+        const int w1 = (int)fdiv((unsigned)i, p.fH), h1 = i - w1 * p.H;
+        col[i] = (unsigned short)(by_col ? w1 * (p.H + 1) + h1 : h1 * (p.W + 1) + w1);
+    }
+}
+
 // Without tables (TAB false: planes of kBandMinL pixels or more, whose tables would
 // take shared memory from the plane and are used for one plane only) the indices
 // are computed where they are used.
@@ -71,17 +71,6 @@ __device__ __forceinline__ PlaneIndex row_index(const unsigned short* tab, const
 }
 __device__ __forceinline__ PlaneIndex col_index(const unsigned short* tab, const CsmParams& p, bool by_col) {
     return {tab, p.fH, by_col ? p.H + 1 : 1, by_col ? 1 : p.W + 1};
-}
-
-// instructions): row[r] of pixel r in row-major order, col[m] of the m-th pixel in
-// column-major order.
-__device__ __forceinline__ void plane_tables(unsigned short* row, unsigned short* col, const CsmParams& p, bool by_col) {
-    for (int i = threadIdx.x; i < p.L; i += kThreads) {
-        const int h = (int)fdiv((unsigned)i, p.fW), w = i - h * p.W;
-        row[i] = (unsigned short)(by_col ? w * (p.H + 1) + h : h * (p.W + 1) + w);
-        const int w1 = (int)fdiv((unsigned)i, p.fH), h1 = i - w1 * p.H;
-        col[i] = (unsigned short)(by_col ? w1 * (p.H + 1) + h1 : h1 * (p.W + 1) + w1);
-    }
 }
 
 // Directions 0 and 2 are written straight from the loaded values, 1 and 3 (the same
@@ -237,13 +226,6 @@ __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p
 
 // ---------------------------------------------------------------- band kernels
 // Maps of at least kBandMinL pixels: one CTA per band of rows of one map, so
-// Rows of a merge band: 32 (fp32) or 16 (bf16), fewer while the tiles would not fit.
-inline int merge_band_rows(int W, int es) {
-    int mrb = es == 4 ? 32 : 16;
-    while (mrb > kRB && (size_t)2 * mrb * (W + 1) * es > kMaxSmem) mrb /= 2;
-    return mrb;
-}
-
 // that even a batch-1 problem has enough CTAs.  Directions 0 and 2 of a band are
 // one contiguous run of the sequence; directions 1 and 3 are W runs of one step
 // per row of the band, written from (scan) or read into (merge) a [rows][W+1]
@@ -254,6 +236,13 @@ inline int merge_band_rows(int W, int es) {
 constexpr int kRB = 8;
 constexpr int kBandMinL = 1024;
 constexpr int kBandThreads = 128;
+
+// Rows of a merge band: 32 (fp32) or 16 (bf16), fewer while the tiles would not fit.
+inline int merge_band_rows(int W, int es) {
+    int mrb = es == 4 ? 32 : 16;
+    while (mrb > kRB && (size_t)2 * mrb * (W + 1) * es > kMaxSmem) mrb /= 2;
+    return mrb;
+}
 
 struct BandParams {
     const void* in;
@@ -426,6 +415,17 @@ __global__ void cross_merge_direct(const T* ys, T* out, int D, int H, int W, lon
     pdl_wait();
     pdl_launch_dependents();
     const long long L = (long long)H * W;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const long long pos = e % L, pl = e / L, d = pl % D, b = pl / D;
+        const long long h = pos / W, w = pos % W, p1 = w * H + h;
+        const T* r = ys + (b * 4 * D + d) * L;
+        const long long st = (long long)D * L;
+        const float a = io<T>::cvt(r[pos]) + io<T>::cvt(r[2 * st + L - 1 - pos]);
+        const float c = io<T>::cvt(r[st + p1]) + io<T>::cvt(r[3 * st + L - 1 - p1]);
+        out[e] = io<T>::to(a + c);
+    }
+}
+
 }  // namespace
 
 // Kernel of a cross-scan or cross-merge.  Below 1024 pixels whole planes are staged
@@ -462,17 +462,6 @@ CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, b
 }
 
 namespace {
-
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const long long pos = e % L, pl = e / L, d = pl % D, b = pl / D;
-        const long long h = pos / W, w = pos % W, p1 = w * H + h;
-        const T* r = ys + (b * 4 * D + d) * L;
-        const long long st = (long long)D * L;
-        const float a = io<T>::cvt(r[pos]) + io<T>::cvt(r[2 * st + L - 1 - pos]);
-        const float c = io<T>::cvt(r[st + p1]) + io<T>::cvt(r[3 * st + L - 1 - p1]);
-        out[e] = io<T>::to(a + c);
-    }
-}
 
 template <typename T>
 vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int H, int W, cudaStream_t stream) {
@@ -753,11 +742,6 @@ vmb_status launch_mean_merge_t(const void* x, const float* ybar, const float* Ds
 // vector's columns and the vector reads of a row both spread over the banks.
 constexpr int kTrThreads = 512;
 constexpr int kTrVals = 4;    // vectors (VEC) or 4-element groups a thread holds
-inline bool transpose_vec(const void* x, const void* xt, int H, int W, int es) {
-    return W % (16 / es) == 0 && H % (16 / es) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(xt)) & 15u) == 0;
-}
-inline int transpose_stride(int H, int VE, bool vec) { return vec ? (H + 8 * VE - 1) / (8 * VE) * (8 * VE) : H | 1; }
-
 constexpr size_t kTrSmem = kTransposeSmem - 1024;
 
 struct TransposeParams {
@@ -768,6 +752,11 @@ struct TransposeParams {
     long long planes, items;
     FastDiv fP, fA, fB;  // units per plane, per row of x, per row of xt
 };
+
+inline bool transpose_vec(const void* x, const void* xt, int H, int W, int es) {
+    return W % (16 / es) == 0 && H % (16 / es) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(xt)) & 15u) == 0;
+}
+inline int transpose_stride(int H, int VE, bool vec) { return vec ? (H + 8 * VE - 1) / (8 * VE) * (8 * VE) : H | 1; }
 
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(kTrThreads) map_transpose_kernel(const TransposeParams p) {

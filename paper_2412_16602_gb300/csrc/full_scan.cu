@@ -1508,6 +1508,10 @@ KernelInfo info_for() {
 template <typename T, bool ZOH>
 KernelInfo lanes_info() {
     using LY = Layout<T, 16, LanesShape>;
+    // at most three CTAs per SM: with a fourth, grids of two to three per SM, launched behind
+    // a kernel that still runs, stack on the SMs freed first (14 sequences of 512 channels, 48 steps,
+    // bf16: 6.1 us with three, 8.8 with four)
+    constexpr size_t kSmem = LY::raw_bytes > 58 * 1024 ? LY::raw_bytes : 58 * 1024;
     const void* fn = reinterpret_cast<const void*>(&full_scan_lanes_kernel<T, ZOH>);
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
@@ -1520,10 +1524,6 @@ KernelInfo lanes_info() {
 template <typename T, class CS>
 KernelInfo chunk_info() {
     using LY = ChunkLayout<T, CS>;
-    // at most three CTAs per SM: with a fourth, grids of two to three per SM, launched behind
-    // a kernel that still runs, stack on the SMs freed first (14 sequences of 512 channels, 48 steps,
-    // bf16: 6.1 us with three, 8.8 with four)
-    constexpr size_t kSmem = LY::raw_bytes > 58 * 1024 ? LY::raw_bytes : 58 * 1024;
     const void* fa = reinterpret_cast<const void*>(&full_chunk_kernel<T, CS, false>);
     const void* ff = reinterpret_cast<const void*>(&full_chunk_kernel<T, CS, true>);
     static std::once_flag once;
@@ -1749,20 +1749,20 @@ int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (!seq_ok) return 1;
     return map && small_map_one_lane(a.L) ? 1 : 0;
 }
-
-// Estimated time (ns) of the warp-specialised kernel, and the number of chunks
-// it would take (1: one pass).  A CTA takes a fixed time per step that grows
-// with the CTAs that share an SM; cut into P + 1 chunks, P CTAs a tile run
-// concurrently and each passes over two chunks.  ns per step with one, two and
-// three CTAs per SM, measured on GB300 (fp32, 56x56 maps): 16 states, two lanes a
-// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8).
-double ws_estimate(int np, long long tiles, int L, int sms, int ts, int* chunks) {
-    const double per_step[4][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {51, 79, 111}};
-    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 : 3];
-    double best = 0.0;
 // Short sequences alone, in rows that the barrier-staged kernels copy 16 bytes at a time: the
 // lane-per-state kernel instead of 4 or 16 lanes of whole sequences.  It streams stages of 32
 // steps, so a length just past one pays for the next; the whole-sequence kernel's loads of
+// 2-byte elements wait.  us, lane-per-state and whole sequences, fp32: 5 rows per SM of 96 steps 5.0 and
+// 5.4, of 100 6.1 and 5.6; 10 of 224 steps 9.5 and 20.2, 22 of 64 steps 5.1 and 7.4; 30 of 40 steps
+// 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
+// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.
+bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
+    const int staged = (L + 31) / 32 * 32;
+    if (dt == VMB_BF16) return L >= 16;
+    if (rows <= 6LL * sms) return 16 * staged <= 17 * L;
+    if (rows <= 24LL * sms) return L >= 16;
+    return rows <= 48LL * sms && (L >= 64 || 8 * staged <= 9 * L);
+}
 
 // Estimated time (ns) of the warp-specialised kernel, and the number of chunks
 // it would take (1: one pass).  A CTA takes a fixed time per step that grows
@@ -1776,17 +1776,6 @@ double ws_estimate(int np, bool two, long long tiles, int L, int sms, int ts, in
     const double per_step[5][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {41, 59, 72}, {51, 79, 111}};
     const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 + two : 4];
     double best = 0.0;
-// 2-byte elements wait.  us, lane-per-state and whole sequences, fp32: 5 rows per SM of 96 steps 5.0 and
-// 5.4, of 100 6.1 and 5.6; 10 of 224 steps 9.5 and 20.2, 22 of 64 steps 5.1 and 7.4; 30 of 40 steps
-// 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
-// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.
-bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
-    const int staged = (L + 31) / 32 * 32;
-    if (dt == VMB_BF16) return L >= 16;
-    if (rows <= 6LL * sms) return 16 * staged <= 17 * L;
-    if (rows <= 24LL * sms) return L >= 16;
-    return rows <= 48LL * sms && (L >= 64 || 8 * staged <= 9 * L);
-}
     for (int P = 1; P <= 24; ++P) {
         if (P > 1 && L / (P + 1) < 4 * ts) break;
         const long long per_sm = (tiles * P + sms - 1) / sms;
@@ -1935,6 +1924,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                 if (a.L / want_n >= 256) {
                     shape = r.chunk_narrow;
                     ki = kn;
+                    res = rn;
                     n_chunks = (int)want_n;
                 } else {
                     KernelInfo kw{};
@@ -1943,8 +1933,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                     const long long tiles_w = a.B * a.K * (long long)((a.D + kw.DT - 1) / kw.DT);
                     const long long want_w = (rw + tiles_w - 1) / tiles_w, mx = (a.L + 127) / 128;
                     shape = r.chunk_wide;
-                    res = rn;
                     ki = kw;
+                    res = rw;
                     n_chunks = (int)(want_w < mx ? want_w : mx);
                 }
             }
@@ -1953,7 +1943,6 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     if (const int G = small_lanes(np, shape)) {
         ki = KernelInfo{};
         ki.G = G;
-                    res = rw;
         ki.DT = 32 / G;
         ki.ts = a.L;
         n_chunks = 1;

@@ -33,20 +33,6 @@ constexpr int kSmThreads = 128;  // four warps
 constexpr int kNP = 16;          // states, zero padded
 constexpr int kBC = 2 * kNP;     // floats of one step's B and C
 
-// Division by an invariant integer by multiply-high (Granlund & Montgomery,
-// "Division by invariant integers using multiplication", PLDI 1994), for
-// dividends below 2^31.
-struct FastDiv {
-    unsigned d, m, s;
-};
-FastDiv make_fastdiv(unsigned d) {
-    unsigned s = 0;
-    while ((1ull << s) < d) ++s;
-    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
-    return {d, (unsigned)m, s};
-}
-__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
-
 struct SmallParams {
     const void* u;  // [B][K][D][L], or (MAP) the map x [B][D][L]
     const void* dl;
@@ -66,10 +52,7 @@ struct SmallParams {
     FastDiv fL, fW;
 };
 
-__device__ __forceinline__ void load_elem(float* dst, const float* src) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(src) : "memory");
-}
+__device__ __forceinline__ void load_elem(float* dst, const float* src) { cp_async4(dst, src, 4); }
 __device__ __forceinline__ void load_elem(float* dst, const __nv_bfloat16* src) { *dst = __bfloat162float(*src); }
 
 // `rows` consecutive rows of L elements into rows of stride RX, by `step`
@@ -120,7 +103,6 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     const int rows = min(CT, p.D - d0);
     const long long bk = MAP ? seq * 4 + warp : seq;
     const int k = MAP ? warp : (int)(bk % p.K);
-    // lane g owns the states g, g + G, ...: their columns lie together
     // shared memory: the map tile (MAP) or each warp's u rows, then each warp's
     // Delta / y rows, then each warp's B and C rows
     float* ut = sm + (MAP ? 0 : warp * CT * RX);
@@ -138,6 +120,7 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     if (p.N < kNP)
         for (int i = lane; i < L * kBC; i += 32) bc[i] = 0.0f;
     __syncwarp();
+    // lane g owns the states g, g + G, ...: their columns lie together
 #pragma unroll 4
     for (int i = lane; i < p.N * L; i += 32) {
         const int n = (int)fdiv((unsigned)i, p.fL), t = i - n * L;
@@ -183,10 +166,6 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     auto block = [&](int t0, auto tail_tag) {
         constexpr bool TAIL = decltype(tail_tag)::value;
         float us[BS], yp[BS];
-                // sum over the states: one chain, as in the other kernels with one lane
-                // a channel, or (G = 4) the first two levels of the tree over the 16
-                // states that the lane-per-state kernels add across lanes (scalar additions,
-                // with which the products are not fused)
 #pragma unroll
         for (int j = 0; j < BS; ++j) {
             const bool in = !TAIL || t0 + j < L;  // past the end: delta = u = 0, an identity step
@@ -204,6 +183,10 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
                 h[0] = fmaf(ex2(dv * A2[0]), h[0], du * b);
                 yp[j] = cc * h[0];
             } else {
+                // sum over the states: one chain, as in the other kernels with one lane
+                // a channel, or (G = 4) the first two levels of the tree over the 16
+                // states that the lane-per-state kernels add across lanes (scalar additions,
+                // with which the products are not fused)
                 const float2 dd = make_float2(dv, dv), uu = make_float2(du, du);
                 float2 ya = make_float2(0.0f, 0.0f), half = ya;
 #pragma unroll
