@@ -79,65 +79,10 @@ __device__ __forceinline__ float sel4(const float (&v)[4], int j) {
     return j == 0 ? v[0] : j == 1 ? v[1] : j == 2 ? v[2] : v[3];
 }
 
-// load_tile for rows that are not 16-byte aligned.
-template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B>
-__device__ __forceinline__ void load_tile_elements(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
-                                                   int l0) {
-    // element by element: thread i copies step i % kTS of rows i / kTS + k RPP, u and
-    // delta (B and C) together; fp32 as 4-byte asynchronous copies, in flight like
-    // the 16-byte ones, bf16 (2-byte elements) through registers, a batch of
-    // independent loads at a time.  Only rows of the problem are visited: rows of u
-    // and delta past nrows keep what they held (the lanes that read them store
-    // nothing), those of B and C past N are zeroed (GB300, bf16, unaligned rows, us:
-    // 21 maps of 38x51x3, two states, 243 visiting every row of the tile, see the
-    // test of narrow tiles).
-    constexpr int RPP = kThreads / kTS;
-    static_assert(kThreads % kTS == 0, "tile loader mapping");
-    const int t = threadIdx.x % kTS, r0 = threadIdx.x / kTS;
-    const bool colok = l0 + t < p.L;
-    // `n` rows, of which the first `valid` come from src
-    auto rows = [&](T* to, const void* src, size_t first, int valid, int n) {
-        const T* g = static_cast<const T*>(src) + (first + r0) * p.L + (colok ? l0 + t : 0);
-        const size_t step = (size_t)RPP * p.L;
-        to += r0 * RS + t;
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll 2
-            for (int r = r0; r < n; r += RPP, g += step, to += RPP * RS) {
-                const bool ok = colok && r < valid;
-                cp_async4(to, ok ? g : src, ok ? 4 : 0);
-            }
-        } else {
-            constexpr int kBatch = 8;
-#pragma unroll 1
-            for (int r = r0; r < n; r += kBatch * RPP) {
-                T v[kBatch];
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q, g += step) v[q] = colok && r + q * RPP < valid ? *g : T(0.0f);
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q, to += RPP * RS)
-                    if (r + q * RPP < n) *to = v[q];
-            }
-        }
-    };
-    rows(dst, p.u, row0, nrows, nrows);
-    rows(dst + DT * RS, p.dl, row0, nrows, nrows);
-    if constexpr (WITH_B) {
-        rows(dst + 2 * DT * RS, p.Bs, bcrow0, p.N, NP);
-        if constexpr (WITH_C) rows(dst + (2 * DT + NP) * RS, p.Cs, bcrow0, p.N, NP);
-    }
-}
-
-// The same as a function of its own, for the kernels whose registers are all taken.
-template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B>
-__device__ __noinline__ void load_tile_elements_call(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
-                                                     int l0) {
-    load_tile_elements<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
-}
-
 // Copy kTS steps (from l0) of DT u and delta rows and of the NP B (and C) rows
 // into shared memory rows of stride RS: u at row 0, delta at row DT, B at 2 DT,
-// C at 2 DT + NP.  Steps past the problem and rows of B and C past N are zero-filled.
-template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B = true, bool CALL = false>
+// C at 2 DT + NP.  Rows and steps past the problem are zero-filled.
+template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B = true>
 __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
                                           int l0) {
     constexpr int VE = 16 / sizeof(T);  // elements per 16-byte chunk
@@ -179,10 +124,53 @@ __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t ro
             }
         }
     } else {
-        if constexpr (CALL)
-            load_tile_elements_call<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
-        else
-            load_tile_elements<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
+        // element by element: fp32 as 4-byte asynchronous copies, in flight like the
+        // 16-byte ones; bf16 (2-byte elements) through registers, a batch of
+        // independent loads at a time
+        constexpr int nU = DT * kTS, nB = NP * kTS;
+        constexpr int total = 2 * nU + (WITH_B ? (WITH_C ? 2 : 1) * nB : 0);
+        auto locate = [&](int i, const T** src, int* at) -> bool {  // source, offset in dst; false: zero
+            if (i < 2 * nU) {
+                const int j = i < nU ? i : i - nU;
+                const int r = j / kTS, t = j % kTS;
+                *at = (i < nU ? 0 : DT * RS) + r * RS + t;
+                *src = (i < nU ? u : dl) + (row0 + r) * (size_t)L + l0 + t;
+                return r < nrows && l0 + t < L;
+            }
+            const int i2 = i - 2 * nU;
+            const int j = i2 < nB ? i2 : i2 - nB;
+            const int r = j / kTS, t = j % kTS;
+            *at = 2 * DT * RS + (i2 < nB ? 0 : NP * RS) + r * RS + t;
+            *src = (i2 < nB ? Bs : Cs) + (bcrow0 + r) * (size_t)L + l0 + t;
+            return r < p.N && l0 + t < L;
+        };
+        if constexpr (sizeof(T) == 4) {
+            for (int i = threadIdx.x; i < total; i += kThreads) {
+                const T* src;
+                int at;
+                const bool ok = locate(i, &src, &at);
+                cp_async4(dst + at, ok ? src : u, ok ? 4 : 0);
+            }
+        } else {
+            constexpr int kBatch = 8;
+            for (int i0 = threadIdx.x; i0 < total; i0 += kBatch * kThreads) {
+                T v[kBatch];
+                int at[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q) {
+                    const int i = i0 + q * kThreads;
+                    v[q] = T(0.0f);
+                    at[q] = -1;
+                    if (i < total) {
+                        const T* src;
+                        if (locate(i, &src, &at[q])) v[q] = *src;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (at[q] >= 0) dst[at[q]] = v[q];
+            }
+        }
     }
 }
 
@@ -1299,7 +1287,7 @@ __global__ void __launch_bounds__(PackedLayout<T, PS>::THREADS, PS::MINB) full_p
     const int nst = (L + TS - 1) / TS;
 #pragma unroll
     for (int q = 0; q < NSTG - 1; ++q) {
-        if (q < nst) load_tile<T, NP, DT, TS, RS, THREADS, true, true, true>(p, raw + q * SLOT, row0, bcrow0, nrows, q * TS);
+        if (q < nst) load_tile<T, NP, DT, TS, RS, THREADS, true>(p, raw + q * SLOT, row0, bcrow0, nrows, q * TS);
         cp_async_commit();
     }
     const float bias = cval ? p.bias[(size_t)k * p.D + d] : 0.0f;
@@ -1347,7 +1335,7 @@ __global__ void __launch_bounds__(PackedLayout<T, PS>::THREADS, PS::MINB) full_p
         cp_async_wait<NSTG - 3>();  // stages <= s+1 have landed
         __syncthreads();            // ... for every thread; stage s is prepared
         if (s + NSTG - 1 < nst)
-            load_tile<T, NP, DT, TS, RS, THREADS, true, true, true>(p, raw + ((s + NSTG - 1) % NSTG) * SLOT, row0, bcrow0, nrows,
+            load_tile<T, NP, DT, TS, RS, THREADS, true>(p, raw + ((s + NSTG - 1) % NSTG) * SLOT, row0, bcrow0, nrows,
                                                         l0 + (NSTG - 1) * TS);
         cp_async_commit();
         if (s + 1 < nst) prepare(s + 1);
@@ -1508,17 +1496,13 @@ KernelInfo info_for() {
 template <typename T, bool ZOH>
 KernelInfo lanes_info() {
     using LY = Layout<T, 16, LanesShape>;
-    // at most three CTAs per SM: with a fourth, grids of two to three per SM, launched behind
-    // a kernel that still runs, stack on the SMs freed first (14 sequences of 512 channels, 48 steps,
-    // bf16: 6.1 us with three, 8.8 with four)
-    constexpr size_t kSmem = LY::raw_bytes > 58 * 1024 ? LY::raw_bytes : 58 * 1024;
     const void* fn = reinterpret_cast<const void*>(&full_scan_lanes_kernel<T, ZOH>);
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::raw_bytes);
     });
-    return {attr_err == cudaSuccess ? fn : nullptr, kSmem, 16, LY::DT, 256, LY::TS};
+    return {attr_err == cudaSuccess ? fn : nullptr, LY::raw_bytes, 16, LY::DT, 256, LY::TS};
 }
 
 template <typename T, class CS>
@@ -1612,7 +1596,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows, long long planes, int box_ts,
                  int box_rows, bool swizzled = false) {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc || refuse_tensor_maps()) return false;
+    if (!enc) return false;
     const cuuint64_t es = dt == VMB_BF16 ? 2 : 4;
     const cuuint64_t dims[3] = {(cuuint64_t)L, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)L * es, (cuuint64_t)rows * L * es};
@@ -1628,7 +1612,7 @@ bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows
 
 // Tile shapes per padded state count, in order of preference (fewest lanes
 // per channel first).  The zero-order-hold variant uses the first shape.
-int shape_count(int np) { return np <= 4 ? 2 : np == 8 ? 4 : 24; }
+int shape_count(int np) { return np <= 4 ? 2 : np == 8 ? 3 : 24; }
 constexpr int kLanesShape = 7;   // index of the lane-per-state variant (N <= 16 padded to 16)
 constexpr int kChunkShape = 8;   // first index of the three-launch chunked variant (shapes 8 to 11)
 bool is_chunk_shape(int np, int shape) { return np == 16 && shape >= kChunkShape && shape < kChunkShape + 4; }
@@ -1636,13 +1620,14 @@ constexpr int kStreamShape = 12;  // first index of the streaming one-lane varia
 bool is_stream_shape(int np, int shape) { return np == 16 && shape >= kStreamShape && shape < kStreamShape + 4; }
 constexpr int kPackedShape = 16;  // first index of the packed streaming variant (shapes 16 to 18: G = 1, 2, 4)
 bool is_packed_shape(int np, int shape) { return np == 16 && shape >= kPackedShape && shape < kPackedShape + 3; }
-// The warp-specialised variant (tensor copies; 16-byte rows and aligned tensors): one
-// lane per channel, and two with 8 or 16 states.
+// The warp-specialised variant (tensor copies; 16-byte rows and aligned tensors): the
+// last shape of fewer states; 16 states: one lane per channel (19) or two (23).
 constexpr int kWsShape = 19, kWsTwoShape = 23;
 int ws_shape(int np) { return np <= 4 ? 1 : np == 8 ? 2 : kWsShape; }
-int ws_two_shape(int np) { return np == 16 ? kWsTwoShape : np == 8 ? 3 : -1; }
-bool is_ws_shape(int np, int shape) { return shape == ws_shape(np) || shape == ws_two_shape(np); }
-int ws_variant(int np, int shape) { return shape == ws_two_shape(np) ? kWsTwoLanes : kWsOneLane; }
+bool is_ws_shape(int np, int shape) {
+    return shape == ws_shape(np) || (np == 16 && shape == kWsTwoShape);
+}
+int ws_variant(int np, int shape) { return np == 16 && shape == kWsTwoShape ? kWsTwoLanes : kWsOneLane; }
 constexpr int kSmallShape = 20;  // whole short sequences in shared memory (shapes 20 to 22: G = 1, 4, 16; small_map.cu)
 int small_lanes(int np, int shape) {
     return np == 16 && shape >= kSmallShape && shape < kSmallShape + 3 ? 1 << (2 * (shape - kSmallShape)) : 0;
@@ -1733,9 +1718,8 @@ ShapeRoles roles(int np) {
 // One lane, the warp-specialised and the packed streaming kernel share their
 // arithmetic, so the block is bit-identical to the separate calls either way
 // (where the block may take one lane the scan alone keeps to one lane and one
-// pass, so the rule for both goes by the tensors of the scan alone: `seq_ok`); 4 and
-// 16 lanes sum over the states in the order of the lane-per-state kernel, which the
-// scan alone takes instead where it is faster (lanes_beat_small).
+// pass, so the rule for both goes by the tensors of the scan alone: `seq_ok`); 4 and 16
+// lanes (other sums over the states) are taken by both or by neither.
 bool small_map_one_lane(int L) { return 2 * (small_scan_smem(1, L, true) + 1024) <= kSmemPerSm; }
 int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (a.L > 256) return 0;
@@ -1749,32 +1733,16 @@ int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (!seq_ok) return 1;
     return map && small_map_one_lane(a.L) ? 1 : 0;
 }
-// Short sequences alone, in rows that the barrier-staged kernels copy 16 bytes at a time: the
-// lane-per-state kernel instead of 4 or 16 lanes of whole sequences.  It streams stages of 32
-// steps, so a length just past one pays for the next; the whole-sequence kernel's loads of
-// 2-byte elements wait.  us, lane-per-state and whole sequences, fp32: 5 rows per SM of 96 steps 5.0 and
-// 5.4, of 100 6.1 and 5.6; 10 of 224 steps 9.5 and 20.2, 22 of 64 steps 5.1 and 7.4; 30 of 40 steps
-// 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
-// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.
-bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
-    const int staged = (L + 31) / 32 * 32;
-    if (dt == VMB_BF16) return L >= 16;
-    if (rows <= 6LL * sms) return 16 * staged <= 17 * L;
-    if (rows <= 24LL * sms) return L >= 16;
-    return rows <= 48LL * sms && (L >= 64 || 8 * staged <= 9 * L);
-}
 
 // Estimated time (ns) of the warp-specialised kernel, and the number of chunks
 // it would take (1: one pass).  A CTA takes a fixed time per step that grows
 // with the CTAs that share an SM; cut into P + 1 chunks, P CTAs a tile run
 // concurrently and each passes over two chunks.  ns per step with one, two and
 // three CTAs per SM, measured on GB300 (fp32, 56x56 maps): 16 states, two lanes a
-// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8), two
-// lanes 41, 59, 72.  (bf16 takes the same numbers: its steps are up to 13% longer, alike
-// in every plan.)
-double ws_estimate(int np, bool two, long long tiles, int L, int sms, int ts, int* chunks) {
-    const double per_step[5][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {41, 59, 72}, {51, 79, 111}};
-    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 + two : 4];
+// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8).
+double ws_estimate(int np, long long tiles, int L, int sms, int ts, int* chunks) {
+    const double per_step[4][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {51, 79, 111}};
+    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 : 3];
     double best = 0.0;
     for (int P = 1; P <= 24; ++P) {
         if (P > 1 && L / (P + 1) < 4 * ts) break;
@@ -1807,16 +1775,13 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // kernel (small_rule).  Tensors that tensor copies can read, at least two
     // channel rows per SM -> the warp-specialised kernel: one lane per channel from
     // 256 rows per SM on, two lanes below (16 states, fp32, us: 24576 rows of 56x56
-    // 350 with two lanes, 471 with one; 49152 rows of 28x28 168 and 163; 8 states, by the
-    // estimate: 9728 rows of 64 steps 5.2 with two, 7.2 with one, the barrier-staged
-    // kernel 7.0, 19456 rows of 28x28 46 and 73, 30464 rows 81 and 77), L cut into
+    // 350 with two lanes, 471 with one; 49152 rows of 28x28 168 and 163), L cut into
     // chunks where ws_estimate expects a gain (6144 rows of 128x128 bf16 605, one
     // pass 1126, look-back chunks 870; 3072 rows of 56x56 80, look-back 187; one state, 131072 rows
     // of 56x56 779, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
     // the three-launch chunked variant while a grid of 64-step one-lane chunks
     // fits in two waves (768 rows of 56x56 30.2, chunked warp-specialised 34.8; at 1536
-    // rows 56.9 and 46.6), just past the short sequences (up to 320 steps) and up to 16 rows per SM
-    // the lane-per-state kernel (1520 rows of 288 steps 11.8, warp-specialised 17.0).  Other tensors: at least 256 rows per SM and L >= 128 ->
+    // rows 56.9 and 46.6).  Other tensors: at least 256 rows per SM and L >= 128 ->
     // the packed streaming kernel; otherwise plenty of rows -> one lane per
     // channel; a fair number -> two lanes; too few -> cut L into chunks: the
     // three-launch variant as above, else look-back chunks with one lane per
@@ -1861,29 +1826,16 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             n_chunks = (int)(want < mx ? want : mx);
         }
     } else if (const int G = np == 16 ? small_rule(a, map, seq_ok, sms) : 0) {
-        if (!map && seq_ok && G > 1 && lanes_beat_small(a.L, rows, a.dtype, sms)) {
-            shape = kLanesShape;
-            if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
-        } else {
-            shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
-        }
-    } else if (np == 16 && seq_ok && a.L > 256 && a.L <= 320 && rows <= 16LL * sms) {
-        shape = kLanesShape;
-        if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+        shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
     } else if (np == 16 && tma_ok && rows < 6LL * sms && chunk_grid_fits()) {
         shape = kChunkShape + 1;
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
     } else if (tma_ok && rows >= 2LL * sms) {
         const bool few = rows < 256LL * sms && (np < 16 || !small_map_one_lane(a.L));
-        auto estimate = [&](bool two, int* chunks) {
-            const KernelInfo k = pick(a.dtype, np, two ? ws_two_shape(np) : ws_shape(np), false);
-            return ws_estimate(np, two, a.B * a.K * (long long)((a.D + k.DT - 1) / k.DT), a.L, sms, k.ts, chunks);
-        };
-        int c1 = 1, c2 = 1;
-        const bool two = few && (np == 16 || (np == 8 && a.L >= 16 && estimate(true, &c2) <= estimate(false, &c1)));
-        shape = two ? ws_two_shape(np) : ws_shape(np);
+        shape = np == 16 && few ? kWsTwoShape : ws_shape(np);
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
-        if (few) estimate(two, &n_chunks);
+        if (few)
+            ws_estimate(np, a.B * a.K * (long long)((a.D + ki.DT - 1) / ki.DT), a.L, sms, ki.ts, &n_chunks);
     } else if (np == 16 && rows >= 256LL * sms && a.L >= 128) {
         // many rows: the packed streaming one-lane kernel, one pass over L (on
         // very short sequences its stage prologue does not pay off)
@@ -1924,7 +1876,6 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                 if (a.L / want_n >= 256) {
                     shape = r.chunk_narrow;
                     ki = kn;
-                    res = rn;
                     n_chunks = (int)want_n;
                 } else {
                     KernelInfo kw{};
@@ -1934,7 +1885,6 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                     const long long want_w = (rw + tiles_w - 1) / tiles_w, mx = (a.L + 127) / 128;
                     shape = r.chunk_wide;
                     ki = kw;
-                    res = rw;
                     n_chunks = (int)(want_w < mx ? want_w : mx);
                 }
             }
@@ -1970,20 +1920,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // idle for its whole life (measured on GB300, batch-32 56x56 map after the
     // map transpose: 514 us alone, about 900 us launched early); from a full
     // wave up the early launch is about 3% faster (batch-128 map)
-    // The barrier-staged kernels likewise (us, block from the map: 3 maps of 2x64x1536 bf16, rows
-    // out of line, 125 launched early, 49 not; 36 maps of 12x12x64 fp32, zero-order hold, 881 and
-    // 482; 2304 rows of 784 steps 2395 and 1414); sequences of less than 48 steps are over before
-    // their placement matters (16 with the zero-order hold), and start 0.3 to 0.5 us sooner early.
-    // The kernels of short sequences only in place, behind the kernel that filled y (9 maps of
-    // 10x4x172, low-rank Delta: 16.1 launched early).  Not the chunked three launches, whose CTAs
-    // are short.
-    const bool in_place = a.y == a.u || a.y == a.delta;
-    if (small_lanes(np, shape))
-        p.early = !in_place || a.L < 16;
-    else if (is_ws_shape(np, shape) ||
-             (!is_chunk_shape(np, shape) &&
-              (np == 16 && shape == kLanesShape && !zoh ? in_place && a.L >= 16 : a.L >= (zoh ? 16 : 48))))
-        p.early = (long long)p.n_seq * p.n_chunks >= res;
+    if (is_ws_shape(np, shape)) p.early = (long long)p.n_seq * p.n_chunks >= res;
     *plan = p;
     return VMB_OK;
 }
@@ -2034,12 +1971,12 @@ int full_plan_launches(const ScanPlan& plan) {
     return (is_chunk_shape(plan.np, plan.split) && plan.n_chunks > 1) ? 3 : 1;
 }
 
-vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream, bool* refused) {
+vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream) {
     const bool lowrank = a.R > 0;
     const bool ws_plan = is_ws_shape(plan.np, plan.split);
     if ((lowrank && !full_plan_lowrank(plan)) || (a.gather_h > 0 && !ws_plan)) return VMB_ERR_UNSUPPORTED;
     if (lowrank && a.gather_h > 0) return VMB_ERR_UNSUPPORTED;
-    if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream, plan.early);
+    if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream);
     KernelInfo ki = ws_plan ? ws_info(a.dtype, plan.np, ws_variant(plan.np, plan.split), a.gather_h > 0, a.R)
                             : pick(a.dtype, plan.np, plan.split, (a.flags & VMB_FLAG_B_ZOH) != 0);
     if (!ki.fn) return VMB_ERR_CUDA;
@@ -2112,12 +2049,11 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
             // launched early, behind a kernel that still holds shared memory, a CTA that
             // fills its share of the SM waits for it or lands elsewhere (128 maps of
             // 56x56x256 as the block: four slots 1966 us, five 2081)
-            // gathering, the kernel before is the transpose: one CTA per SM, beside which
-            // half of the grid runs, unless its planes are too large for that: launched early at any size in one pass (24576 rows
+            // gathering, the kernel before is the one-CTA-per-SM transpose, beside which
+            // half of the grid runs: launched early at any size in one pass (24576 rows
             // of 56x56: 436 us, 452 launched after it), but not chunked (6144 rows of
             // 128x128 bf16: 747, 705)
-            const bool beside = gather && plan.n_chunks == 1 &&
-                                transpose_by_planes(a.u, a.u_t, a.gather_h, a.L / a.gather_h, a.dtype);
+            const bool beside = gather && plan.n_chunks == 1;
             p.nstg = plan.early && !sub_wave ? kWsMinSlots
                                              : ws_slots(ki, ctas, device_sm_count(), beside ? kTransposeSmem : 0);
             const bool early = plan.early || beside;
@@ -2136,23 +2072,15 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
                        ? VMB_OK
                        : VMB_ERR_CUDA;
         }
-        // the encoder refused the tensors: nothing is launched here; a scan of materialised
-        // sequences takes the plan of tensors that tensor copies cannot read, the other forms
-        // are the caller's
-        if (refused) *refused = true;
-        if (gather || lowrank) return VMB_ERR_UNSUPPORTED;
-        ScanArgs m = a;
-        m.no_tma = true;
-        ScanPlan mplan{};
-        const vmb_status st = plan_full(m, &mplan);
-        if (st != VMB_OK) return st;
-        if (is_ws_shape(mplan.np, mplan.split)) return VMB_ERR_UNSUPPORTED;
-        if (a.ws_bytes < mplan.ws_bytes) return VMB_ERR_WORKSPACE;
-        return launch_full(m, mplan, stream);
+        // the encoder refused the tensors: the packed streaming variant (same tiles, same
+        // results), which reads materialised sequences only (no fallback of the other variants)
+        if (gather || lowrank || plan.np != 16 || ws_variant(plan.np, plan.split) == kWsTwoLanes)
+            return VMB_ERR_UNSUPPORTED;
+        ki = pick(a.dtype, plan.np, kPackedShape, false);
+        if (!ki.fn) return VMB_ERR_CUDA;
     }
-    return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream, plan.early) == cudaSuccess
-               ? VMB_OK
-               : VMB_ERR_CUDA;
+    return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream) == cudaSuccess ? VMB_OK
+                                                                                                   : VMB_ERR_CUDA;
 }
 
 }  // namespace vmb

@@ -33,6 +33,20 @@ constexpr int kSmThreads = 128;  // four warps
 constexpr int kNP = 16;          // states, zero padded
 constexpr int kBC = 2 * kNP;     // floats of one step's B and C
 
+// Division by an invariant integer by multiply-high (Granlund & Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994), for
+// dividends below 2^31.
+struct FastDiv {
+    unsigned d, m, s;
+};
+FastDiv make_fastdiv(unsigned d) {
+    unsigned s = 0;
+    while ((1ull << s) < d) ++s;
+    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
+    return {d, (unsigned)m, s};
+}
+__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
+
 struct SmallParams {
     const void* u;  // [B][K][D][L], or (MAP) the map x [B][D][L]
     const void* dl;
@@ -52,7 +66,10 @@ struct SmallParams {
     FastDiv fL, fW;
 };
 
-__device__ __forceinline__ void load_elem(float* dst, const float* src) { cp_async4(dst, src, 4); }
+__device__ __forceinline__ void load_elem(float* dst, const float* src) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(src) : "memory");
+}
 __device__ __forceinline__ void load_elem(float* dst, const __nv_bfloat16* src) { *dst = __bfloat162float(*src); }
 
 // `rows` consecutive rows of L elements into rows of stride RX, by `step`
@@ -67,7 +84,7 @@ __device__ __forceinline__ void load_rows(float* dst, const T* src, int rows, co
     }
 }
 
-// Word of column q (B: q = 0..15, C: 16 + the same) at step t: the columns of a
+// Word of state column q (B: q = n, C: q = 16 + n) at step t: the columns of a
 // step are rotated by four per step, so that the stores of one column at
 // consecutive steps spread over eight banks; a quad of columns stays contiguous.
 __device__ __forceinline__ int bc_word(int t, int q) { return t * kBC + ((q + 4 * t) & (kBC - 1)); }
@@ -120,13 +137,11 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     if (p.N < kNP)
         for (int i = lane; i < L * kBC; i += 32) bc[i] = 0.0f;
     __syncwarp();
-    // lane g owns the states g, g + G, ...: their columns lie together
 #pragma unroll 4
     for (int i = lane; i < p.N * L; i += 32) {
         const int n = (int)fdiv((unsigned)i, p.fL), t = i - n * L;
-        const int q = G == 4 ? (n & 3) * 4 + (n >> 2) : n;
-        load_elem(bc + bc_word(t, q), Bs + i);
-        load_elem(bc + bc_word(t, kNP + q), Cs + i);
+        load_elem(bc + bc_word(t, n), Bs + i);
+        load_elem(bc + bc_word(t, kNP + n), Cs + i);
     }
     cp_async_commit();
     const int c = lane / G, g = lane % G;
@@ -137,7 +152,7 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     float A2[NG], h[NG];
 #pragma unroll
     for (int i = 0; i < NG; ++i) {
-        const int n = g + i * G;
+        const int n = g * NG + i;
         A2[i] = (cval && n < p.N) ? __ldg(p.A + ((size_t)k * p.D + d) * p.N + n) * kLog2e : 0.0f;
         h[i] = 0.0f;
     }
@@ -183,12 +198,8 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
                 h[0] = fmaf(ex2(dv * A2[0]), h[0], du * b);
                 yp[j] = cc * h[0];
             } else {
-                // sum over the states: one chain, as in the other kernels with one lane
-                // a channel, or (G = 4) the first two levels of the tree over the 16
-                // states that the lane-per-state kernels add across lanes (scalar additions,
-                // with which the products are not fused)
                 const float2 dd = make_float2(dv, dv), uu = make_float2(du, du);
-                float2 ya = make_float2(0.0f, 0.0f), half = ya;
+                float2 ya = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int q = 0; q < NG / 4; ++q) {
                     const float4 b = *reinterpret_cast<const float4*>(bc + bc_word(t, g * NG + 4 * q));
@@ -203,12 +214,7 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
                                                      __fmul2_rn(uu, b2[e]));
                         h[n] = hn.x;
                         h[n + 1] = hn.y;
-                        if constexpr (G == 1) ya = __ffma2_rn(c2[e], hn, ya);
-                        else if (e == 0) half = __fmul2_rn(c2[0], hn);
-                        else {
-                            const float2 p1 = __fmul2_rn(c2[1], hn);
-                            ya = make_float2(__fadd_rn(half.x, p1.x), __fadd_rn(half.y, p1.y));
-                        }
+                        ya = __ffma2_rn(c2[e], hn, ya);
                     }
                 }
                 yp[j] = ya.x + ya.y;
@@ -282,7 +288,7 @@ size_t small_scan_smem(int G, int L, bool map) {
     return (((map ? 5 : 8) * ct * rx + 3) / 4 * 4 + (size_t)4 * L * kBC) * 4;
 }
 
-vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early) {
+vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream) {
     const bool map = out != nullptr;
     const void* fn = a.dtype == VMB_BF16 ? (map ? small_pick<__nv_bfloat16, true>(G) : small_pick<__nv_bfloat16, false>(G))
                                          : (map ? small_pick<float, true>(G) : small_pick<float, false>(G));
@@ -311,7 +317,7 @@ vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaS
     p.fW = make_fastdiv((unsigned)(W > 0 ? W : 1));
     const long long grid = map ? p.units : (p.units + 3) / 4;
     void* args[] = {&p};
-    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSmThreads), small_scan_smem(G, a.L, map), args, stream, early) ==
+    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSmThreads), small_scan_smem(G, a.L, map), args, stream) ==
                    cudaSuccess
                ? VMB_OK
                : VMB_ERR_CUDA;

@@ -35,7 +35,7 @@ struct ScanArgs {
     float* saved = nullptr;  // mean path: the group means kept for the backward, [B*K][N + 1][L] fp32
     const float* Wup = nullptr;  // full path, low-rank Delta: delta is z [B*K][R][L] fp32 and
     int R = 0;                   // delta_raw = Wup z (Wup [K][D][R]); warp-specialised plans only
-    bool no_tma = false;         // full path: plan as for tensors that tensor copies cannot read
+    bool no_tma = false;         // full path, workspace query: plan as for tensors that tensor copies cannot read
 };
 
 // Execution plan of an L-chunked scan: how the (sequence, chunk) grid is cut
@@ -163,15 +163,10 @@ vmb_status validate_scan(const ScanArgs& a, bool mean, bool* empty);
 // Test-only plan overrides (vmb_testing.h); -1 / 0 when unset.
 int forced_full_shape(int* chunks);
 int forced_mean_chunk();
-int forced_mean_steps();
-bool refuse_tensor_maps();
 
 vmb_status plan_full(const ScanArgs& a, ScanPlan* plan);
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan);
-// (*refused: the driver's tensor-map encoder refused the tensors of a warp-specialised plan.  A
-// scan of materialised sequences has then been launched with another plan; one that gathers or
-// expands has not been, and its tensors have to be materialised, ScanArgs::no_tma.)
-vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream, bool* refused = nullptr);
+vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
 int full_plan_launches(const ScanPlan& plan);  // kernels launch_full starts for this plan
 // Whether launch_full can read the plan's u gathered from the map (ScanArgs::gather_h):
 // the warp-specialised plans; or expand a low-rank Delta (ScanArgs::R): those of 16 states.
@@ -186,27 +181,17 @@ int full_plan_small(const ScanPlan& plan);
 constexpr size_t kSmallMaxSmem = 227 * 1024;
 size_t small_scan_smem(int G, int L, bool map);
 // out = null: the scan alone (a.u the sequences); else a.u is the map [B][D][H][W] and K = 4.
-vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early = true);
+vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream);
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
-bool mean_two_steps(long long n, int D, long long res1, long long res2, int sms, bool with_y);
-// Kernels of the cross-scan and the cross-merge; `aligned`: both tensors 16-byte aligned.
-enum class CsmKernel { kPlane, kBand, kGather };
-CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, bool aligned, int sms);
 vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W, vmb_dtype dt,
                              cudaStream_t stream);
 vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, int W, vmb_dtype dt,
                               cudaStream_t stream);
-// The transpose by whole planes (transpose_by_planes: they fit) runs as one CTA per SM of at
-// most this shared memory (1 KB of the CTA's own included), beside which the scan starts;
-// otherwise 32 x 32 tiles.
+// The transpose runs as one CTA per SM of at most this shared memory (1 KB of the CTA's own included).
 constexpr size_t kTransposeSmem = 33 * 1024;
-bool transpose_by_planes(const void* x, const void* xt, int H, int W, vmb_dtype dt);
-vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, bool planes,
+vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt,
                                 cudaStream_t stream);
-// Whether the channel-mean scan of this plan runs beside the transpose by planes.
-bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W);
 vmb_status launch_discretise(const DiscArgs& a, bool mean, cudaStream_t stream);
-bool selection_two_buffers(long long grid, int D, int sms);
 vmb_status launch_selection(const SelArgs& a, cudaStream_t stream);
 size_t mean_bwd_workspace_bytes(long long B, long long K, long long D, long long N, long long L, long long G);
 vmb_status launch_mean_bwd(const MeanBwdArgs& a, cudaStream_t stream);
