@@ -1496,13 +1496,17 @@ KernelInfo info_for() {
 template <typename T, bool ZOH>
 KernelInfo lanes_info() {
     using LY = Layout<T, 16, LanesShape>;
+    // at most three CTAs per SM: with a fourth, grids of two to three per SM, launched behind
+    // a kernel that still runs, stack on the SMs freed first (14 sequences of 512 channels, 48 steps,
+    // bf16: 6.1 us with three, 8.8 with four)
+    constexpr size_t kSmem = LY::raw_bytes > 58 * 1024 ? LY::raw_bytes : 58 * 1024;
     const void* fn = reinterpret_cast<const void*>(&full_scan_lanes_kernel<T, ZOH>);
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::raw_bytes);
+        attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     });
-    return {attr_err == cudaSuccess ? fn : nullptr, LY::raw_bytes, 16, LY::DT, 256, LY::TS};
+    return {attr_err == cudaSuccess ? fn : nullptr, kSmem, 16, LY::DT, 256, LY::TS};
 }
 
 template <typename T, class CS>
@@ -1718,8 +1722,9 @@ ShapeRoles roles(int np) {
 // One lane, the warp-specialised and the packed streaming kernel share their
 // arithmetic, so the block is bit-identical to the separate calls either way
 // (where the block may take one lane the scan alone keeps to one lane and one
-// pass, so the rule for both goes by the tensors of the scan alone: `seq_ok`); 4 and 16
-// lanes (other sums over the states) are taken by both or by neither.
+// pass, so the rule for both goes by the tensors of the scan alone: `seq_ok`); 4 and
+// 16 lanes sum over the states in the order of the lane-per-state kernel, which the
+// scan alone takes instead where it is faster (lanes_beat_small).
 bool small_map_one_lane(int L) { return 2 * (small_scan_smem(1, L, true) + 1024) <= kSmemPerSm; }
 int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (a.L > 256) return 0;
@@ -1732,6 +1737,20 @@ int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (small_scan_smem(1, a.L, false) > kSmallMaxSmem) return 0;
     if (!seq_ok) return 1;
     return map && small_map_one_lane(a.L) ? 1 : 0;
+}
+// Short sequences alone, in rows that the barrier-staged kernels copy 16 bytes at a time: the
+// lane-per-state kernel instead of 4 or 16 lanes of whole sequences.  It streams stages of 32
+// steps, so a length just past one pays for the next; the whole-sequence kernel's loads of
+// 2-byte elements wait.  us, lane-per-state and whole sequences, fp32: 5 rows per SM of 96 steps 5.0 and
+// 5.4, of 100 6.1 and 5.6; 10 of 224 steps 9.5 and 20.2, 22 of 64 steps 5.1 and 7.4; 30 of 40 steps
+// 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
+// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.
+bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
+    const int staged = (L + 31) / 32 * 32;
+    if (dt == VMB_BF16) return L >= 16;
+    if (rows <= 6LL * sms) return 16 * staged <= 17 * L;
+    if (rows <= 24LL * sms) return L >= 16;
+    return rows <= 48LL * sms && (L >= 64 || 8 * staged <= 9 * L);
 }
 
 // Estimated time (ns) of the warp-specialised kernel, and the number of chunks
@@ -1781,7 +1800,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // of 56x56 779, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
     // the three-launch chunked variant while a grid of 64-step one-lane chunks
     // fits in two waves (768 rows of 56x56 30.2, chunked warp-specialised 34.8; at 1536
-    // rows 56.9 and 46.6).  Other tensors: at least 256 rows per SM and L >= 128 ->
+    // rows 56.9 and 46.6), just past the short sequences (up to 320 steps) and up to 16 rows per SM
+    // the lane-per-state kernel (1520 rows of 288 steps 11.8, warp-specialised 17.0).  Other tensors: at least 256 rows per SM and L >= 128 ->
     // the packed streaming kernel; otherwise plenty of rows -> one lane per
     // channel; a fair number -> two lanes; too few -> cut L into chunks: the
     // three-launch variant as above, else look-back chunks with one lane per
@@ -1826,7 +1846,15 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             n_chunks = (int)(want < mx ? want : mx);
         }
     } else if (const int G = np == 16 ? small_rule(a, map, seq_ok, sms) : 0) {
-        shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
+        if (!map && seq_ok && G > 1 && lanes_beat_small(a.L, rows, a.dtype, sms)) {
+            shape = kLanesShape;
+            if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+        } else {
+            shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
+        }
+    } else if (np == 16 && seq_ok && a.L > 256 && a.L <= 320 && rows <= 16LL * sms) {
+        shape = kLanesShape;
+        if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
     } else if (np == 16 && tma_ok && rows < 6LL * sms && chunk_grid_fits()) {
         shape = kChunkShape + 1;
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;

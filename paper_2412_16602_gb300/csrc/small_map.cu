@@ -84,7 +84,7 @@ __device__ __forceinline__ void load_rows(float* dst, const T* src, int rows, co
     }
 }
 
-// Word of state column q (B: q = n, C: q = 16 + n) at step t: the columns of a
+// Word of column q (B: q = 0..15, C: 16 + the same) at step t: the columns of a
 // step are rotated by four per step, so that the stores of one column at
 // consecutive steps spread over eight banks; a quad of columns stays contiguous.
 __device__ __forceinline__ int bc_word(int t, int q) { return t * kBC + ((q + 4 * t) & (kBC - 1)); }
@@ -137,11 +137,13 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     if (p.N < kNP)
         for (int i = lane; i < L * kBC; i += 32) bc[i] = 0.0f;
     __syncwarp();
+    // lane g owns the states g, g + G, ...: their columns lie together
 #pragma unroll 4
     for (int i = lane; i < p.N * L; i += 32) {
         const int n = (int)fdiv((unsigned)i, p.fL), t = i - n * L;
-        load_elem(bc + bc_word(t, n), Bs + i);
-        load_elem(bc + bc_word(t, kNP + n), Cs + i);
+        const int q = G == 4 ? (n & 3) * 4 + (n >> 2) : n;
+        load_elem(bc + bc_word(t, q), Bs + i);
+        load_elem(bc + bc_word(t, kNP + q), Cs + i);
     }
     cp_async_commit();
     const int c = lane / G, g = lane % G;
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
     float A2[NG], h[NG];
 #pragma unroll
     for (int i = 0; i < NG; ++i) {
-        const int n = g * NG + i;
+        const int n = g + i * G;
         A2[i] = (cval && n < p.N) ? __ldg(p.A + ((size_t)k * p.D + d) * p.N + n) * kLog2e : 0.0f;
         h[i] = 0.0f;
     }
@@ -198,8 +200,12 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
                 h[0] = fmaf(ex2(dv * A2[0]), h[0], du * b);
                 yp[j] = cc * h[0];
             } else {
+                // sum over the states: one chain, as in the other kernels with one lane
+                // a channel, or (G = 4) the first two levels of the tree over the 16
+                // states that the lane-per-state kernels add across lanes (scalar additions,
+                // with which the products are not fused)
                 const float2 dd = make_float2(dv, dv), uu = make_float2(du, du);
-                float2 ya = make_float2(0.0f, 0.0f);
+                float2 ya = make_float2(0.0f, 0.0f), half = ya;
 #pragma unroll
                 for (int q = 0; q < NG / 4; ++q) {
                     const float4 b = *reinterpret_cast<const float4*>(bc + bc_word(t, g * NG + 4 * q));
@@ -214,7 +220,12 @@ __global__ void __launch_bounds__(kSmThreads) small_scan_kernel(const SmallParam
                                                      __fmul2_rn(uu, b2[e]));
                         h[n] = hn.x;
                         h[n + 1] = hn.y;
-                        ya = __ffma2_rn(c2[e], hn, ya);
+                        if constexpr (G == 1) ya = __ffma2_rn(c2[e], hn, ya);
+                        else if (e == 0) half = __fmul2_rn(c2[0], hn);
+                        else {
+                            const float2 p1 = __fmul2_rn(c2[1], hn);
+                            ya = make_float2(__fadd_rn(half.x, p1.x), __fadd_rn(half.y, p1.y));
+                        }
                     }
                 }
                 yp[j] = ya.x + ya.y;

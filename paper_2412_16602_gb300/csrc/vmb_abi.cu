@@ -673,6 +673,35 @@ const char* vmb_status_string(vmb_status s) {
 
 int vmb_version(void) { return 100; }
 
+int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
+                          int* out) {
+    ScanArgs a{};
+    a.B = B;
+    a.K = K;
+    a.D = D;
+    a.N = N;
+    a.L = H * W;
+    a.flags = flags;
+    a.dtype = dtype;
+    alignas(16) static const float dummy[8] = {};
+    const char* base = reinterpret_cast<const char*>(dummy);
+    a.u = base + (off & 1 ? esize(dtype) : 0);
+    a.delta = base + (off & 2 ? esize(dtype) : 0);
+    a.Bs = a.Cs = dummy;
+    a.A = a.Dskip = a.bias = dummy;
+    a.y = const_cast<float*>(dummy + 4);  // not in place
+    if (map) {
+        a.gather_h = H;
+        a.u_t = dummy;
+    }
+    ScanPlan plan{};
+    const vmb_status s = plan_full(a, &plan);
+    out[0] = plan.split;
+    out[1] = plan.n_chunks;
+    out[2] = plan.early ? 1 : 0;
+    return s;
+}
+
 int vmb_testing_force_full_plan(int shape, int chunks) {
     g_force_chunks.store(chunks, std::memory_order_relaxed);
     g_force_shape.store(shape < 0 ? -1 : shape, std::memory_order_relaxed);

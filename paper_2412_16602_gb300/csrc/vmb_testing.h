@@ -16,6 +16,12 @@
 extern "C" {
 #endif
 
+/* What the planner answers, without a launch: out = {tile shape, L-chunks, launched
+ * early} of a full scan (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or
+ * delta (off & 2) one element past 16-byte alignment.  Returns the status. */
+int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
+                          int* out);
+
 /* Force the full scan's tile shape (0..23 for 16 states; taken modulo the
  * number of shapes of the padded state count) and, for the look-back and
  * warp-specialised shapes, the number of L-chunks (<= 1: one chunk).  shape < 0 restores the planner.

@@ -14,6 +14,27 @@ def pytest_configure(config):
 
 
 @pytest.fixture
+def full_plan():
+    """(tile shape, L-chunks, launched early) that the planner picks for a full scan
+    (needs a GPU); `off`: u or x (1), delta (2) one element past 16-byte alignment."""
+    import ctypes
+
+    import paper_2412_16602_gb300 as vmb
+
+    i = ctypes.c_int
+    vmb.lib.vmb_testing_full_plan.argtypes = [i] * 6 + [ctypes.c_uint, i, i, i, ctypes.c_void_p]
+
+    def plan(B, K, D, N, H, W, dt, map=False, off=0, flags=vmb.VMB_FLAG_SOFTPLUS):
+        out = (i * 3)()
+        s = vmb.lib.vmb_testing_full_plan(B, K, D, N, H, W, flags, vmb.VMB_F32 if dt == "f32" else vmb.VMB_BF16, int(map),
+                                          off, out)
+        assert s == vmb.VMB_OK
+        return tuple(out)
+
+    return plan
+
+
+@pytest.fixture
 def force_plan():
     """Force a tile shape / chunk count of the full scan ("shape[,chunks]") or a
     chunk length of the channel-mean scan through libvmb's test-only controls

@@ -54,6 +54,44 @@ def test_short_sequences(shape, plan, force_plan):
     check(to_numpy(out), out_ref, dt, "full out from the map")
 
 
+@pytest.mark.parametrize("shape", [s for s in SHAPES if s[3] * s[4] > 1], ids=lambda s: "B{}_D{}_N{}_{}x{}_{}".format(*s))
+def test_whole_sequences_and_lane_per_state_agree_bit_for_bit(shape, force_plan):
+    """4 and 16 lanes of whole sequences (the block) add the states in the order of the
+    lane-per-state kernel (shape 7), which the scan alone may take instead."""
+    B, D, N, H, W, dt = shape
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=310 + D)
+    g = to_device(workloads.make_inputs(wl, params="random"), DEV)
+    args = (vmb.vmb_cross_scan(g["x"]), g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W)
+    ys = []
+    for plan in ("7", "21", "22"):
+        force_plan.full(plan)
+        ys.append(vmb.vmb_selective_scan_fwd(*args))
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
+
+
+LANES, FOUR, SIXTEEN = 7, 21, 22
+
+
+@pytest.mark.parametrize("case,map_shape,scan_shape", [
+    # (B, D, H, W, dtype): rows per SM from 2 to 50
+    ((2, 32, 8, 8, "f32"), SIXTEEN, LANES), ((12, 32, 14, 16, "f32"), FOUR, LANES), ((19, 32, 4, 56, "bf16"), FOUR, LANES),
+    ((2, 32, 2, 4, "f32"), SIXTEEN, SIXTEEN), ((36, 32, 5, 8, "f32"), FOUR, FOUR), ((36, 32, 8, 12, "f32"), FOUR, LANES),
+    ((1, 40, 10, 10, "f32"), SIXTEEN, SIXTEEN), ((3, 64, 16, 18, "f32"), LANES, LANES),
+    ((30, 64, 16, 18, "f32"), 23, 23), ((60, 32, 8, 12, "f32"), FOUR, FOUR), ((60, 32, 8, 10, "bf16"), FOUR, LANES),
+])
+def test_planner_of_short_sequences(case, map_shape, scan_shape, full_plan):
+    B, D, H, W, dt = case
+    assert full_plan(B, 4, D, 16, H, W, dt, map=True)[0] == map_shape
+    assert full_plan(B, 4, D, 16, H, W, dt)[0] == scan_shape
+    wl = workloads.small_case(B=B, D=D, N=16, H=H, W=W, dtype=dt, seed=B)
+    g = workloads.make_device_inputs(wl, DEV, seed=B, params="random")
+    args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+    out, y = vmb.vmb_ss2d_full_fwd(g["x"], *args)
+    y2 = vmb.vmb_selective_scan_fwd(vmb.vmb_cross_scan(g["x"]), *args, H, W)
+    assert torch.equal(y, y2) and torch.equal(out, vmb.vmb_cross_merge(y2, H, W))
+
+
 @pytest.mark.parametrize("case", [(8, 512, 10, 12, "f32"), (8, 512, 8, 13, "bf16"), (3, 700, 9, 12, "f32"),
                                   (8, 512, 8, 8, "f32"), (2, 40, 10, 12, "f32"), (8, 256, 12, 12, "f32"), (2, 64, 28, 28, "f32"),
                                   (1, 40, 40, 42, "bf16")],
