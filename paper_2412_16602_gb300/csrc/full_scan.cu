@@ -79,10 +79,65 @@ __device__ __forceinline__ float sel4(const float (&v)[4], int j) {
     return j == 0 ? v[0] : j == 1 ? v[1] : j == 2 ? v[2] : v[3];
 }
 
+// load_tile for rows that are not 16-byte aligned.
+template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B>
+__device__ __forceinline__ void load_tile_elements(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
+                                                   int l0) {
+    // element by element: thread i copies step i % kTS of rows i / kTS + k RPP, u and
+    // delta (B and C) together; fp32 as 4-byte asynchronous copies, in flight like
+    // the 16-byte ones, bf16 (2-byte elements) through registers, a batch of
+    // independent loads at a time.  Only rows of the problem are visited: rows of u
+    // and delta past nrows keep what they held (the lanes that read them store
+    // nothing), those of B and C past N are zeroed (GB300, bf16, unaligned rows, us:
+    // 21 maps of 38x51x3, two states, 243 visiting every row of the tile, see the
+    // test of narrow tiles).
+    constexpr int RPP = kThreads / kTS;
+    static_assert(kThreads % kTS == 0, "tile loader mapping");
+    const int t = threadIdx.x % kTS, r0 = threadIdx.x / kTS;
+    const bool colok = l0 + t < p.L;
+    // `n` rows, of which the first `valid` come from src
+    auto rows = [&](T* to, const void* src, size_t first, int valid, int n) {
+        const T* g = static_cast<const T*>(src) + (first + r0) * p.L + (colok ? l0 + t : 0);
+        const size_t step = (size_t)RPP * p.L;
+        to += r0 * RS + t;
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll 2
+            for (int r = r0; r < n; r += RPP, g += step, to += RPP * RS) {
+                const bool ok = colok && r < valid;
+                cp_async4(to, ok ? g : src, ok ? 4 : 0);
+            }
+        } else {
+            constexpr int kBatch = 8;
+#pragma unroll 1
+            for (int r = r0; r < n; r += kBatch * RPP) {
+                T v[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q, g += step) v[q] = colok && r + q * RPP < valid ? *g : T(0.0f);
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q, to += RPP * RS)
+                    if (r + q * RPP < n) *to = v[q];
+            }
+        }
+    };
+    rows(dst, p.u, row0, nrows, nrows);
+    rows(dst + DT * RS, p.dl, row0, nrows, nrows);
+    if constexpr (WITH_B) {
+        rows(dst + 2 * DT * RS, p.Bs, bcrow0, p.N, NP);
+        if constexpr (WITH_C) rows(dst + (2 * DT + NP) * RS, p.Cs, bcrow0, p.N, NP);
+    }
+}
+
+// The same as a function of its own, for the kernels whose registers are all taken.
+template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B>
+__device__ __noinline__ void load_tile_elements_call(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
+                                                     int l0) {
+    load_tile_elements<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
+}
+
 // Copy kTS steps (from l0) of DT u and delta rows and of the NP B (and C) rows
 // into shared memory rows of stride RS: u at row 0, delta at row DT, B at 2 DT,
-// C at 2 DT + NP.  Rows and steps past the problem are zero-filled.
-template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B = true>
+// C at 2 DT + NP.  Steps past the problem and rows of B and C past N are zero-filled.
+template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B = true, bool CALL = false>
 __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
                                           int l0) {
     constexpr int VE = 16 / sizeof(T);  // elements per 16-byte chunk
@@ -124,53 +179,10 @@ __device__ __forceinline__ void load_tile(const FullParams& p, T* dst, size_t ro
             }
         }
     } else {
-        // element by element: fp32 as 4-byte asynchronous copies, in flight like the
-        // 16-byte ones; bf16 (2-byte elements) through registers, a batch of
-        // independent loads at a time
-        constexpr int nU = DT * kTS, nB = NP * kTS;
-        constexpr int total = 2 * nU + (WITH_B ? (WITH_C ? 2 : 1) * nB : 0);
-        auto locate = [&](int i, const T** src, int* at) -> bool {  // source, offset in dst; false: zero
-            if (i < 2 * nU) {
-                const int j = i < nU ? i : i - nU;
-                const int r = j / kTS, t = j % kTS;
-                *at = (i < nU ? 0 : DT * RS) + r * RS + t;
-                *src = (i < nU ? u : dl) + (row0 + r) * (size_t)L + l0 + t;
-                return r < nrows && l0 + t < L;
-            }
-            const int i2 = i - 2 * nU;
-            const int j = i2 < nB ? i2 : i2 - nB;
-            const int r = j / kTS, t = j % kTS;
-            *at = 2 * DT * RS + (i2 < nB ? 0 : NP * RS) + r * RS + t;
-            *src = (i2 < nB ? Bs : Cs) + (bcrow0 + r) * (size_t)L + l0 + t;
-            return r < p.N && l0 + t < L;
-        };
-        if constexpr (sizeof(T) == 4) {
-            for (int i = threadIdx.x; i < total; i += kThreads) {
-                const T* src;
-                int at;
-                const bool ok = locate(i, &src, &at);
-                cp_async4(dst + at, ok ? src : u, ok ? 4 : 0);
-            }
-        } else {
-            constexpr int kBatch = 8;
-            for (int i0 = threadIdx.x; i0 < total; i0 += kBatch * kThreads) {
-                T v[kBatch];
-                int at[kBatch];
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q) {
-                    const int i = i0 + q * kThreads;
-                    v[q] = T(0.0f);
-                    at[q] = -1;
-                    if (i < total) {
-                        const T* src;
-                        if (locate(i, &src, &at[q])) v[q] = *src;
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q)
-                    if (at[q] >= 0) dst[at[q]] = v[q];
-            }
-        }
+        if constexpr (CALL)
+            load_tile_elements_call<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
+        else
+            load_tile_elements<T, NP, DT, kTS, RS, kThreads, WITH_C, WITH_B>(p, dst, row0, bcrow0, nrows, l0);
     }
 }
 
@@ -1287,7 +1299,7 @@ __global__ void __launch_bounds__(PackedLayout<T, PS>::THREADS, PS::MINB) full_p
     const int nst = (L + TS - 1) / TS;
 #pragma unroll
     for (int q = 0; q < NSTG - 1; ++q) {
-        if (q < nst) load_tile<T, NP, DT, TS, RS, THREADS, true>(p, raw + q * SLOT, row0, bcrow0, nrows, q * TS);
+        if (q < nst) load_tile<T, NP, DT, TS, RS, THREADS, true, true, true>(p, raw + q * SLOT, row0, bcrow0, nrows, q * TS);
         cp_async_commit();
     }
     const float bias = cval ? p.bias[(size_t)k * p.D + d] : 0.0f;
@@ -1335,7 +1347,7 @@ __global__ void __launch_bounds__(PackedLayout<T, PS>::THREADS, PS::MINB) full_p
         cp_async_wait<NSTG - 3>();  // stages <= s+1 have landed
         __syncthreads();            // ... for every thread; stage s is prepared
         if (s + NSTG - 1 < nst)
-            load_tile<T, NP, DT, TS, RS, THREADS, true>(p, raw + ((s + NSTG - 1) % NSTG) * SLOT, row0, bcrow0, nrows,
+            load_tile<T, NP, DT, TS, RS, THREADS, true, true, true>(p, raw + ((s + NSTG - 1) % NSTG) * SLOT, row0, bcrow0, nrows,
                                                         l0 + (NSTG - 1) * TS);
         cp_async_commit();
         if (s + 1 < nst) prepare(s + 1);

@@ -79,3 +79,37 @@ def test_workspace_of_the_query_serves_any_alignment(N):
         y = vmb.vmb_selective_scan_fwd(u, g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W, workspace=ws)
         assert vmb.vmb_read_status(ws) == vmb.VMB_OK
         check(to_numpy(y), y_ref, "f32", f"full y, shifted by {shift}")
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("case", [
+    # (B, K, D, N, L, dtype): narrow tiles, whole tiles and one row more, stages cut short
+    (2, 4, 3, 2, 67, "bf16"), (1, 4, 3, 8, 67, "f32"), (1, 2, 129, 1, 51, "bf16"), (1, 2, 129, 4, 51, "f32"),
+    (2, 4, 35, 9, 301, "bf16"), (1, 4, 16, 16, 1201, "f32"), (1, 2, 65, 16, 1201, "bf16"), (3, 4, 17, 5, 130, "bf16"),
+], ids=lambda c: "B{}_K{}_D{}_N{}_L{}_{}".format(*c))
+def test_rows_out_of_line(case, off):
+    """Rows that are not 16-byte aligned, by length (off 0) or also by address (off 1),
+    in every barrier-staged plan that the planner takes for them: against the oracle."""
+    B, K, D, N, L, dt = case
+    gen = torch.Generator().manual_seed(L + D)
+    td = torch.float32 if dt == "f32" else torch.bfloat16
+    u, delta = (torch.randn(B, K, D, L, generator=gen).to(td) for _ in range(2))
+    Bs, Cs = (torch.randn(B, K, N, L, generator=gen).to(td) for _ in range(2))
+    A = -(torch.arange(N) + 1.0) * (0.8 + 0.4 * torch.rand(K * D, N, generator=gen))
+    dsk, bias = 0.75 + 0.5 * torch.rand(K * D, generator=gen), torch.randn(K * D, generator=gen) * 0.3 - 3.0
+
+    def put(t):
+        buf = torch.empty(t.numel() + off, dtype=t.dtype, device=DEV)[off:]
+        return buf.view(t.shape).copy_(t)
+
+    y = vmb.vmb_selective_scan_fwd(put(u), put(delta), A.to(DEV), put(Bs), put(Cs), dsk.to(DEV), bias.to(DEV), 1, L)
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    # Eqs. 3, 4 and 6 in fp64
+    d = torch.nn.functional.softplus(delta.double() + bias.double().view(1, K, D, 1))
+    h = torch.zeros(B, K, D, N, dtype=torch.float64)
+    ref = torch.empty(B, K, D, L, dtype=torch.float64)
+    a64 = A.double().view(1, K, D, N)
+    for t in range(L):
+        h = torch.exp(d[..., t, None] * a64) * h + (d[..., t] * u[..., t].double())[..., None] * Bs.double()[:, :, None, :, t]
+        ref[..., t] = (h * Cs.double()[:, :, None, :, t]).sum(-1) + dsk.double().view(1, K, D) * u[..., t].double()
+    check(to_numpy(y), ref.numpy(), dt, "y of rows out of line")
