@@ -1916,6 +1916,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                 if (a.L / want_n >= 256) {
                     shape = r.chunk_narrow;
                     ki = kn;
+                    res = rn;
                     n_chunks = (int)want_n;
                 } else {
                     KernelInfo kw{};
@@ -1925,6 +1926,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
                     const long long want_w = (rw + tiles_w - 1) / tiles_w, mx = (a.L + 127) / 128;
                     shape = r.chunk_wide;
                     ki = kw;
+                    res = rw;
                     n_chunks = (int)(want_w < mx ? want_w : mx);
                 }
             }
@@ -1960,7 +1962,20 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // idle for its whole life (measured on GB300, batch-32 56x56 map after the
     // map transpose: 514 us alone, about 900 us launched early); from a full
     // wave up the early launch is about 3% faster (batch-128 map)
-    if (is_ws_shape(np, shape)) p.early = (long long)p.n_seq * p.n_chunks >= res;
+    // The barrier-staged kernels likewise (us, block from the map: 3 maps of 2x64x1536 bf16, rows
+    // out of line, 125 launched early, 49 not; 36 maps of 12x12x64 fp32, zero-order hold, 881 and
+    // 482; 2304 rows of 784 steps 2395 and 1414); sequences of less than 48 steps are over before
+    // their placement matters (16 with the zero-order hold), and start 0.3 to 0.5 us sooner early.
+    // The kernels of short sequences only in place, behind the kernel that filled y (9 maps of
+    // 10x4x172, low-rank Delta: 16.1 launched early).  Not the chunked three launches, whose CTAs
+    // are short.
+    const bool in_place = a.y == a.u || a.y == a.delta;
+    if (small_lanes(np, shape))
+        p.early = !in_place || a.L < 16;
+    else if (is_ws_shape(np, shape) ||
+             (!is_chunk_shape(np, shape) &&
+              (np == 16 && shape == kLanesShape && !zoh ? in_place && a.L >= 16 : a.L >= (zoh ? 16 : 48))))
+        p.early = (long long)p.n_seq * p.n_chunks >= res;
     *plan = p;
     return VMB_OK;
 }
@@ -2016,7 +2031,7 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
     const bool ws_plan = is_ws_shape(plan.np, plan.split);
     if ((lowrank && !full_plan_lowrank(plan)) || (a.gather_h > 0 && !ws_plan)) return VMB_ERR_UNSUPPORTED;
     if (lowrank && a.gather_h > 0) return VMB_ERR_UNSUPPORTED;
-    if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream);
+    if (const int G = full_plan_small(plan)) return launch_small(a, G, nullptr, 0, 0, stream, plan.early);
     KernelInfo ki = ws_plan ? ws_info(a.dtype, plan.np, ws_variant(plan.np, plan.split), a.gather_h > 0, a.R)
                             : pick(a.dtype, plan.np, plan.split, (a.flags & VMB_FLAG_B_ZOH) != 0);
     if (!ki.fn) return VMB_ERR_CUDA;
@@ -2119,8 +2134,9 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
         ki = pick(a.dtype, plan.np, kPackedShape, false);
         if (!ki.fn) return VMB_ERR_CUDA;
     }
-    return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream) == cudaSuccess ? VMB_OK
-                                                                                                   : VMB_ERR_CUDA;
+    return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream, plan.early) == cudaSuccess
+               ? VMB_OK
+               : VMB_ERR_CUDA;
 }
 
 }  // namespace vmb

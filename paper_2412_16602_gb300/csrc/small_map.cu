@@ -299,7 +299,7 @@ size_t small_scan_smem(int G, int L, bool map) {
     return (((map ? 5 : 8) * ct * rx + 3) / 4 * 4 + (size_t)4 * L * kBC) * 4;
 }
 
-vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream) {
+vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early) {
     const bool map = out != nullptr;
     const void* fn = a.dtype == VMB_BF16 ? (map ? small_pick<__nv_bfloat16, true>(G) : small_pick<__nv_bfloat16, false>(G))
                                          : (map ? small_pick<float, true>(G) : small_pick<float, false>(G));
@@ -328,7 +328,7 @@ vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaS
     p.fW = make_fastdiv((unsigned)(W > 0 ? W : 1));
     const long long grid = map ? p.units : (p.units + 3) / 4;
     void* args[] = {&p};
-    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSmThreads), small_scan_smem(G, a.L, map), args, stream) ==
+    return launch_kernel(fn, dim3((unsigned)grid), dim3(kSmThreads), small_scan_smem(G, a.L, map), args, stream, early) ==
                    cudaSuccess
                ? VMB_OK
                : VMB_ERR_CUDA;

@@ -181,7 +181,7 @@ int full_plan_small(const ScanPlan& plan);
 constexpr size_t kSmallMaxSmem = 227 * 1024;
 size_t small_scan_smem(int G, int L, bool map);
 // out = null: the scan alone (a.u the sequences); else a.u is the map [B][D][H][W] and K = 4.
-vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream);
+vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early = true);
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
 vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W, vmb_dtype dt,
                              cudaStream_t stream);

@@ -81,6 +81,18 @@ def test_workspace_of_the_query_serves_any_alignment(N):
         check(to_numpy(y), y_ref, "f32", f"full y, shifted by {shift}")
 
 
+@pytest.mark.parametrize("case,early", [
+    # (B, D, N, H, W, dtype, off, flags beyond softplus): barrier-staged plans; a grid of less than one wave
+    # of long-lived CTAs is not launched early, tiny sequences and full waves are
+    ((36, 64, 16, 12, 12, "f32", 0, vmb.VMB_FLAG_B_ZOH), 0), ((3, 1536, 3, 2, 64, "bf16", 1, 0), 0),
+    ((2, 256, 4, 28, 28, "f32", 0, vmb.VMB_FLAG_B_ZOH), 0), ((2, 96, 5, 20, 20, "bf16", 1, 0), 0),
+    ((2, 96, 16, 20, 20, "bf16", 1, 0), 1), ((3, 1536, 3, 2, 16, "bf16", 1, 0), 1), ((128, 512, 4, 8, 8, "f32", 1, 0), 1),
+])
+def test_barrier_staged_grids_launched_early(case, early, full_plan):
+    B, D, N, H, W, dt, off, flags = case
+    assert full_plan(B, 4, D, N, H, W, dt, off=off, flags=vmb.VMB_FLAG_SOFTPLUS | flags)[2] == early
+
+
 @pytest.mark.parametrize("off", [0, 1])
 @pytest.mark.parametrize("case", [
     # (B, K, D, N, L, dtype): narrow tiles, whole tiles and one row more, stages cut short
