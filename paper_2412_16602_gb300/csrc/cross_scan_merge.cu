@@ -8,11 +8,7 @@
 // conflicts; global loads and stores are 16-byte vectors when rows are 16-byte
 // aligned.  Larger maps use band kernels: one CTA per band of rows of one map
 // (eight for the scan, up to 32 for the merge; see below), which keeps batch-1
-// problems parallel.
-//
-// Index arithmetic uses division by invariant integers via multiply-high
-// (Granlund & Montgomery, "Division by invariant integers using
-// multiplication", PLDI 1994, round-up variant), valid for dividends < 2^31.
+// problems parallel.  Which kernel takes rows too long for that: csm_kernel.
 #include <algorithm>
 #include <type_traits>
 
@@ -66,17 +62,40 @@ __device__ __forceinline__ void plane_tables(unsigned short* row, unsigned short
     }
 }
 
+// Without tables (TAB false: planes of kBandMinL pixels or more, whose tables would
+// take shared memory from the plane and are used for one plane only) the indices
+// are computed where they are used.
+struct PlaneIndex {
+    const unsigned short* tab;
+    FastDiv f;   // positions along one row of this order
+    int sm, sq;  // tile strides of the quotient and of the remainder
+    template <bool TAB>
+    __device__ __forceinline__ unsigned at(unsigned i) const {
+        if constexpr (TAB) return tab[i];
+        const unsigned q = fdiv(i, f);
+        return q * sm + (i - q * f.d) * sq;
+    }
+};
+// Index of the tile [H][W+1] (by_col false) or [W][H+1] in row-major and column-major order.
+__device__ __forceinline__ PlaneIndex row_index(const unsigned short* tab, const CsmParams& p, bool by_col) {
+    return {tab, p.fW, by_col ? 1 : p.W + 1, by_col ? p.H + 1 : 1};
+}
+__device__ __forceinline__ PlaneIndex col_index(const unsigned short* tab, const CsmParams& p, bool by_col) {
+    return {tab, p.fH, by_col ? p.H + 1 : 1, by_col ? 1 : p.W + 1};
+}
+
 // Directions 0 and 2 are written straight from the loaded values, 1 and 3 (the same
 // values in opposite orders) from the staged planes.
-template <typename T>
+template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = p.L, PS = p.H * (p.W + 1);
-    unsigned short* row = reinterpret_cast<unsigned short*>(smem_raw);  // [L]
-    unsigned short* col = row + p.tabn;                                 // [L]
-    T* sp = reinterpret_cast<T*>(col + p.tabn);                         // [ppc][H][W+1]
+    unsigned short* rtab = reinterpret_cast<unsigned short*>(smem_raw);  // [L] (TAB)
+    unsigned short* ctab = rtab + p.tabn;                                // [L]
+    T* sp = reinterpret_cast<T*>(ctab + p.tabn);                         // [ppc][H][W+1]
     constexpr int VE = 16 / sizeof(T);
-    plane_tables(row, col, p, false);
+    if constexpr (TAB) plane_tables(rtab, ctab, p, false);
+    const PlaneIndex row = row_index(rtab, p, false), col = col_index(ctab, p, false);
     pdl_wait();
     pdl_launch_dependents();
     __syncthreads();
@@ -100,7 +119,7 @@ __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p)
             const unsigned j = fdiv(i, p.fL), l = i - j * L;
 #pragma unroll
             for (int q = 0; q < VE; ++q) {
-                sp[j * PS + row[l + q]] = v.e[q];
+                sp[j * PS + row.template at<TAB>(l + q)] = v.e[q];
                 r.e[q] = v.e[VE - 1 - q];
             }
             T* o = base(j);
@@ -112,7 +131,7 @@ __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p)
         for (unsigned i = threadIdx.x; i < n; i += kThreads) {
             const T v = src[i];
             const unsigned j = fdiv(i, p.fL), l = i - j * L;
-            sp[j * PS + row[l]] = v;
+            sp[j * PS + row.template at<TAB>(l)] = v;
             T* o = base(j);
             o[l] = v;
             o[2 * DL + (L - 1 - l)] = v;
@@ -126,7 +145,7 @@ __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p)
             Vec<T> v, r;
 #pragma unroll
             for (int q = 0; q < VE; ++q) {
-                v.e[q] = sp[j * PS + col[l + q]];
+                v.e[q] = sp[j * PS + col.template at<TAB>(l + q)];
                 r.e[VE - 1 - q] = v.e[q];
             }
             T* o = base(j);
@@ -137,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p)
 #pragma unroll 2
         for (unsigned i = threadIdx.x; i < n; i += kThreads) {
             const unsigned j = fdiv(i, p.fL), l = i - j * L;
-            const T v = sp[j * PS + col[l]];
+            const T v = sp[j * PS + col.template at<TAB>(l)];
             T* o = base(j);
             o[DL + l] = v;
             o[3 * DL + (L - 1 - l)] = v;
@@ -147,15 +166,16 @@ __global__ void __launch_bounds__(kThreads) cross_scan_kernel(const CsmParams p)
 
 // ys1 + ys3 of every pixel is formed in column-major order and staged in fp32,
 // then added to ys0 + ys2 in row order (the sums and their order as stated above).
-template <typename T>
+template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = p.L, PS = p.W * (p.H + 1);
-    unsigned short* row = reinterpret_cast<unsigned short*>(smem_raw);  // [L]
-    unsigned short* col = row + p.tabn;                                 // [L]
-    float* sp = reinterpret_cast<float*>(col + p.tabn);                 // [ppc][W][H+1]
+    unsigned short* rtab = reinterpret_cast<unsigned short*>(smem_raw);  // [L] (TAB)
+    unsigned short* ctab = rtab + p.tabn;                                // [L]
+    float* sp = reinterpret_cast<float*>(ctab + p.tabn);                 // [ppc][W][H+1]
     constexpr int VE = 16 / sizeof(T);
-    plane_tables(row, col, p, true);
+    if constexpr (TAB) plane_tables(rtab, ctab, p, true);
+    const PlaneIndex row = row_index(rtab, p, true), col = col_index(ctab, p, true);
     pdl_wait();
     pdl_launch_dependents();
     __syncthreads();
@@ -178,14 +198,14 @@ __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p
             v1.v = *reinterpret_cast<const uint4*>(o + DL + l);
             v3.v = *reinterpret_cast<const uint4*>(o + 3 * DL + (L - VE - l));  // reversed block
 #pragma unroll
-            for (int q = 0; q < VE; ++q) sp[j * PS + col[l + q]] = io<T>::cvt(v1.e[q]) + io<T>::cvt(v3.e[VE - 1 - q]);
+            for (int q = 0; q < VE; ++q) sp[j * PS + col.template at<TAB>(l + q)] = io<T>::cvt(v1.e[q]) + io<T>::cvt(v3.e[VE - 1 - q]);
         }
     } else {
 #pragma unroll 2
         for (unsigned i = threadIdx.x; i < n; i += kThreads) {
             const unsigned j = fdiv(i, p.fL), l = i - j * L;
             const T* o = base(j);
-            sp[j * PS + col[l]] = io<T>::cvt(o[DL + l]) + io<T>::cvt(o[3 * DL + (L - 1 - l)]);
+            sp[j * PS + col.template at<TAB>(l)] = io<T>::cvt(o[DL + l]) + io<T>::cvt(o[3 * DL + (L - 1 - l)]);
         }
     }
     __syncthreads();
@@ -200,7 +220,7 @@ __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p
 #pragma unroll
             for (int q = 0; q < VE; ++q) {
                 const float a = io<T>::cvt(v0.e[q]) + io<T>::cvt(v2.e[VE - 1 - q]);
-                o.e[q] = io<T>::to(a + sp[j * PS + row[l + q]]);
+                o.e[q] = io<T>::to(a + sp[j * PS + row.template at<TAB>(l + q)]);
             }
             *reinterpret_cast<uint4*>(out + i) = o.v;
         }
@@ -210,7 +230,7 @@ __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p
             const unsigned j = fdiv(i, p.fL), l = i - j * L;
             const T* y = base(j);
             const float a = io<T>::cvt(y[l]) + io<T>::cvt(y[2 * DL + (L - 1 - l)]);
-            out[i] = io<T>::to(a + sp[j * PS + row[l]]);
+            out[i] = io<T>::to(a + sp[j * PS + row.template at<TAB>(l)]);
         }
     }
 }
@@ -227,6 +247,13 @@ __global__ void __launch_bounds__(kThreads) cross_merge_kernel(const CsmParams p
 constexpr int kRB = 8;
 constexpr int kBandMinL = 1024;
 constexpr int kBandThreads = 128;
+
+// Rows of a merge band: 32 (fp32) or 16 (bf16), fewer while the tiles would not fit.
+inline int merge_band_rows(int W, int es) {
+    int mrb = es == 4 ? 32 : 16;
+    while (mrb > kRB && (size_t)2 * mrb * (W + 1) * es > kMaxSmem) mrb /= 2;
+    return mrb;
+}
 
 struct BandParams {
     const void* in;
@@ -410,15 +437,52 @@ __global__ void cross_merge_direct(const T* ys, T* out, int D, int H, int W, lon
     }
 }
 
+}  // namespace
+
+// Kernel of a cross-scan or cross-merge.  Below 1024 pixels whole planes are staged
+// with index tables.  From there on bands of rows, or, where a row is too long for a band,
+// whole planes with their indices computed, if there is a plane for every SM and whole vectors
+// can be copied (scanning fp32, also single elements of planes that leave room for two); and where neither fits, or a plane takes more
+// than kMaxSmem of staging (counted as two storage-type planes for the merge), bands only
+// where enough of them share an SM, else the gather of single elements.  GB300, us,
+// planes x H x W: scan 192x1x9000 fp32 staged 7.3, gather 34; 192x8x6000 72 and 170; out of
+// line 192x15x2999 187 and 160, 32x3x3297 34 and 13, 216x3x6803 32 and 62;
+// merge 192x2x8000 12 and 18, 16x2x8000 8.7 and 3.9, 192x4x6000 (117 KB staged) 41 and 29.  Merge in bands and
+// gather: 192x256x256 fp32 (64 KB a band) 92 and 104, bf16 30 and 102; 192x64x800 fp32
+// (100 KB) 99 and 80; 16x512x512 fp32 (128 KB) 60 and 36; rows out of line 192x201x201 fp32
+// (50 KB) 127 and 61, 16x401x399 bf16 (25 KB) 17 and 22, 192x7001x12 bf16 166 and 91.
+// Scan 192x15x2999 fp32 out of line (94 KB) 188 and 160, 192x61x997 (31 KB) 123 and 219.
+CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, bool aligned, int sms) {
+    const long long L = (long long)H * W, es = dt == VMB_BF16 ? 2 : 4;
+    if (planes >= (1ll << 31) || L * 4 >= (1ll << 31)) return CsmKernel::kGather;
+    if (L < kBandMinL) return CsmKernel::kPlane;
+    const bool band_fits = 2ll * kRB * (W + 1) * es <= (long long)kMaxSmem &&
+                           planes * ((H + kRB - 1) / kRB) < (1ll << 31);
+    const long long staged = merge ? 2ll * W * (H + 1) * es : (long long)H * (W + 1) * es;
+    if (!band_fits) {
+        const bool vec = aligned && L * es % 16 == 0;
+        const bool whole = staged <= (vec ? (long long)kMaxSmem : !merge && es == 4 ? 96 * 1024 : 0) && planes >= sms;
+        return whole ? CsmKernel::kPlane : CsmKernel::kGather;
+    }
+    if (staged <= (long long)kMaxSmem) return CsmKernel::kBand;
+    const int VE = (int)(16 / es);
+    const bool vec = aligned && W % VE == 0 && H % VE == 0;
+    const long long smem = merge ? 2ll * merge_band_rows(W, (int)es) * (W + 1) * es : (long long)kRB * (W + 1) * es;
+    const bool fast = merge ? (vec ? smem <= 65 * 1024 : smem <= 32 * 1024 && (W >= 64 || planes < sms)) : vec || smem <= 64 * 1024;
+    return fast ? CsmKernel::kBand : CsmKernel::kGather;
+}
+
+namespace {
+
 template <typename T>
 vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int H, int W, cudaStream_t stream) {
     const int L = H * W;
     const long long planes = (long long)B * D;
     const size_t es = sizeof(T);
-    const bool small_enough = planes < (1ll << 31) && (long long)L * 4 < (1ll << 31);
-    const bool band = small_enough && L >= kBandMinL && (size_t)2 * kRB * (W + 1) * es <= kMaxSmem &&
-                      planes * ((H + kRB - 1) / kRB) < (1ll << 31);
-    if (!small_enough || (L >= kBandMinL && !band)) {
+    const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    const bool aligned = al16(in) && al16(outp);
+    const CsmKernel kernel = csm_kernel(merge, sizeof(T) == 2 ? VMB_BF16 : VMB_F32, planes, H, W, aligned, device_sm_count());
+    if (kernel == CsmKernel::kGather) {
         const long long total = merge ? planes * L : planes * 4 * L;
         const int grid = (int)std::min<long long>((total + kThreads - 1) / kThreads, 152ll * 32);
         const void* fn = merge ? reinterpret_cast<const void*>(&cross_merge_direct<T>)
@@ -428,7 +492,7 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
         void* args[] = {&src, &dst, &D, &H, &W, const_cast<long long*>(&total)};
         return launch_kernel(fn, dim3(grid), dim3(kThreads), 0, args, stream) == cudaSuccess ? VMB_OK : VMB_ERR_CUDA;
     }
-    if (band) {
+    if (kernel == CsmKernel::kBand) {
         BandParams bp{};
         bp.in = in;
         bp.out = outp;
@@ -436,15 +500,11 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
         bp.H = H;
         bp.W = W;
         bp.L = L;
-        // merge bands: 32 rows (fp32) or 16 (bf16), fewer while the tiles would
-        // not fit
-        int mrb = es == 4 ? 32 : 16;
-        while (mrb > kRB && (size_t)2 * mrb * (W + 1) * es > kMaxSmem) mrb /= 2;
+        const int mrb = merge_band_rows(W, (int)es);
         bp.mrb = mrb;
         bp.nbands = merge ? (H + mrb - 1) / mrb : (H + kRB - 1) / kRB;
         const int VE = (int)(16 / es);
-        const auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-        bp.vec = (W % VE == 0) && (H % VE == 0) && a16(in) && a16(outp);
+        bp.vec = (W % VE == 0) && (H % VE == 0) && aligned;
         const size_t smem = merge ? 2 * (size_t)mrb * (W + 1) * es : (size_t)kRB * (W + 1) * es;
         const void* fn = merge ? reinterpret_cast<const void*>(&cross_merge_band_kernel<T>)
                                : reinterpret_cast<const void*>(&cross_scan_band_kernel<T>);
@@ -458,7 +518,8 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
     }
     // about 8K elements per CTA, bounded by shared memory, fewer while the grid would
     // leave SMs idle
-    const int tabn = (L + 7) / 8 * 8;
+    const bool tab = L < kBandMinL;  // index tables
+    const int tabn = tab ? (L + 7) / 8 * 8 : 0;
     const size_t tables = (size_t)2 * tabn * 2, plane = merge ? (size_t)W * (H + 1) * 4 : (size_t)H * (W + 1) * es;
     long long want = std::max<long long>(1, std::min<long long>(8192 / L, planes / (4LL * device_sm_count())));
     while (want > 1 && tables + (size_t)want * plane > kMaxSmem) --want;
@@ -473,15 +534,16 @@ vmb_status launch_csm(bool merge, const void* in, void* outp, int B, int D, int 
     p.planes = planes;
     p.ppc = ppc;
     p.tabn = tabn;
-    const auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    p.vec = ((size_t)L * es % 16 == 0) && al16(in) && al16(outp);
+    p.vec = ((size_t)L * es % 16 == 0) && aligned;
     p.fL = make_fastdiv((unsigned)L);
     p.fW = make_fastdiv((unsigned)W);
     p.fH = make_fastdiv((unsigned)H);
     p.fD = make_fastdiv((unsigned)D);
     const size_t smem = tables + (size_t)ppc * plane;
-    const void* fn = merge ? reinterpret_cast<const void*>(&cross_merge_kernel<T>)
-                           : reinterpret_cast<const void*>(&cross_scan_kernel<T>);
+    const void* fn = merge ? (tab ? reinterpret_cast<const void*>(&cross_merge_kernel<T, true>)
+                                  : reinterpret_cast<const void*>(&cross_merge_kernel<T, false>))
+                           : (tab ? reinterpret_cast<const void*>(&cross_scan_kernel<T, true>)
+                                  : reinterpret_cast<const void*>(&cross_scan_kernel<T, false>));
     if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
         return VMB_ERR_CUDA;
     const unsigned grid = (unsigned)((planes + ppc - 1) / ppc);

@@ -673,6 +673,10 @@ const char* vmb_status_string(vmb_status s) {
 
 int vmb_version(void) { return 100; }
 
+int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, int W, int aligned, int sms) {
+    return (int)csm_kernel(merge != 0, dtype, planes, H, W, aligned != 0, sms);
+}
+
 int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
                           int* out) {
     ScanArgs a{};

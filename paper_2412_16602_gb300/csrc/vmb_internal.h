@@ -183,6 +183,9 @@ size_t small_scan_smem(int G, int L, bool map);
 // out = null: the scan alone (a.u the sequences); else a.u is the map [B][D][H][W] and K = 4.
 vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early = true);
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
+// Kernels of the cross-scan and the cross-merge; `aligned`: both tensors 16-byte aligned.
+enum class CsmKernel { kPlane, kBand, kGather };
+CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, bool aligned, int sms);
 vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W, vmb_dtype dt,
                              cudaStream_t stream);
 vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, int W, vmb_dtype dt,

@@ -16,6 +16,10 @@
 extern "C" {
 #endif
 
+/* vmb_testing_csm_kernel: kernel of a cross-scan (merge 0) or cross-merge (1) of `planes`
+ * maps, without a GPU: 0 whole planes, 1 bands, 2 the gather of single elements. */
+int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, int W, int aligned, int sms);
+
 /* What the planner answers, without a launch: out = {tile shape, L-chunks, launched
  * early} of a full scan (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or
  * delta (off & 2) one element past 16-byte alignment.  Returns the status. */

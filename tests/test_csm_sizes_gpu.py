@@ -15,7 +15,10 @@ import paper_2412_16602_gb300 as vmb  # noqa: E402
 DEV = torch.device("cuda", 0)
 
 CASES = [(1, 1, 1, 1), (2, 3, 1, 9), (3, 2, 31, 33), (1, 3, 33, 31), (2, 2, 1, 1023), (1, 2, 1023, 1), (7, 900, 4, 4),
-         (5, 130, 3, 5), (1, 2, 230, 232), (1, 1, 3, 3300)]
+         (5, 130, 3, 5), (1, 2, 230, 232), (1, 1, 3, 3300),
+         # long rows and tall planes: whole planes without index tables, bands, single elements
+         (1, 3, 1, 9000), (2, 2, 7, 3201), (1, 2, 2, 8001), (1, 2, 3, 8793), (1, 1, 201, 201), (1, 2, 14, 1948),
+         (1, 1, 300, 256), (1, 1, 7001, 12), (1, 1, 128, 800)]
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
