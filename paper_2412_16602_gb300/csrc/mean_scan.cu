@@ -916,6 +916,26 @@ KInfo mpick_pair(vmb_dtype dt, int np, int tc, bool lr) {
 
 }  // namespace
 
+// Whether `n` CTAs are faster with two steps per thread, of which res2 are resident at once on
+// `sms` SMs, than with one (res1).  A grid of at most one wave of the one-step kernel is not: fewer
+// threads share an SM, which tells once the channels are more than a few dozen.  Beyond that the waves decide: an SM's share of a two-step wave costs
+// 0.86 of as many one-step CTAs; a last wave is as long as a full one, without y (whose broadcast
+// keeps the last CTAs busy) down to 0.6 of it.  GB300, one step's time over two's, bf16 with y: 72 maps
+// of 56x12x123, one direction (432 CTAs) 0.83, 20 of 28x28x192 (560) 1.16, 32 (896) 0.90, 96 (2688)
+// 1.05; without y 560 CTAs 1.23, 416 CTAs 0.94 (fp32 1.06 and 0.87), 21 maps of 24x24x7 fp32 (420) 1.21.  Over 680 sizes of 150 to 5000
+// CTAs, both types, 8 and 16 states, the rule's choice is within 0.3% of the better one on average
+// and within 12% always.
+bool mean_two_steps(long long n, int D, long long res1, long long res2, int sms, bool with_y) {
+    if (res1 < 1 || res2 < 1 || (n <= res1 && D > 48)) return false;
+    auto cost = [&](long long res, double least) {
+        const double full = (double)res / sms;
+        const long long rest = n % res;
+        const double last = rest ? (double)((rest + sms - 1) / sms) : 0.0;
+        return (n / res) * full + (rest ? (last > least * full ? last : least * full) : 0.0);
+    };
+    return 0.86 * cost(res2, with_y ? 1.0 : 0.6) <= cost(res1, 1.0);
+}
+
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
     if (a.N < 1 || a.N > 16) return VMB_ERR_UNSUPPORTED;
     if ((long long)a.D * a.L >= (1LL << 31)) return VMB_ERR_UNSUPPORTED;  // 32-bit offsets within a (b, k) slab
@@ -973,20 +993,14 @@ vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
                      (a.no_bcast || a.dtype == VMB_BF16) && al2(a.u) && (lr || al2(a.delta)) &&
                      (a.gather_h == 0 || al2(a.u_t));
     KInfo ki = mpick(a.dtype, plan.np, plan.chunk_len, zoh, lr);
-    if (two) {
-        // ... and where its waves do not cost more than they save: four CTAs share an
-        // SM at 0.87 of the time each takes of it, but a last wave costs at least
-        // three quarters of a full one (4 maps of 62x117x384: 912 CTAs, two full waves
-        // of three per SM, 228 us, or one and a half of four, 238)
+    const int forced = forced_mean_steps();  // (test-only)
+    if (forced == 2 && !two) return VMB_ERR_UNSUPPORTED;
+    if (two && forced != 1) {
         const KInfo k2 = mpick_pair(a.dtype, plan.np, plan.chunk_len, lr);
-        const long long sms = device_sm_count(), n = (long long)plan.n_seq * plan.n_chunks;
-        auto cost = [&](const KInfo& k) {
-            const long long res = k.fn ? resident_ctas(k.fn, k.threads, k.smem) : 0;
-            if (res < 1) return 1e30;
-            const double full = (double)res / sms, rest = (double)(n % res) / sms;
-            return (n / res) * full + (n % res ? (rest > 0.75 * full ? rest : 0.75 * full) : 0.0);
-        };
-        if (0.87 * cost(k2) <= cost(ki)) ki = k2;
+        if (!k2.fn || !ki.fn) return VMB_ERR_CUDA;
+        if (forced == 2 || mean_two_steps((long long)plan.n_seq * plan.n_chunks, a.D, resident_ctas(ki.fn, ki.threads, ki.smem),
+                                          resident_ctas(k2.fn, k2.threads, k2.smem), device_sm_count(), !a.no_bcast))
+            ki = k2;
     }
     if (!ki.fn) return VMB_ERR_CUDA;
     MeanParams p{};

@@ -12,7 +12,7 @@
 namespace vmb {
 
 namespace {
-std::atomic<int> g_force_shape{-1}, g_force_chunks{0}, g_force_tc{0};
+std::atomic<int> g_force_shape{-1}, g_force_chunks{0}, g_force_tc{0}, g_force_steps{0};
 }  // namespace
 
 int forced_full_shape(int* chunks) {
@@ -20,6 +20,7 @@ int forced_full_shape(int* chunks) {
     return g_force_shape.load(std::memory_order_relaxed);
 }
 int forced_mean_chunk() { return g_force_tc.load(std::memory_order_relaxed); }
+int forced_mean_steps() { return g_force_steps.load(std::memory_order_relaxed); }
 
 int device_sm_count() {
     static std::mutex mu;
@@ -677,6 +678,10 @@ int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, 
     return (int)csm_kernel(merge != 0, dtype, planes, H, W, aligned != 0, sms);
 }
 
+int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long long res_two, int sms, int with_y) {
+    return mean_two_steps(ctas, D, res_one, res_two, sms, with_y != 0) ? 1 : 0;
+}
+
 int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
                           int* out) {
     ScanArgs a{};
@@ -715,6 +720,12 @@ int vmb_testing_force_full_plan(int shape, int chunks) {
 int vmb_testing_force_mean_chunk(int tc) {
     if (tc != 0 && tc != 32 && tc != 64 && tc != 128) return 1;
     g_force_tc.store(tc, std::memory_order_relaxed);
+    return 0;
+}
+
+int vmb_testing_force_mean_steps(int steps) {
+    if (steps < 0 || steps > 2) return 1;
+    g_force_steps.store(steps, std::memory_order_relaxed);
     return 0;
 }
 

@@ -163,6 +163,7 @@ vmb_status validate_scan(const ScanArgs& a, bool mean, bool* empty);
 // Test-only plan overrides (vmb_testing.h); -1 / 0 when unset.
 int forced_full_shape(int* chunks);
 int forced_mean_chunk();
+int forced_mean_steps();
 
 vmb_status plan_full(const ScanArgs& a, ScanPlan* plan);
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan);
@@ -183,6 +184,7 @@ size_t small_scan_smem(int G, int L, bool map);
 // out = null: the scan alone (a.u the sequences); else a.u is the map [B][D][H][W] and K = 4.
 vmb_status launch_small(const ScanArgs& a, int G, void* out, int H, int W, cudaStream_t stream, bool early = true);
 vmb_status launch_mean(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
+bool mean_two_steps(long long n, int D, long long res1, long long res2, int sms, bool with_y);
 // Kernels of the cross-scan and the cross-merge; `aligned`: both tensors 16-byte aligned.
 enum class CsmKernel { kPlane, kBand, kGather };
 CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, bool aligned, int sms);

@@ -20,6 +20,10 @@ extern "C" {
  * maps, without a GPU: 0 whole planes, 1 bands, 2 the gather of single elements. */
 int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, int W, int aligned, int sms);
 
+/* vmb_testing_mean_two_steps: 1 if `ctas` channel-mean CTAs of D channels take two steps
+ * per thread, given the CTAs that `sms` SMs hold at once with one and with two. */
+int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long long res_two, int sms, int with_y);
+
 /* What the planner answers, without a launch: out = {tile shape, L-chunks, launched
  * early} of a full scan (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or
  * delta (off & 2) one element past 16-byte alignment.  Returns the status. */
@@ -35,6 +39,11 @@ int vmb_testing_force_full_plan(int shape, int chunks);
 /* Force the chunk length of the channel-mean scan (32, 64 or 128; 0 restores
  * the planner).  Returns 0, or 1 for another value (nothing changes). */
 int vmb_testing_force_mean_chunk(int tc);
+
+/* Force one or two steps per thread in the channel-mean scan (0 restores the
+ * rule).  A call that cannot take two returns VMB_ERR_UNSUPPORTED while two are
+ * forced.  Returns 0, or 1 for another value (nothing changes). */
+int vmb_testing_force_mean_steps(int steps);
 
 /* Workspace bytes of the plan one scan call with these exact flags would run
  * (vmb_scan_workspace_bytes returns the larger over the two Bbar forms).

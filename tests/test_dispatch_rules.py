@@ -1,5 +1,5 @@
 """Rules of the dispatch that need no GPU: which kernel takes a cross-scan or
-cross-merge of long rows."""
+cross-merge of long rows, and when the channel-mean scan takes two steps per thread."""
 import ctypes
 
 import pytest
@@ -15,6 +15,7 @@ def lib():
     lib = ctypes.CDLL(_build.build())
     i, ll = ctypes.c_int, ctypes.c_longlong
     lib.vmb_testing_csm_kernel.argtypes = [i, i, ll, i, i, i, i]
+    lib.vmb_testing_mean_two_steps.argtypes = [ll, i, ll, ll, i, i]
     return lib
 
 
@@ -46,3 +47,23 @@ def test_csm_kernel_of_few_planes(lib):
 def test_csm_kernel_of_the_largest_problems(lib):
     assert lib.vmb_testing_csm_kernel(0, F32, 1 << 31, 4, 4, 1, SMS) == GATHER
     assert lib.vmb_testing_csm_kernel(0, F32, 1, 1 << 15, 1 << 15, 1, SMS) == GATHER
+
+
+@pytest.mark.parametrize("ctas,with_y,two", [
+    (1, 0, 0), (304, 0, 0), (416, 0, 0), (416, 1, 0), (432, 1, 0), (456, 1, 0),  # at most one wave with one step
+    (457, 1, 1), (560, 1, 1), (560, 0, 1), (608, 1, 1),                         # one wave with two, two with one
+    (896, 1, 0), (624, 1, 0), (624, 0, 1), (1344, 0, 1),
+    (4096, 0, 1), (4992, 1, 1), (12800, 0, 1), (12800, 1, 1),
+])
+def test_mean_two_steps(lib, ctas, with_y, two):
+    assert lib.vmb_testing_mean_two_steps(ctas, 192, 3 * SMS, 4 * SMS, SMS, with_y) == two
+
+
+def test_mean_two_steps_of_few_channels(lib):
+    assert lib.vmb_testing_mean_two_steps(420, 7, 3 * SMS, 4 * SMS, SMS, 0) == 1
+    assert lib.vmb_testing_mean_two_steps(216, 32, 3 * SMS, 4 * SMS, SMS, 1) == 0
+
+
+def test_mean_two_steps_without_a_kernel(lib):
+    assert lib.vmb_testing_mean_two_steps(4096, 192, 3 * SMS, 0, SMS, 0) == 0
+    assert lib.vmb_testing_mean_two_steps(4096, 192, 0, 4 * SMS, SMS, 0) == 0
