@@ -1628,7 +1628,7 @@ bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows
 
 // Tile shapes per padded state count, in order of preference (fewest lanes
 // per channel first).  The zero-order-hold variant uses the first shape.
-int shape_count(int np) { return np <= 4 ? 2 : np == 8 ? 3 : 24; }
+int shape_count(int np) { return np <= 4 ? 2 : np == 8 ? 4 : 24; }
 constexpr int kLanesShape = 7;   // index of the lane-per-state variant (N <= 16 padded to 16)
 constexpr int kChunkShape = 8;   // first index of the three-launch chunked variant (shapes 8 to 11)
 bool is_chunk_shape(int np, int shape) { return np == 16 && shape >= kChunkShape && shape < kChunkShape + 4; }
@@ -1636,14 +1636,13 @@ constexpr int kStreamShape = 12;  // first index of the streaming one-lane varia
 bool is_stream_shape(int np, int shape) { return np == 16 && shape >= kStreamShape && shape < kStreamShape + 4; }
 constexpr int kPackedShape = 16;  // first index of the packed streaming variant (shapes 16 to 18: G = 1, 2, 4)
 bool is_packed_shape(int np, int shape) { return np == 16 && shape >= kPackedShape && shape < kPackedShape + 3; }
-// The warp-specialised variant (tensor copies; 16-byte rows and aligned tensors): the
-// last shape of fewer states; 16 states: one lane per channel (19) or two (23).
+// The warp-specialised variant (tensor copies; 16-byte rows and aligned tensors): one
+// lane per channel, and two with 8 or 16 states.
 constexpr int kWsShape = 19, kWsTwoShape = 23;
 int ws_shape(int np) { return np <= 4 ? 1 : np == 8 ? 2 : kWsShape; }
-bool is_ws_shape(int np, int shape) {
-    return shape == ws_shape(np) || (np == 16 && shape == kWsTwoShape);
-}
-int ws_variant(int np, int shape) { return np == 16 && shape == kWsTwoShape ? kWsTwoLanes : kWsOneLane; }
+int ws_two_shape(int np) { return np == 16 ? kWsTwoShape : np == 8 ? 3 : -1; }
+bool is_ws_shape(int np, int shape) { return shape == ws_shape(np) || shape == ws_two_shape(np); }
+int ws_variant(int np, int shape) { return shape == ws_two_shape(np) ? kWsTwoLanes : kWsOneLane; }
 constexpr int kSmallShape = 20;  // whole short sequences in shared memory (shapes 20 to 22: G = 1, 4, 16; small_map.cu)
 int small_lanes(int np, int shape) {
     return np == 16 && shape >= kSmallShape && shape < kSmallShape + 3 ? 1 << (2 * (shape - kSmallShape)) : 0;
@@ -1770,10 +1769,12 @@ bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
 // with the CTAs that share an SM; cut into P + 1 chunks, P CTAs a tile run
 // concurrently and each passes over two chunks.  ns per step with one, two and
 // three CTAs per SM, measured on GB300 (fp32, 56x56 maps): 16 states, two lanes a
-// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8).
-double ws_estimate(int np, long long tiles, int L, int sms, int ts, int* chunks) {
-    const double per_step[4][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {51, 79, 111}};
-    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 : 3];
+// channel 51, 79, 111; fewer states 33, 50, 75 (1), 40, 63, 95 (4), 62, 93, 130 (8), two
+// lanes 41, 59, 72.  (bf16 takes the same numbers: its steps are up to 13% longer, alike
+// in every plan.)
+double ws_estimate(int np, bool two, long long tiles, int L, int sms, int ts, int* chunks) {
+    const double per_step[5][3] = {{33, 50, 75}, {40, 63, 95}, {62, 93, 130}, {41, 59, 72}, {51, 79, 111}};
+    const double* c = per_step[np <= 2 ? 0 : np == 4 ? 1 : np == 8 ? 2 + two : 4];
     double best = 0.0;
     for (int P = 1; P <= 24; ++P) {
         if (P > 1 && L / (P + 1) < 4 * ts) break;
@@ -1806,7 +1807,9 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // kernel (small_rule).  Tensors that tensor copies can read, at least two
     // channel rows per SM -> the warp-specialised kernel: one lane per channel from
     // 256 rows per SM on, two lanes below (16 states, fp32, us: 24576 rows of 56x56
-    // 350 with two lanes, 471 with one; 49152 rows of 28x28 168 and 163), L cut into
+    // 350 with two lanes, 471 with one; 49152 rows of 28x28 168 and 163; 8 states, by the
+    // estimate: 9728 rows of 64 steps 5.2 with two, 7.2 with one, the barrier-staged
+    // kernel 7.0, 19456 rows of 28x28 46 and 73, 30464 rows 81 and 77), L cut into
     // chunks where ws_estimate expects a gain (6144 rows of 128x128 bf16 605, one
     // pass 1126, look-back chunks 870; 3072 rows of 56x56 80, look-back 187; one state, 131072 rows
     // of 56x56 779, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
@@ -1872,10 +1875,15 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
     } else if (tma_ok && rows >= 2LL * sms) {
         const bool few = rows < 256LL * sms && (np < 16 || !small_map_one_lane(a.L));
-        shape = np == 16 && few ? kWsTwoShape : ws_shape(np);
+        auto estimate = [&](bool two, int* chunks) {
+            const KernelInfo k = pick(a.dtype, np, two ? ws_two_shape(np) : ws_shape(np), false);
+            return ws_estimate(np, two, a.B * a.K * (long long)((a.D + k.DT - 1) / k.DT), a.L, sms, k.ts, chunks);
+        };
+        int c1 = 1, c2 = 1;
+        const bool two = few && (np == 16 || (np == 8 && a.L >= 16 && estimate(true, &c2) <= estimate(false, &c1)));
+        shape = two ? ws_two_shape(np) : ws_shape(np);
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
-        if (few)
-            ws_estimate(np, a.B * a.K * (long long)((a.D + ki.DT - 1) / ki.DT), a.L, sms, ki.ts, &n_chunks);
+        if (few) estimate(two, &n_chunks);
     } else if (np == 16 && rows >= 256LL * sms && a.L >= 128) {
         // many rows: the packed streaming one-lane kernel, one pass over L (on
         // very short sequences its stage prologue does not pay off)

@@ -537,7 +537,9 @@ WsKernel ws_pick(int np, int variant, bool gather, int R) {
     case 1: return ws_pick_form<T, 1, 1, 16, 8, 3>(gather, 0);
     case 2: return ws_pick_form<T, 2, 1, 16, 8, 3>(gather, 0);
     case 4: return ws_pick_form<T, 4, 1, 16, 8, 3>(gather, 0);
-    case 8: return ws_pick_form<T, 8, 1, 8, 8, 4>(gather, 0);
+    case 8:
+        if (variant == kWsTwoLanes) return ws_pick_form<T, 8, 2, 16, 16, 3>(gather, 0);
+        return ws_pick_form<T, 8, 1, 8, 8, 4>(gather, 0);
     default:
         if (variant == kWsTwoLanes) return ws_pick_form<T, 16, 2, 16, 16, 3>(gather, R);
         return ws_pick_form<T, 16, 1, 8, 8, 4>(gather, R);

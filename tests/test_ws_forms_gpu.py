@@ -1,7 +1,7 @@
 """The forms of the warp-specialised full scan beyond one lane per channel and 16
-states: two lanes per channel (shape 23), L cut into chunks by two launches
-(chunks of shapes 19 and 23 and of fewer states), and 1 to 8 states (the last
-shape of their padded count), against the fp64 oracle, deterministic, and as the
+states: two lanes per channel (shape 23, with 8 padded states 3), L cut into chunks by
+two launches (chunks of shapes 19 and 23 and of fewer states), and 1 to 8 states (shape 1,
+with 8 padded states 2), against the fp64 oracle, deterministic, and as the
 block from the map bit for bit against the three separate calls.  Sizes: ragged
 last stages and chunks, ragged channel tiles, padded states, bf16."""
 import pytest
@@ -36,6 +36,9 @@ CASES = [
     ("2", 1, 40, 8, 16, 24, "bf16"),
     ("1,4", 1, 130, 1, 20, 30, "f32"),
     ("2,5", 1, 40, 8, 20, 30, "f32"),
+    ("3", 2, 72, 5, 9, 12, "f32"),       # padded to 8 states, two lanes
+    ("3", 1, 65, 8, 16, 24, "bf16"),
+    ("3,5", 1, 40, 8, 20, 30, "f32"),
 ]
 
 
@@ -79,6 +82,17 @@ def test_workspace_of_the_query_serves_any_alignment(N):
         y = vmb.vmb_selective_scan_fwd(u, g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W, workspace=ws)
         assert vmb.vmb_read_status(ws) == vmb.VMB_OK
         check(to_numpy(y), y_ref, "f32", f"full y, shifted by {shift}")
+
+
+@pytest.mark.parametrize("case,shape", [
+    # (B, D, N, H, W, dtype): 8 padded states take two lanes for few rows of 16 steps or more
+    ((38, 64, 8, 8, 8, "f32"), 3), ((38, 64, 5, 8, 8, "bf16"), 3), ((4, 64, 8, 128, 128, "bf16"), 3),
+    ((38, 64, 8, 2, 4, "f32"), 2), ((160, 64, 8, 8, 8, "f32"), 2), ((38, 64, 4, 8, 8, "f32"), 1),
+])
+def test_planner_of_eight_states(case, shape, full_plan):
+    B, D, N, H, W, dt = case
+    assert full_plan(B, 4, D, N, H, W, dt)[0] == shape
+    assert full_plan(B, 4, D, N, H, W, dt, map=True)[0] == shape
 
 
 @pytest.mark.parametrize("case,early", [
