@@ -764,6 +764,11 @@ struct TransposeParams {
     FastDiv fP, fA, fB;  // units per plane, per row of x, per row of xt
 };
 
+inline bool transpose_vec(const void* x, const void* xt, int H, int W, int es) {
+    return W % (16 / es) == 0 && H % (16 / es) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(xt)) & 15u) == 0;
+}
+inline int transpose_stride(int H, int VE, bool vec) { return vec ? (H + 8 * VE - 1) / (8 * VE) * (8 * VE) : H | 1; }
+
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(kTrThreads) map_transpose_kernel(const TransposeParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -824,7 +829,7 @@ __global__ void __launch_bounds__(kTrThreads) map_transpose_kernel(const Transpo
     }
 }
 
-// Maps that do not fit an item: 32 x 32 tiles through shared memory (one padded
+// Maps that do not fit an item, or as the caller asks: 32 x 32 tiles through shared memory (one padded
 // column so the transposed reads hit distinct banks), coalesced on both sides.
 constexpr int kTT = 32, kTR = 8;  // tile edge, rows per thread pass
 
@@ -855,21 +860,18 @@ __global__ void __launch_bounds__(kTT * kTR) tile_transpose_kernel(const T* x, T
 
 
 template <typename T>
-vmb_status launch_plane_transpose(const void* x, void* xt, long long planes, int H, int W, cudaStream_t stream, bool* done) {
-    constexpr int VE = 16 / (int)sizeof(T);
-    const auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    const bool vec = W % VE == 0 && H % VE == 0 && a16(x) && a16(xt);
+vmb_status launch_plane_transpose(const void* x, void* xt, long long planes, int H, int W, cudaStream_t stream) {
+    const int VE = 16 / (int)sizeof(T);
+    const bool vec = transpose_vec(x, xt, H, W, (int)sizeof(T));
     const int ve = vec ? VE : 1, nv = vec ? kTrVals : 4 * kTrVals;
     TransposeParams p{};
     p.x = x;
     p.xt = xt;
     p.H = H;
     p.W = W;
-    p.HP = vec ? (H + 8 * VE - 1) / (8 * VE) * (8 * VE) : H | 1;
+    p.HP = transpose_stride(H, VE, vec);
     const long long L = (long long)H * W;
     const size_t plane_bytes = (size_t)W * p.HP * sizeof(T);
-    *done = L <= (long long)nv * kTrThreads * ve && plane_bytes <= kTrSmem;
-    if (!*done) return VMB_OK;
     const long long fit = std::min<long long>((long long)nv * kTrThreads * ve / L, (long long)(kTrSmem / plane_bytes));
     const int sms = device_sm_count();
     p.ppi = (int)std::max<long long>(1, std::min(fit, (planes + sms - 1) / sms));
@@ -889,11 +891,18 @@ vmb_status launch_plane_transpose(const void* x, void* xt, long long planes, int
 
 }  // namespace
 
-vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, cudaStream_t stream) {
-    bool done = false;
-    const vmb_status st = dt == VMB_BF16 ? launch_plane_transpose<__nv_bfloat16>(x, xt, (long long)B * D, H, W, stream, &done)
-                                         : launch_plane_transpose<float>(x, xt, (long long)B * D, H, W, stream, &done);
-    if (done) return st;
+bool transpose_by_planes(const void* x, const void* xt, int H, int W, vmb_dtype dt) {
+    const int es = dt == VMB_BF16 ? 2 : 4, VE = 16 / es;
+    const bool vec = transpose_vec(x, xt, H, W, es);
+    return (long long)H * W <= (long long)(vec ? kTrVals * VE : 4 * kTrVals) * kTrThreads &&
+           (size_t)W * transpose_stride(H, VE, vec) * es <= kTrSmem;
+}
+
+vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, bool planes,
+                                cudaStream_t stream) {
+    if (planes)
+        return dt == VMB_BF16 ? launch_plane_transpose<__nv_bfloat16>(x, xt, (long long)B * D, H, W, stream)
+                              : launch_plane_transpose<float>(x, xt, (long long)B * D, H, W, stream);
     const int tiles_h = (H + kTT - 1) / kTT, tiles_w = (W + kTT - 1) / kTT;
     const long long grid = (long long)B * D * tiles_h * tiles_w;
     if (grid > INT32_MAX) return VMB_ERR_UNSUPPORTED;

@@ -2112,11 +2112,12 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
             // launched early, behind a kernel that still holds shared memory, a CTA that
             // fills its share of the SM waits for it or lands elsewhere (128 maps of
             // 56x56x256 as the block: four slots 1966 us, five 2081)
-            // gathering, the kernel before is the one-CTA-per-SM transpose, beside which
-            // half of the grid runs: launched early at any size in one pass (24576 rows
+            // gathering, the kernel before is the transpose: one CTA per SM, beside which
+            // half of the grid runs, unless its planes are too large for that: launched early at any size in one pass (24576 rows
             // of 56x56: 436 us, 452 launched after it), but not chunked (6144 rows of
             // 128x128 bf16: 747, 705)
-            const bool beside = gather && plan.n_chunks == 1;
+            const bool beside = gather && plan.n_chunks == 1 &&
+                                transpose_by_planes(a.u, a.u_t, a.gather_h, a.L / a.gather_h, a.dtype);
             p.nstg = plan.early && !sub_wave ? kWsMinSlots
                                              : ws_slots(ki, ctas, device_sm_count(), beside ? kTransposeSmem : 0);
             const bool early = plan.early || beside;

@@ -936,6 +936,21 @@ bool mean_two_steps(long long n, int D, long long res1, long long res2, int sms,
     return 0.86 * cost(res2, with_y ? 1.0 : 0.6) <= cost(res1, 1.0);
 }
 
+// Beside the transpose by planes the CTAs of half of the directions start at once; a grid that
+// leaves SMs with free slots is then placed unevenly, and stays so (us: 2 maps of 22x48x1024
+// fp32 out of line 58, after the transpose by tiles 47; one of 88x16x1536 54 and 45).  Planes that
+// leave most of a tile empty, maps of less than 2.5 MB and more than 8192 tiles are not cut into
+// tiles all the same (1 map of 10x10x1536 62 us by planes, 85 by tiles; of 24x24x768 23.8 and 25.8; 16
+// of 28x20x576 57 and 61).
+bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W) {
+    if (!transpose_by_planes(a.u, a.u_t, H, W, a.dtype)) return false;
+    const long long tiles = (long long)a.B * a.D * ((H + 31) / 32) * ((W + 31) / 32);
+    const long long pixels = (long long)a.B * a.D * H * W;
+    if (tiles > 8192 || 20 * pixels < 9 * 1024 * tiles || pixels * (a.dtype == VMB_BF16 ? 2 : 4) < 2500000) return true;
+    const KInfo ki = mpick(a.dtype, plan.np, plan.chunk_len, (a.flags & VMB_FLAG_B_ZOH) != 0, false);
+    return ki.fn && (long long)plan.n_seq * plan.n_chunks >= resident_ctas(ki.fn, ki.threads, ki.smem);
+}
+
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {
     if (a.N < 1 || a.N > 16) return VMB_ERR_UNSUPPORTED;
     if ((long long)a.D * a.L >= (1LL << 31)) return VMB_ERR_UNSUPPORTED;  // 32-bit offsets within a (b, k) slab

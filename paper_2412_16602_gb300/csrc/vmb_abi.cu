@@ -369,7 +369,7 @@ vmb_status vmb_ss2d_mean_fwd(const void* x, void* xt, const void* delta, const f
     s = plan_mean(a, &plan);
     if (s != VMB_OK) return s;
     if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
-    s = launch_map_transpose(x, xt, B, D, H, W, dtype, stream);
+    s = launch_map_transpose(x, xt, B, D, H, W, dtype, mean_beside_transpose(a, plan, H, W), stream);
     if (s != VMB_OK) return s;
     s = launch_mean(a, plan, stream);
     if (s != VMB_OK) return s;
@@ -482,7 +482,7 @@ vmb_status vmb_ss2d_full_fwd(const void* x, void* xt, const void* delta, const f
     if ((small || full_plan_gathers(plan)) && workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
     if (small) return launch_small(a, small, out, H, W, stream);
     if (full_plan_gathers(plan)) {
-        s = launch_map_transpose(x, xt, B, D, H, W, dtype, stream);
+        s = launch_map_transpose(x, xt, B, D, H, W, dtype, transpose_by_planes(x, xt, H, W, dtype), stream);
         if (s != VMB_OK) return s;
         s = launch_full(a, plan, stream);
     } else {

@@ -192,10 +192,15 @@ vmb_status launch_cross_scan(const void* x, void* xs, int B, int D, int H, int W
                              cudaStream_t stream);
 vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, int W, vmb_dtype dt,
                               cudaStream_t stream);
-// The transpose runs as one CTA per SM of at most this shared memory (1 KB of the CTA's own included).
+// The transpose by whole planes (transpose_by_planes: they fit) runs as one CTA per SM of at
+// most this shared memory (1 KB of the CTA's own included), beside which the scan starts;
+// otherwise 32 x 32 tiles.
 constexpr size_t kTransposeSmem = 33 * 1024;
-vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt,
+bool transpose_by_planes(const void* x, const void* xt, int H, int W, vmb_dtype dt);
+vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, bool planes,
                                 cudaStream_t stream);
+// Whether the channel-mean scan of this plan runs beside the transpose by planes.
+bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W);
 vmb_status launch_discretise(const DiscArgs& a, bool mean, cudaStream_t stream);
 vmb_status launch_selection(const SelArgs& a, cudaStream_t stream);
 size_t mean_bwd_workspace_bytes(long long B, long long K, long long D, long long N, long long L, long long G);
