@@ -350,6 +350,14 @@ const void* sel_fn() {
 
 }  // namespace
 
+// Two buffers while the grid is at most two CTAs per SM (GB300, low-rank form,
+// 32 maps of 14x14x768, 256 CTAs: 57.0 us with two buffers, 60.7 with one, 50.9
+// with two chunks' loads in flight as well); more CTAs hide a chunk's latencies
+// behind one another better than a second buffer does.  Up to two chunks have little
+// to overlap and pay for setting up the buffers (38 maps of 4x4x27: 4.68 us with two,
+// 4.25 with one).
+bool selection_two_buffers(long long grid, int D, int sms) { return grid <= 2LL * sms && D > 2 * kSelKC; }
+
 vmb_status launch_selection(const SelArgs& a, cudaStream_t stream) {
     SelParams p{};
     p.u = a.u;
@@ -369,11 +377,7 @@ vmb_status launch_selection(const SelArgs& a, cudaStream_t stream) {
     p.nlb = (a.L + kSelThreads - 1) / kSelThreads;
     const long long grid = (long long)a.B * a.K * p.nlb;
     if (grid > INT32_MAX) return VMB_ERR_UNSUPPORTED;
-    // Two buffers while the grid is at most two CTAs per SM (GB300, low-rank form,
-    // 32 maps of 14x14x768, 256 CTAs: 57.0 us with two buffers, 60.7 with one, 50.9
-    // with two chunks' loads in flight as well); more CTAs hide a chunk's latencies
-    // behind one another better than a second buffer does.
-    const bool two = grid <= 2LL * device_sm_count();
+    const bool two = selection_two_buffers(grid, a.D, device_sm_count());
     const void* fn = a.dtype == VMB_BF16 ? (two ? sel_fn<__nv_bfloat16, 2>() : sel_fn<__nv_bfloat16, 1>())
                                          : (two ? sel_fn<float, 2>() : sel_fn<float, 1>());
     if (!fn) return VMB_ERR_CUDA;

@@ -682,6 +682,8 @@ int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long lo
     return mean_two_steps(ctas, D, res_one, res_two, sms, with_y != 0) ? 1 : 0;
 }
 
+int vmb_testing_selection_buffers(long long grid, int D, int sms) { return selection_two_buffers(grid, D, sms) ? 2 : 1; }
+
 int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
                           int* out) {
     ScanArgs a{};

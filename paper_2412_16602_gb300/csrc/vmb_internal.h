@@ -202,6 +202,7 @@ vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, in
 // Whether the channel-mean scan of this plan runs beside the transpose by planes.
 bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W);
 vmb_status launch_discretise(const DiscArgs& a, bool mean, cudaStream_t stream);
+bool selection_two_buffers(long long grid, int D, int sms);
 vmb_status launch_selection(const SelArgs& a, cudaStream_t stream);
 size_t mean_bwd_workspace_bytes(long long B, long long K, long long D, long long N, long long L, long long G);
 vmb_status launch_mean_bwd(const MeanBwdArgs& a, cudaStream_t stream);

@@ -24,6 +24,9 @@ int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, 
  * per thread, given the CTAs that `sms` SMs hold at once with one and with two. */
 int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long long res_two, int sms, int with_y);
 
+/* vmb_testing_selection_buffers: operand buffers of a selection grid. */
+int vmb_testing_selection_buffers(long long grid, int D, int sms);
+
 /* What the planner answers, without a launch: out = {tile shape, L-chunks, launched
  * early} of a full scan (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or
  * delta (off & 2) one element past 16-byte alignment.  Returns the status. */

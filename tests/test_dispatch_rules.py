@@ -1,5 +1,6 @@
 """Rules of the dispatch that need no GPU: which kernel takes a cross-scan or
-cross-merge of long rows, and when the channel-mean scan takes two steps per thread."""
+cross-merge of long rows, when the channel-mean scan takes two steps per thread, and
+when the selection kernel takes two operand buffers."""
 import ctypes
 
 import pytest
@@ -16,6 +17,7 @@ def lib():
     i, ll = ctypes.c_int, ctypes.c_longlong
     lib.vmb_testing_csm_kernel.argtypes = [i, i, ll, i, i, i, i]
     lib.vmb_testing_mean_two_steps.argtypes = [ll, i, ll, ll, i, i]
+    lib.vmb_testing_selection_buffers.argtypes = [ll, i, i]
     return lib
 
 
@@ -67,3 +69,8 @@ def test_mean_two_steps_of_few_channels(lib):
 def test_mean_two_steps_without_a_kernel(lib):
     assert lib.vmb_testing_mean_two_steps(4096, 192, 3 * SMS, 0, SMS, 0) == 0
     assert lib.vmb_testing_mean_two_steps(4096, 192, 0, 4 * SMS, SMS, 0) == 0
+
+
+@pytest.mark.parametrize("grid,D,buffers", [(256, 768, 2), (304, 33, 2), (305, 768, 1), (38, 27, 1), (300, 32, 1)])
+def test_selection_buffers(lib, grid, D, buffers):
+    assert lib.vmb_testing_selection_buffers(grid, D, SMS) == buffers
