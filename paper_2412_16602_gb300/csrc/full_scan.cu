@@ -1612,7 +1612,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 bool encode_rows(CUtensorMap* m, const void* base, vmb_dtype dt, int L, int rows, long long planes, int box_ts,
                  int box_rows, bool swizzled = false) {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc) return false;
+    if (!enc || refuse_tensor_maps()) return false;
     const cuuint64_t es = dt == VMB_BF16 ? 2 : 4;
     const cuuint64_t dims[3] = {(cuuint64_t)L, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)L * es, (cuuint64_t)rows * L * es};
@@ -2034,7 +2034,7 @@ int full_plan_launches(const ScanPlan& plan) {
     return (is_chunk_shape(plan.np, plan.split) && plan.n_chunks > 1) ? 3 : 1;
 }
 
-vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream) {
+vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream, bool* refused) {
     const bool lowrank = a.R > 0;
     const bool ws_plan = is_ws_shape(plan.np, plan.split);
     if ((lowrank && !full_plan_lowrank(plan)) || (a.gather_h > 0 && !ws_plan)) return VMB_ERR_UNSUPPORTED;
@@ -2136,12 +2136,19 @@ vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t str
                        ? VMB_OK
                        : VMB_ERR_CUDA;
         }
-        // the encoder refused the tensors: the packed streaming variant (same tiles, same
-        // results), which reads materialised sequences only (no fallback of the other variants)
-        if (gather || lowrank || plan.np != 16 || ws_variant(plan.np, plan.split) == kWsTwoLanes)
-            return VMB_ERR_UNSUPPORTED;
-        ki = pick(a.dtype, plan.np, kPackedShape, false);
-        if (!ki.fn) return VMB_ERR_CUDA;
+        // the encoder refused the tensors: nothing is launched here; a scan of materialised
+        // sequences takes the plan of tensors that tensor copies cannot read, the other forms
+        // are the caller's
+        if (refused) *refused = true;
+        if (gather || lowrank) return VMB_ERR_UNSUPPORTED;
+        ScanArgs m = a;
+        m.no_tma = true;
+        ScanPlan mplan{};
+        const vmb_status st = plan_full(m, &mplan);
+        if (st != VMB_OK) return st;
+        if (is_ws_shape(mplan.np, mplan.split)) return VMB_ERR_UNSUPPORTED;
+        if (a.ws_bytes < mplan.ws_bytes) return VMB_ERR_WORKSPACE;
+        return launch_full(m, mplan, stream);
     }
     return launch_kernel(ki.fn, dim3(grid), dim3(ki.threads), ki.smem, args, stream, plan.early) == cudaSuccess
                ? VMB_OK

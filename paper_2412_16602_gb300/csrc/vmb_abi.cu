@@ -12,7 +12,7 @@
 namespace vmb {
 
 namespace {
-std::atomic<int> g_force_shape{-1}, g_force_chunks{0}, g_force_tc{0}, g_force_steps{0};
+std::atomic<int> g_force_shape{-1}, g_force_chunks{0}, g_force_tc{0}, g_force_steps{0}, g_refuse_maps{0};
 }  // namespace
 
 int forced_full_shape(int* chunks) {
@@ -21,6 +21,7 @@ int forced_full_shape(int* chunks) {
 }
 int forced_mean_chunk() { return g_force_tc.load(std::memory_order_relaxed); }
 int forced_mean_steps() { return g_force_steps.load(std::memory_order_relaxed); }
+bool refuse_tensor_maps() { return g_refuse_maps.load(std::memory_order_relaxed) != 0; }
 
 int device_sm_count() {
     static std::mutex mu;
@@ -371,6 +372,7 @@ vmb_status vmb_ss2d_mean_fwd(const void* x, void* xt, const void* delta, const f
     if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
     s = launch_map_transpose(x, xt, B, D, H, W, dtype, mean_beside_transpose(a, plan, H, W), stream);
     if (s != VMB_OK) return s;
+    // (nothing may be enqueued in between, as in vmb_ss2d_full_fwd)
     s = launch_mean(a, plan, stream);
     if (s != VMB_OK) return s;
     return launch_mean_merge(x, ybar, Dskip, out, B, D, H, W, (flags & VMB_FLAG_SKIP_MEAN) == 0, dtype, stream);
@@ -398,12 +400,18 @@ vmb_status vmb_selective_scan_lowrank_fwd(const void* u, const float* z, const f
     ScanPlan plan{};
     s = plan_full(a, &plan);
     if (s != VMB_OK) return s;
-    if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
-    if (full_plan_lowrank(plan)) return launch_full(a, plan, stream);
-    // a plan whose kernel reads materialised raw Deltas: they are written into
-    // y and the scan runs in place (each of its CTAs reads the steps of its own
-    // rows before it writes them, and no other CTA touches them)
+    bool refused = false;
+    if (full_plan_lowrank(plan)) {
+        if (workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
+        s = launch_full(a, plan, stream, &refused);
+        if (!refused) return s;
+    }
+    // a plan whose kernel reads materialised raw Deltas (or tensors whose maps the
+    // driver refused): they are written into y and the scan runs in place (each step
+    // is written by one CTA, after every CTA that reads it has: the chunked plans
+    // read a chunk once more, for its aggregate, in the launch before)
     ScanArgs m = a;
+    m.no_tma = refused;
     m.delta = y;
     m.Wup = nullptr;
     m.R = 0;
@@ -481,15 +489,22 @@ vmb_status vmb_ss2d_full_fwd(const void* x, void* xt, const void* delta, const f
     const int small = full_plan_small(plan);
     if ((small || full_plan_gathers(plan)) && workspace_bytes < plan.ws_bytes) return VMB_ERR_WORKSPACE;
     if (small) return launch_small(a, small, out, H, W, stream);
+    bool refused = false;
     if (full_plan_gathers(plan)) {
         s = launch_map_transpose(x, xt, B, D, H, W, dtype, transpose_by_planes(x, xt, H, W, dtype), stream);
         if (s != VMB_OK) return s;
-        s = launch_full(a, plan, stream);
-    } else {
-        // a plan whose kernel reads materialised sequences: the cross-scan goes
-        // into y and the scan runs in place (each of its CTAs reads the steps of
-        // its own rows before it writes them, and no other CTA touches them)
+        // (nothing may be enqueued in between: half of the scan's CTAs do not wait for the
+        // launch before them, see pdl_wait)
+        s = launch_full(a, plan, stream, &refused);
+    }
+    if (refused || !full_plan_gathers(plan)) {
+        // a plan whose kernel reads materialised sequences (or tensors whose maps the
+        // driver refused): the cross-scan goes into y and the scan runs in place (each
+        // step is written by one CTA, after every CTA that reads it has: the chunked
+        // plans read a chunk once more, for its aggregate, in the launch before, or in the
+        // CTA that writes it)
         ScanArgs m = a;
+        m.no_tma = refused;
         m.u = y;
         m.gather_h = 0;
         m.u_t = nullptr;
@@ -722,6 +737,11 @@ int vmb_testing_force_full_plan(int shape, int chunks) {
 int vmb_testing_force_mean_chunk(int tc) {
     if (tc != 0 && tc != 32 && tc != 64 && tc != 128) return 1;
     g_force_tc.store(tc, std::memory_order_relaxed);
+    return 0;
+}
+
+int vmb_testing_refuse_tensor_maps(int on) {
+    g_refuse_maps.store(on != 0, std::memory_order_relaxed);
     return 0;
 }
 

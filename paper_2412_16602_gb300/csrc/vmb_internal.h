@@ -35,7 +35,7 @@ struct ScanArgs {
     float* saved = nullptr;  // mean path: the group means kept for the backward, [B*K][N + 1][L] fp32
     const float* Wup = nullptr;  // full path, low-rank Delta: delta is z [B*K][R][L] fp32 and
     int R = 0;                   // delta_raw = Wup z (Wup [K][D][R]); warp-specialised plans only
-    bool no_tma = false;         // full path, workspace query: plan as for tensors that tensor copies cannot read
+    bool no_tma = false;         // full path: plan as for tensors that tensor copies cannot read
 };
 
 // Execution plan of an L-chunked scan: how the (sequence, chunk) grid is cut
@@ -164,10 +164,14 @@ vmb_status validate_scan(const ScanArgs& a, bool mean, bool* empty);
 int forced_full_shape(int* chunks);
 int forced_mean_chunk();
 int forced_mean_steps();
+bool refuse_tensor_maps();
 
 vmb_status plan_full(const ScanArgs& a, ScanPlan* plan);
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan);
-vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream);
+// (*refused: the driver's tensor-map encoder refused the tensors of a warp-specialised plan.  A
+// scan of materialised sequences has then been launched with another plan; one that gathers or
+// expands has not been, and its tensors have to be materialised, ScanArgs::no_tma.)
+vmb_status launch_full(const ScanArgs& a, const ScanPlan& plan, cudaStream_t stream, bool* refused = nullptr);
 int full_plan_launches(const ScanPlan& plan);  // kernels launch_full starts for this plan
 // Whether launch_full can read the plan's u gathered from the map (ScanArgs::gather_h):
 // the warp-specialised plans; or expand a low-rank Delta (ScanArgs::R): those of 16 states.

@@ -16,20 +16,19 @@
 extern "C" {
 #endif
 
-/* vmb_testing_csm_kernel: kernel of a cross-scan (merge 0) or cross-merge (1) of `planes`
- * maps, without a GPU: 0 whole planes, 1 bands, 2 the gather of single elements. */
+/* What the rules of the dispatch answer, without a launch (csm, mean steps and selection
+ * also without a GPU).
+ * vmb_testing_csm_kernel: kernel of a cross-scan (merge 0) or cross-merge (1) of
+ *   `planes` maps: 0 whole planes, 1 bands, 2 the gather of single elements.
+ * vmb_testing_mean_two_steps: 1 if `ctas` channel-mean CTAs take two steps per
+ *   thread, given the CTAs that `sms` SMs hold at once with one and with two.
+ * vmb_testing_selection_buffers: operand buffers of a selection grid.
+ * vmb_testing_full_plan: out = {tile shape, L-chunks, launched early} of a full scan
+ *   (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or delta (off & 2) one element
+ *   past 16-byte alignment.  Returns the status. */
 int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, int W, int aligned, int sms);
-
-/* vmb_testing_mean_two_steps: 1 if `ctas` channel-mean CTAs of D channels take two steps
- * per thread, given the CTAs that `sms` SMs hold at once with one and with two. */
 int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long long res_two, int sms, int with_y);
-
-/* vmb_testing_selection_buffers: operand buffers of a selection grid. */
 int vmb_testing_selection_buffers(long long grid, int D, int sms);
-
-/* What the planner answers, without a launch: out = {tile shape, L-chunks, launched
- * early} of a full scan (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or
- * delta (off & 2) one element past 16-byte alignment.  Returns the status. */
 int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
                           int* out);
 
@@ -47,6 +46,10 @@ int vmb_testing_force_mean_chunk(int tc);
  * rule).  A call that cannot take two returns VMB_ERR_UNSUPPORTED while two are
  * forced.  Returns 0, or 1 for another value (nothing changes). */
 int vmb_testing_force_mean_steps(int steps);
+
+/* Let every tensor-map encoding fail (1), as a driver that refuses the tensors
+ * would (0 restores it).  Returns 0. */
+int vmb_testing_refuse_tensor_maps(int on);
 
 /* Workspace bytes of the plan one scan call with these exact flags would run
  * (vmb_scan_workspace_bytes returns the larger over the two Bbar forms).

@@ -37,7 +37,8 @@ def full_plan():
 @pytest.fixture
 def force_plan():
     """Force a tile shape / chunk count of the full scan ("shape[,chunks]") or a
-    chunk length or the steps per thread of the channel-mean scan through libvmb's test-only controls
+    chunk length or the steps per thread of the channel-mean scan, or let the
+    encoding of tensor maps fail, through libvmb's test-only controls
     (declared in paper_2412_16602_gb300/csrc/vmb_testing.h, not in the public
     header); the planners are restored when the test ends."""
     import ctypes
@@ -51,6 +52,7 @@ def force_plan():
     lib.vmb_testing_force_mean_chunk.argtypes = [ctypes.c_int]
     lib.vmb_testing_force_mean_chunk.restype = ctypes.c_int
     lib.vmb_testing_force_mean_steps.argtypes = [ctypes.c_int]
+    lib.vmb_testing_refuse_tensor_maps.argtypes = [ctypes.c_int]
 
     def full(spec: str):
         shape, _, chunks = str(spec).partition(",")
@@ -62,9 +64,13 @@ def force_plan():
     def mean_steps(n):
         assert lib.vmb_testing_force_mean_steps(int(n)) == 0
 
+    def refuse_tensor_maps(on=True):
+        assert lib.vmb_testing_refuse_tensor_maps(int(on)) == 0
+
     try:
-        yield types.SimpleNamespace(full=full, mean=mean, mean_steps=mean_steps)
+        yield types.SimpleNamespace(full=full, mean=mean, mean_steps=mean_steps, refuse_tensor_maps=refuse_tensor_maps)
     finally:
         lib.vmb_testing_force_mean_steps(0)
+        lib.vmb_testing_refuse_tensor_maps(0)
         lib.vmb_testing_force_full_plan(-1, 0)
         lib.vmb_testing_force_mean_chunk(0)

@@ -107,6 +107,45 @@ def test_barrier_staged_grids_launched_early(case, early, full_plan):
     assert full_plan(B, 4, D, N, H, W, dt, off=off, flags=vmb.VMB_FLAG_SOFTPLUS | flags)[2] == early
 
 
+@pytest.mark.parametrize("case", [
+    # (plan, B, D, N, H, W, dtype)
+    ("", 2, 200, 1, 16, 24, "f32"), ("", 4, 200, 4, 20, 30, "bf16"), ("", 2, 200, 8, 16, 24, "f32"),
+    ("23", 2, 72, 16, 20, 30, "f32"), ("23,4", 1, 72, 16, 20, 30, "bf16"), ("19", 2, 130, 13, 9, 12, "f32"),
+    ("19,4", 1, 130, 16, 20, 30, "f32"),
+], ids=lambda c: "plan{}_B{}_D{}_N{}_{}x{}_{}".format(*c))
+def test_tensor_maps_refused(case, force_plan, full_plan):
+    """Where the driver refuses the tensor maps, a call runs on kernels without tensor
+    copies: the scan, the block from the map and the low-rank form."""
+    plan, B, D, N, H, W, dt = case
+    if plan:
+        force_plan.full(plan)
+    else:
+        shape = full_plan(B, 4, D, N, H, W, dt)[0]
+        assert shape >= (1 if N <= 4 else 2)  # the warp-specialised kernel
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=600 + D + N)
+    inp = workloads.make_inputs(wl, params="random")
+    g = to_device(inp, DEV)
+    args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+    xs = vmb.vmb_cross_scan(g["x"])
+    gen = torch.Generator(device=DEV).manual_seed(7)
+    z = torch.randn(B, 4, 5, H * W, device=DEV, generator=gen)
+    wup = 0.2 * torch.randn(4, D, 5, device=DEV, generator=gen)
+    low = (xs, z, wup, g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W)
+    y_low = vmb.vmb_selective_scan_lowrank_fwd(*low)
+    force_plan.refuse_tensor_maps()
+    force_plan.full("-1")
+    y = vmb.vmb_selective_scan_fwd(xs, *args, H, W)
+    out, ym = vmb.vmb_ss2d_full_fwd(g["x"], *args)
+    y_low2 = vmb.vmb_selective_scan_lowrank_fwd(*low)
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    _, y_ref, out_ref = oracle.ss2d_full(inp)
+    check(to_numpy(y), y_ref, dt, "full y")
+    check(to_numpy(ym), y_ref, dt, "full y from the map")
+    check(to_numpy(out), out_ref, dt, "full out from the map")
+    # (the raw Deltas are rounded to bf16 where they are materialised)
+    check(to_numpy(y_low2), to_numpy(y_low).astype("float64"), dt, "low rank")
+
+
 @pytest.mark.parametrize("off", [0, 1])
 @pytest.mark.parametrize("case", [
     # (B, K, D, N, L, dtype): narrow tiles, whole tiles and one row more, stages cut short
