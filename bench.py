@@ -466,6 +466,19 @@ def sweep_configs(vmb, dev, peak, prelude_flush, warmup):
     return table
 
 
+def configs_summary(table):
+    """The sweep for the result line: microseconds per workload (the whole table, twenty
+    times as long, goes to the standard error stream: a reader that keeps the end of the
+    output must find the line whole)."""
+    if table is None:
+        return None
+    return {name: {"calls": r["calls"], "full_scan_us": round(r["kernels"]["full_scan"]["us"], 2),
+                   "mean_scan_us": round(r["kernels"]["mean_scan"]["us"], 2),
+                   "full_map_us": round(r["full_path_from_map"]["us"], 2),
+                   "mean_map_us": round(r["mean_path_fused"]["gathered_from_map"]["us"], 2)}
+            for name, r in table.items()}
+
+
 def run_ours(args, wl, rank, world, local_rank):
     import torch
     import paper_2412_16602_gb300 as vmb
@@ -947,9 +960,9 @@ def main():
                                   "frac_of_peak": kb["mean_scan"] / (us / 1e6) / 1e9 / peak}
                          for G, us in res["grouped_us"].items()},
         "clocks": res["clocks"],
-        # every workload of the configuration list, kernel by kernel (inputs drawn
-        # on the device with the same recipe; the headline above is one of them)
-        "configs": res["configs"],
+        # every workload of the configuration list (inputs drawn on the device with the
+        # same recipe; the headline above is one of them); kernel by kernel on stderr
+        "configs": configs_summary(res["configs"]),
         "e2e": {"value": job_throughput(step_bytes, world, res["e2e_ms"] / args.e2e_steps), "unit": "GB/s",
                 "ms_per_step": res["e2e_ms"] / args.e2e_steps,
                 "h2d_bytes_per_step": res["h2d"], "d2h_bytes_per_step": res["d2h"],
@@ -962,6 +975,8 @@ def main():
         line["cpu_baseline"] = {"value": cpu_bytes / (cms / 1e3) / 1e9, "unit": "GB/s", "cores": nth,
                                 "kind": "oracle", "ms_per_step": cms,
                                 "sample": f"{len(times)} oracle steps, ~10 s: {cpu_sample}"}
+    if res["configs"] is not None:
+        print(json.dumps({"configs": res["configs"]}), file=sys.stderr)
     print(json.dumps(line))
     if world > 1:
         import torch

@@ -68,3 +68,20 @@ def test_alu_view_and_paper_summary():
     assert out["w"]["scan_only_full"]["frac_of_peak"] == pytest.approx(0.1)
     assert out["paper_a6000_base_512x3136"]["scan_only_full_ms"] == 5.86
     assert bench.paper_style_summary(None, 6784.8) is None
+
+
+def test_configs_summary_keeps_the_line_short():
+    """The sweep of all workloads in the result line: a few times each, a small part of a
+    reader's last 14 KB of output."""
+    import json
+
+    import bench
+    import workloads
+    row = {"calls": 50, "kernels": {k: {"us": 14.349440094083548, "gbs": 136.7, "frac_of_peak": 0.02} for k in bench.KERNELS},
+           "full_path_from_map": {"us": 16.4767998829484}, "mean_path_fused": {"gathered_from_map": {"us": 23.489280380308628}}}
+    out = bench.configs_summary({name: row for name in workloads.WORKLOADS})
+    assert set(out) == set(workloads.WORKLOADS)
+    assert out[bench.DEFAULT_WORKLOAD] == {"calls": 50, "full_scan_us": 14.35, "mean_scan_us": 14.35, "full_map_us": 16.48,
+                                           "mean_map_us": 23.49}
+    assert len(json.dumps(out)) < 3000
+    assert bench.configs_summary(None) is None
