@@ -1,7 +1,10 @@
 """The map transpose of the blocks from the map, and the scan CTAs that run beside
 it: the channel-mean block and the full block bit for bit against the calls on
-cross-scanned sequences, several times in a row on one stream (the next call's
-transpose follows the last one's readers at once).  Sizes: 16-byte vectors and
+cross-scanned sequences.  The planner's choice three times in a row with new inputs; then
+the gathering scans themselves (the full scan's plans forced: one pass and chunks, one
+and two lanes; many maps, so that the channel-mean scan runs beside the transpose too) on
+the same buffers, call after call with nothing in between, so that the next call's
+transpose follows the last one's readers at once.  Sizes: 16-byte vectors and
 single elements, several planes an item and a ragged last item, the largest
 plane of each form, and planes that fall back to 32 x 32 tiles."""
 import pytest
@@ -48,3 +51,59 @@ def test_blocks_from_the_map_match_cross_scanned_calls(case):
         assert vmb.vmb_read_status() == vmb.VMB_OK
         assert torch.equal(ybar, ybar2) and torch.equal(om, om2)
         assert torch.equal(y, y2) and torch.equal(of, vmb.vmb_cross_merge(y2, H, W))
+
+
+@pytest.mark.parametrize("plan", ["19", "19,4", "23", "23,4"])
+@pytest.mark.parametrize("case", [(6, 72, 20, 24, "f32"), (3, 130, 16, 44, "bf16"), (2, 33, 28, 28, "f32"),
+                                  (1, 40, 96, 96, "f32")], ids=lambda c: "B{}_D{}_{}x{}_{}".format(*c))
+def test_calls_in_a_row_on_the_same_buffers(case, plan, force_plan):
+    B, D, H, W, dt = case
+    force_plan.full(plan)
+    wl = workloads.small_case(B=B, D=D, N=16, H=H, W=W, dtype=dt, seed=D)
+    sets = [workloads.make_device_inputs(wl, DEV, seed=i, params="random") for i in range(4)]
+    want = []
+    for g in sets:
+        args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+        xs = vmb.vmb_cross_scan(g["x"])
+        y = vmb.vmb_selective_scan_fwd(xs, *args, H, W)
+        om, yb = vmb.vmb_mean_scan_merge_fwd(xs, *args, g["x"], H, W)
+        want.append((y, vmb.vmb_cross_merge(y, H, W), om, yb))
+    x, xt = torch.empty_like(sets[0]["x"]), torch.empty(B, D, W, H, dtype=sets[0]["x"].dtype, device=DEV)
+    delta, y = torch.empty_like(sets[0]["draw"]), torch.empty_like(sets[0]["draw"])
+    out, om, yb = torch.empty_like(x), torch.empty_like(x), torch.empty(B, 4, H * W, device=DEV)
+    ws = torch.zeros(32 << 20, dtype=torch.uint8, device=DEV)
+    got = []
+    torch.cuda.synchronize()
+    for rep in range(8):
+        g = sets[rep % 4]
+        x.copy_(g["x"])
+        delta.copy_(g["draw"])
+        args = (delta, g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+        vmb.vmb_ss2d_full_fwd(x, *args, out=out, y=y, xt=xt, workspace=ws)
+        vmb.vmb_ss2d_mean_fwd(x, *args, out=om, ybar=yb, xt=xt, workspace=ws)
+        vmb.vmb_ss2d_full_fwd(x, *args, out=out, y=y, xt=xt, workspace=ws)
+        got.append(tuple(t.clone() for t in (y, out, om, yb)))
+    assert vmb.vmb_read_status(ws) == vmb.VMB_OK
+    for rep, outs in enumerate(got):
+        assert all(torch.equal(a, b) for a, b in zip(outs, want[rep % 4])), rep
+
+
+def test_mean_block_of_many_maps_in_a_row():
+    """Enough CTAs that the channel-mean scan starts beside the transpose by planes."""
+    B, D, H, W = 40, 24, 24, 28
+    wl = workloads.small_case(B=B, D=D, N=16, H=H, W=W, seed=9)
+    sets = [workloads.make_device_inputs(wl, DEV, seed=i, params="random") for i in range(2)]
+    out, yb = torch.empty_like(sets[0]["x"]), torch.empty(B, 4, H * W, device=DEV)
+    xt, got, want = torch.empty(B, D, W, H, device=DEV), [], []
+    for g in sets:
+        args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+        want.append(vmb.vmb_mean_scan_merge_fwd(vmb.vmb_cross_scan(g["x"]), *args, g["x"], H, W))
+    for rep in range(6):
+        g = sets[rep % 2]
+        args = (g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"])
+        for _ in range(3):
+            vmb.vmb_ss2d_mean_fwd(g["x"], *args, out=out, ybar=yb, xt=xt)
+        got.append((out.clone(), yb.clone()))
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    for rep, (o, y) in enumerate(got):
+        assert torch.equal(o, want[rep % 2][0]) and torch.equal(y, want[rep % 2][1])

@@ -146,6 +146,37 @@ def test_tensor_maps_refused(case, force_plan, full_plan):
     check(to_numpy(y_low2), to_numpy(y_low).astype("float64"), dt, "low rank")
 
 
+@pytest.mark.parametrize("case", [
+    # (plan, B, D, N, R, H, W, dtype)
+    ("23", 1, 72, 16, 5, 20, 30, "f32"), ("23", 2, 40, 13, 12, 9, 12, "f32"), ("23,4", 1, 65, 16, 16, 20, 30, "f32"),
+    ("23", 1, 72, 16, 7, 16, 24, "bf16"), ("23,3", 2, 33, 9, 11, 20, 30, "bf16"),
+    ("3", 1, 72, 8, 5, 20, 30, "f32"), ("3,4", 1, 72, 5, 9, 20, 30, "f32"), ("1,4", 1, 130, 2, 3, 20, 30, "f32"),
+    ("2", 1, 40, 8, 16, 16, 24, "bf16"), ("1,5", 2, 40, 4, 6, 20, 30, "bf16"),
+], ids=lambda c: "plan{}_B{}_D{}_N{}_R{}_{}x{}_{}".format(*c))
+def test_lowrank_forms(case, force_plan):
+    """The low-rank Delta with two lanes per channel and in chunks, and, for 8 states or
+    fewer, expanded into y and scanned in place: against the scan of the materialised
+    raw Deltas with the same plan (bit for bit in fp32, and in bf16 in place)."""
+    plan, B, D, N, R, H, W, dt = case
+    force_plan.full(plan)
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=700 + D + R)
+    g = to_device(workloads.make_inputs(wl, params="random"), DEV)
+    xs = vmb.vmb_cross_scan(g["x"])
+    gen = torch.Generator(device=DEV).manual_seed(R)
+    z = torch.randn(B, 4, R, H * W, device=DEV, generator=gen)
+    wup = 0.3 * torch.randn(4, D, R, device=DEV, generator=gen)
+    y = vmb.vmb_selective_scan_lowrank_fwd(xs, z, wup, g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W)
+    raw = torch.zeros(B, 4, D, H * W, device=DEV, dtype=torch.float64)
+    for r in range(R):  # in the kernel's order, every fused multiply-add rounded to fp32
+        raw = (raw + wup[None, :, :, r, None].double() * z[:, :, None, r].double()).float().double()
+    y2 = vmb.vmb_selective_scan_fwd(xs, raw.to(xs.dtype), g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W)
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    if dt == "f32" or N <= 8:
+        assert torch.equal(y, y2)
+    else:
+        check(to_numpy(y), to_numpy(y2).astype("float64"), dt, "low rank")
+
+
 @pytest.mark.parametrize("off", [0, 1])
 @pytest.mark.parametrize("case", [
     # (B, K, D, N, L, dtype): narrow tiles, whole tiles and one row more, stages cut short
