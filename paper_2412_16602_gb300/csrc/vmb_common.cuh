@@ -47,10 +47,11 @@ __device__ __forceinline__ float rcp(float x) {
 // z = e / (2 + e) <= 1/3 (Abramowitz & Stegun 4.1.27), = z P(z^2) with P the
 // degree-4 minimax polynomial of 2 atanh(z)/z in relative error over z^2 in
 // [0, 1/9] (Remez exchange in 40-digit arithmetic: largest relative error
-// 4.0e-9, below half an ulp; the series truncated after z^12/13 that it replaced
-// had 1.4e-8 and two more terms), so the result keeps the relative accuracy of
+// 4.0e-9, with the coefficients rounded to fp32, as used, 7.8e-9, below half an ulp;
+// the series truncated after z^12/13 that it replaced had 1.4e-8 and two more
+// terms), so the result keeps the relative accuracy of
 // e^-|v| even where log1p(e) is tiny.  No cut-off for large |v|.
-constexpr float kSp0 = 2.00000000792f, kSp1 = 0.666663146851f, kSp2 = 0.400249102072f, kSp3 = 0.279606031296f,
+constexpr float kSp0 = 2.0f, kSp1 = 0.666663146851f, kSp2 = 0.400249102072f, kSp3 = 0.279606031296f,
                 kSp4 = 0.281783355047f;
 __device__ __forceinline__ float softplus_from_e(float v, float e) {
     const float z = e * rcp(2.0f + e);
@@ -95,14 +96,23 @@ __device__ __forceinline__ float2 softplus2(float2 v) { return softplus2_from_e(
 
 // Every kernel of libvmb is launched with programmatic stream serialization,
 // so that its CTAs can be scheduled while the previous kernel of the stream
-// drains.  Each kernel therefore executes pdl_wait() (griddepcontrol.wait:
-// the previous kernel has completed and its writes are visible) before it
-// touches global memory, and only then pdl_launch_dependents(), which lets
-// the next kernel be scheduled.  Because no kernel signals its dependents
-// before its own wait has returned, a kernel that is already running may
-// read data written two or more launches earlier before its own wait (the
-// third launch of the chunked full scan does so).  Both instructions are
-// no-ops in a kernel launched without the attribute.
+// drains.  pdl_wait() (griddepcontrol.wait) returns when the previous kernel has
+// completed and its writes are visible; pdl_launch_dependents() lets the next
+// kernel be scheduled once every CTA of the grid has executed it or exited.
+// What every kernel keeps to:
+//  - some CTA of the grid executes pdl_wait() before it signals, so the dependents
+//    are never released before the previous kernel has completed;
+//  - a warp that has not waited touches only data that was complete before the
+//    previous kernel passed its own wait, and writes only what the previous kernel
+//    does not touch.
+// Nearly all kernels wait at once and signal then.  The third launch of the chunked
+// full scan and the producers of the second launch of the warp-specialised one
+// read their inputs, written two or more launches earlier, before they wait.  In
+// the scans that gather from the map the CTAs of directions 0 and 2 never wait (they
+// read x, B, C and Delta and write y and the workspace, none of which the
+// transpose before them touches), those of directions 1 and 3 wait before they
+// signal: this holds only while the launch right before is the map transpose.
+// Both instructions are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
