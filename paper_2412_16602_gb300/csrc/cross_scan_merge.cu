@@ -21,17 +21,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr size_t kMaxSmem = 200 * 1024;
 
-struct FastDiv {
-    unsigned d, m, s;
-};
-FastDiv make_fastdiv(unsigned d) {
-    unsigned s = 0;
-    while ((1ull << s) < d) ++s;
-    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
-    return {d, (unsigned)m, s};
-}
-__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
-
 struct CsmParams {
     const void* in;
     void* out;

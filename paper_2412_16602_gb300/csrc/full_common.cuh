@@ -57,13 +57,6 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4]) {
     v[3] = __uint_as_float(q.y & 0xffff0000u);
 }
 
-// Two consecutive elements as fp32 (8-byte / 4-byte aligned reads).
-__device__ __forceinline__ float2 load2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-__device__ __forceinline__ float2 load2(const __nv_bfloat16* p) {
-    const unsigned q = *reinterpret_cast<const unsigned*>(p);
-    return make_float2(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
-}
-
 // Store n consecutive outputs of one row (n = 4, 2 or 1), vectorised when aligned.
 template <typename T, int NV>
 __device__ __forceinline__ void store_row(T* dst, const float (&v)[NV], int nvalid_here, bool vec) {

@@ -312,7 +312,6 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
         auto at = [&](const unsigned char* b, int t) {  // address of step t (a multiple of 4) of this channel's row
             return reinterpret_cast<const T*>(b + LY::piece(c, t / E)) + t % E;
         };
-        const auto& at2 = at;  // t even: the two steps of a pair lie in one piece
 #pragma unroll
         for (int j = 0; j < ST; j += 4) {
             float q[4];
@@ -329,20 +328,15 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
         }
         // this lane's steps: t0 + g ST / G .. t0 + (g + 1) ST / G - 1
         constexpr int SPL = ST / G;
+        static_assert(SPL % 4 == 0, "steps per lane: whole reads of four");
         float own[SPL];
         if constexpr (WS::RP == 0) {
 #pragma unroll
-            for (int j = 0; j < SPL; j += SPL < 4 ? 2 : 4) {
-                if constexpr (SPL < 4) {
-                    const float2 w = load2(at2(rd, t0 + g * SPL + j));
-                    own[j] = w.x + bias;
-                    own[j + 1] = w.y + bias;
-                } else {
-                    float w[4];
-                    load4(at(rd, t0 + g * SPL + j), w);
+            for (int j = 0; j < SPL; j += 4) {
+                float w[4];
+                load4(at(rd, t0 + g * SPL + j), w);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) own[j + e] = w[e] + bias;
-                }
+                for (int e = 0; e < 4; ++e) own[j + e] = w[e] + bias;
             }
         } else {
             // raw Delta = sum_r Wup[r] z_r, r in order (the z rows are broadcast reads)
@@ -449,7 +443,7 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
             }
         } else {
             // lane g keeps its half of the steps
-            constexpr int SPL = ST / 2, V = SPL < 4 ? 2 : 4;
+            constexpr int SPL = ST / 2;
             float o[SPL];
 #pragma unroll
             for (int j = 0; j < SPL; ++j) {
@@ -459,11 +453,9 @@ __global__ void __launch_bounds__(WsTileLayout<T, WS>::THREADS, WS::MINB)
             }
             if (!cval) return;
 #pragma unroll
-            for (int j = 0; j < SPL; j += V) {
-                float q[V];
-#pragma unroll
-                for (int e = 0; e < V; ++e) q[e] = o[j + e];
-                store_row<T, V>(yrow + l0 + g * SPL + j, q, nvalid - g * SPL - j, true);
+            for (int j = 0; j < SPL; j += 4) {
+                const float q[4] = {o[j], o[j + 1], o[j + 2], o[j + 3]};
+                store_row<T, 4>(yrow + l0 + g * SPL + j, q, nvalid - g * SPL - j, true);
             }
         }
     };

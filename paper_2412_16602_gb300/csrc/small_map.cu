@@ -33,20 +33,6 @@ constexpr int kSmThreads = 128;  // four warps
 constexpr int kNP = 16;          // states, zero padded
 constexpr int kBC = 2 * kNP;     // floats of one step's B and C
 
-// Division by an invariant integer by multiply-high (Granlund & Montgomery,
-// "Division by invariant integers using multiplication", PLDI 1994), for
-// dividends below 2^31.
-struct FastDiv {
-    unsigned d, m, s;
-};
-FastDiv make_fastdiv(unsigned d) {
-    unsigned s = 0;
-    while ((1ull << s) < d) ++s;
-    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
-    return {d, (unsigned)m, s};
-}
-__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
-
 struct SmallParams {
     const void* u;  // [B][K][D][L], or (MAP) the map x [B][D][L]
     const void* dl;
@@ -66,10 +52,7 @@ struct SmallParams {
     FastDiv fL, fW;
 };
 
-__device__ __forceinline__ void load_elem(float* dst, const float* src) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(src) : "memory");
-}
+__device__ __forceinline__ void load_elem(float* dst, const float* src) { cp_async4(dst, src, 4); }
 __device__ __forceinline__ void load_elem(float* dst, const __nv_bfloat16* src) { *dst = __bfloat162float(*src); }
 
 // `rows` consecutive rows of L elements into rows of stride RX, by `step`

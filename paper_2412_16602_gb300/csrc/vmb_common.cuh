@@ -92,6 +92,21 @@ __device__ __forceinline__ float2 softplus2_from_e(float2 v, float2 e) {
 }
 __device__ __forceinline__ float2 softplus2(float2 v) { return softplus2_from_e(v, softplus2_e(v)); }
 
+// ------------------------------------------- division by invariant integers
+
+// By multiply-high (Granlund & Montgomery, "Division by invariant integers using
+// multiplication", PLDI 1994, round-up variant), valid for dividends below 2^31.
+struct FastDiv {
+    unsigned d, m, s;
+};
+inline FastDiv make_fastdiv(unsigned d) {
+    unsigned s = 0;
+    while ((1ull << s) < d) ++s;
+    const unsigned long long m = ((1ull << 32) * ((1ull << s) - d)) / d + 1;
+    return {d, (unsigned)m, s};
+}
+__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv f) { return (__umulhi(n, f.m) + n) >> f.s; }
+
 // ------------------------------------------- programmatic dependent launch
 
 // Every kernel of libvmb is launched with programmatic stream serialization,
