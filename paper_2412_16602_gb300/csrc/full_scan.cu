@@ -83,14 +83,13 @@ __device__ __forceinline__ float sel4(const float (&v)[4], int j) {
 template <typename T, int NP, int DT, int kTS, int RS, int kThreads, bool WITH_C, bool WITH_B>
 __device__ __forceinline__ void load_tile_elements(const FullParams& p, T* dst, size_t row0, size_t bcrow0, int nrows,
                                                    int l0) {
-    // element by element: thread i copies step i % kTS of rows i / kTS + k RPP, u and
-    // delta (B and C) together; fp32 as 4-byte asynchronous copies, in flight like
+    // element by element: thread i copies step i % kTS of rows i / kTS + k RPP, u, delta, B
+    // and C in turn; fp32 as 4-byte asynchronous copies, in flight like
     // the 16-byte ones, bf16 (2-byte elements) through registers, a batch of
     // independent loads at a time.  Only rows of the problem are visited: rows of u
     // and delta past nrows keep what they held (the lanes that read them store
-    // nothing), those of B and C past N are zeroed (GB300, bf16, unaligned rows, us:
-    // 21 maps of 38x51x3, two states, 243 visiting every row of the tile, see the
-    // test of narrow tiles).
+    // nothing), those of B and C past N are zeroed (GB300, bf16, unaligned rows, 21 maps
+    // of 38x51x3, two states: 82 us, 243 visiting every row of the tile).
     constexpr int RPP = kThreads / kTS;
     static_assert(kThreads % kTS == 0, "tile loader mapping");
     const int t = threadIdx.x % kTS, r0 = threadIdx.x / kTS;
@@ -1812,7 +1811,7 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // kernel 7.0, 19456 rows of 28x28 46 and 73, 30464 rows 81 and 77), L cut into
     // chunks where ws_estimate expects a gain (6144 rows of 128x128 bf16 605, one
     // pass 1126, look-back chunks 870; 3072 rows of 56x56 80, look-back 187; one state, 131072 rows
-    // of 56x56 779, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
+    // of 56x56 796, the barrier-staged kernel 1349).  Below six rows per SM with 16 states
     // the three-launch chunked variant while a grid of 64-step one-lane chunks
     // fits in two waves (768 rows of 56x56 30.2, chunked warp-specialised 34.8; at 1536
     // rows 56.9 and 46.6), just past the short sequences (up to 320 steps) and up to 16 rows per SM
