@@ -1892,15 +1892,13 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         const ShapeRoles r = roles(np);
         if ((st = info(r.wide, &ki, &res)) != VMB_OK) return st;
         shape = r.wide;
-        KernelInfo kl{};
-        long long rl = 0;
         if (np == 16 && a.L <= 1024 && rows * 4 < res * ki.threads * 3) {
-            // short sequences with few rows: one lane per state, single pass
-            if ((st = info(kLanesShape, &kl, &rl)) != VMB_OK) return st;
-            if (rows * 16 <= rl * kl.threads) {
+            // short sequences with few rows: one lane per state, single pass, up to four
+            // CTAs of 16 rows per SM (three are resident; 60 rows per SM of 203 unaligned
+            // steps, 71 maps of 7x29x32: 30.3 us, look-back chunks 77)
+            if (rows <= 64LL * sms) {
                 shape = kLanesShape;
-                ki = kl;
-                res = rl;
+                if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
             }
         }
         if (shape != kLanesShape && rows * 4 < res * ki.threads * 3) {

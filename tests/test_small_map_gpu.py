@@ -79,6 +79,8 @@ LANES, FOUR, SIXTEEN = 7, 21, 22
     ((2, 32, 2, 4, "f32"), SIXTEEN, SIXTEEN), ((36, 32, 5, 8, "f32"), FOUR, FOUR), ((36, 32, 8, 12, "f32"), FOUR, LANES),
     ((1, 40, 10, 10, "f32"), SIXTEEN, SIXTEEN), ((3, 64, 16, 18, "f32"), LANES, LANES),
     ((30, 64, 16, 18, "f32"), 23, 23), ((60, 32, 8, 12, "f32"), FOUR, FOUR), ((60, 32, 8, 10, "bf16"), FOUR, LANES),
+    # rows out of line, up to four CTAs of the lane-per-state kernel per SM
+    ((71, 32, 7, 29, "f32"), LANES, LANES), ((44, 32, 13, 23, "bf16"), LANES, LANES),
 ])
 def test_planner_of_short_sequences(case, map_shape, scan_shape, full_plan):
     B, D, H, W, dt = case
