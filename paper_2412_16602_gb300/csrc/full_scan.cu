@@ -1836,11 +1836,22 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // then runs as two lanes per channel over 32-step chunks, which measured fastest
     // with the launches chained (stage-1 maps at batch 1 to 3: 5 to 6% shorter
     // steps than the 64-step chunks)
-    auto chunk_grid_fits = [&]() -> bool {
+    // CTAs of the three-launch variant as 64-step one-lane chunks; -1 past two waves
+    auto chunk_ctas = [&]() -> long long {
         KernelInfo kc{};
         long long rc = 0;
-        if (info(kChunkShape + 2, &kc, &rc) != VMB_OK) return false;
-        return a.B * a.K * (long long)((a.D + kc.DT - 1) / kc.DT) * ((a.L + kc.ts - 1) / kc.ts) <= 2 * rc;
+        if (info(kChunkShape + 2, &kc, &rc) != VMB_OK) return -1;
+        const long long n = a.B * a.K * (long long)((a.D + kc.DT - 1) / kc.DT) * ((a.L + kc.ts - 1) / kc.ts);
+        return n <= 2 * rc ? n : -1;
+    };
+    auto chunk_grid_fits = [&]() -> bool { return chunk_ctas() >= 0; };
+    // Up to 1024 steps the lane-per-state kernel takes 3.2 us and 33.5 ns a step whatever the
+    // rows (few enough), the three launches about 8 us and 42 ns a CTA on 152 SMs, and their
+    // tiles of 64 channels are mostly padding where a sequence has few (fp32, us: 19 maps
+    // of 20x20x7 16.2 and 29.0; 7 of 32x32x32 37.2 and 25.5)
+    auto chunk_beats_lanes = [&]() -> bool {
+        const long long n = chunk_ctas();
+        return n >= 0 && (a.L > 1024 || 15200 * n <= (86LL * a.L - 20000) * sms);
     };
     int shape = 0, n_chunks = 1, forced_chunks = 0, forced_shape = 0;
     KernelInfo ki{};
@@ -1866,7 +1877,8 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
         } else {
             shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);
         }
-    } else if (np == 16 && seq_ok && a.L > 256 && a.L <= 320 && rows <= 16LL * sms) {
+    } else if (np == 16 && seq_ok && a.L > 256 &&
+               (a.L <= 320 ? rows <= 16LL * sms : a.L <= 1024 && rows < 6LL * sms && !chunk_beats_lanes())) {
         shape = kLanesShape;
         if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
     } else if (np == 16 && tma_ok && rows < 6LL * sms && chunk_grid_fits()) {

@@ -81,6 +81,8 @@ LANES, FOUR, SIXTEEN = 7, 21, 22
     ((30, 64, 16, 18, "f32"), 23, 23), ((60, 32, 8, 12, "f32"), FOUR, FOUR), ((60, 32, 8, 10, "bf16"), FOUR, LANES),
     # rows out of line, up to four CTAs of the lane-per-state kernel per SM
     ((71, 32, 7, 29, "f32"), LANES, LANES), ((44, 32, 13, 23, "bf16"), LANES, LANES),
+    # few channels per sequence: tiles of the chunked three launches would be mostly padding
+    ((19, 7, 20, 20, "f32"), LANES, LANES), ((7, 32, 20, 20, "bf16"), LANES, LANES), ((7, 32, 32, 32, "f32"), 9, 9),
 ])
 def test_planner_of_short_sequences(case, map_shape, scan_shape, full_plan):
     B, D, H, W, dt = case
