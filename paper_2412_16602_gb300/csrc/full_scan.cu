@@ -1748,19 +1748,36 @@ int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
     if (!seq_ok) return 1;
     return map && small_map_one_lane(a.L) ? 1 : 0;
 }
-// Short sequences alone, in rows that the barrier-staged kernels copy 16 bytes at a time: the
-// lane-per-state kernel instead of 4 or 16 lanes of whole sequences.  It streams stages of 32
-// steps, so a length just past one pays for the next; the whole-sequence kernel's loads of
-// 2-byte elements wait.  us, lane-per-state and whole sequences, fp32: 5 rows per SM of 96 steps 5.0 and
+// Short sequences alone: the lane-per-state kernel instead of 4 or 16 lanes of whole
+// sequences.  It streams stages of 32 steps, so a length just past one pays for the next; the
+// whole-sequence kernel's loads of 2-byte elements wait.  us, lane-per-state and whole sequences.
+// Rows copied 16 bytes at a time (`seq_ok`), fp32: 5 rows per SM of 96 steps 5.0 and
 // 5.4, of 100 6.1 and 5.6; 10 of 224 steps 9.5 and 20.2, 22 of 64 steps 5.1 and 7.4; 30 of 40 steps
 // 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
-// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.
-bool lanes_beat_small(int L, long long rows, vmb_dtype dt, int sms) {
-    const int staged = (L + 31) / 32 * 32;
-    if (dt == VMB_BF16) return L >= 16;
+// 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.  Element by element (rows counted with the
+// padding to CTAs of 16 channels), fp32: 5 rows per SM of 143 steps 8.5 and 7.1; 10 of 143 8.6 and
+// 10.0, of 203 11.4 and 18.7; 20 of 35 steps 5.9 and 5.2, of 203 16.1 and 18.7; 46 of 203 21.4 and 18.9.
+// bf16: 5 of 143 steps 8.7 and 10.9, 20 of 203 15.4 and 31.0, 46 20.3 and 29.9; 60 of 35 9.5 and 8.2.
+bool lanes_beat_small(const ScanArgs& a, bool seq_ok, int sms) {
+    const int L = a.L, staged = (L + 31) / 32 * 32;
+    if (!seq_ok) {
+        const long long rows = (long long)a.B * a.K * ((a.D + 15) / 16 * 16);
+        if (a.dtype == VMB_BF16) return L >= 16 && rows <= 48LL * sms;
+        return rows > 8LL * sms && rows <= 24LL * sms && L >= 16 && 8 * staged <= 13 * L;
+    }
+    const long long rows = (long long)a.B * a.K * a.D;
+    if (a.dtype == VMB_BF16) return L >= 16;
     if (rows <= 6LL * sms) return 16 * staged <= 17 * L;
     if (rows <= 24LL * sms) return L >= 16;
     return rows <= 48LL * sms && (L >= 64 || 8 * staged <= 9 * L);
+}
+
+// bf16 rows read element by element, alone and in many waves: the packed streaming kernel, whose
+// loads overlap with the scan, instead of whole sequences with one lane (1000 rows per SM, us:
+// 81 steps 166 and 207, 101 200 and 344; 250 rows per SM of 101 steps 71 and 60; fp32 the
+// other way, 191 and 182).
+bool packed_beats_small(const ScanArgs& a, int sms) {
+    return a.dtype == VMB_BF16 && a.L >= 72 && (long long)a.B * a.K * a.D >= 512LL * sms;
 }
 
 // Estimated time (ns) of the warp-specialised kernel, and the number of chunks
@@ -1871,8 +1888,11 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
             n_chunks = (int)(want < mx ? want : mx);
         }
     } else if (const int G = np == 16 ? small_rule(a, map, seq_ok, sms) : 0) {
-        if (!map && seq_ok && G > 1 && lanes_beat_small(a.L, rows, a.dtype, sms)) {
+        if (!map && G > 1 && lanes_beat_small(a, seq_ok, sms)) {
             shape = kLanesShape;
+            if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
+        } else if (!map && !seq_ok && packed_beats_small(a, sms)) {
+            shape = kPackedShape;
             if ((st = info(shape, &ki, &res)) != VMB_OK) return st;
         } else {
             shape = kSmallShape + (G == 16 ? 2 : G == 4 ? 1 : 0);

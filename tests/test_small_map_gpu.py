@@ -70,7 +70,24 @@ def test_whole_sequences_and_lane_per_state_agree_bit_for_bit(shape, force_plan)
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
 
 
-LANES, FOUR, SIXTEEN = 7, 21, 22
+@pytest.mark.parametrize("shape", [(3, 70, 16, 9, 9, "bf16"), (2, 130, 9, 7, 11, "bf16"), (1, 40, 13, 5, 15, "f32")],
+                         ids=lambda s: "B{}_D{}_N{}_{}x{}_{}".format(*s))
+def test_whole_sequences_and_packed_agree_bit_for_bit(shape, force_plan):
+    """One lane of whole sequences (the block) and the packed streaming kernel (shape 16),
+    which the scan alone may take instead, on rows out of line."""
+    B, D, N, H, W, dt = shape
+    wl = workloads.small_case(B=B, D=D, N=N, H=H, W=W, dtype=dt, seed=320 + D)
+    g = to_device(workloads.make_inputs(wl, params="random"), DEV)
+    args = (vmb.vmb_cross_scan(g["x"]), g["draw"], g["A"], g["Bs"], g["Cs"], g["Dskip"], g["bias"], H, W)
+    ys = []
+    for plan in ("16", "20"):
+        force_plan.full(plan)
+        ys.append(vmb.vmb_selective_scan_fwd(*args))
+    assert vmb.vmb_read_status() == vmb.VMB_OK
+    assert torch.equal(ys[0], ys[1])
+
+
+LANES, PACKED, ONE, FOUR, SIXTEEN = 7, 16, 20, 21, 22
 
 
 @pytest.mark.parametrize("case,map_shape,scan_shape", [
@@ -83,6 +100,9 @@ LANES, FOUR, SIXTEEN = 7, 21, 22
     ((71, 32, 7, 29, "f32"), LANES, LANES), ((44, 32, 13, 23, "bf16"), LANES, LANES),
     # few channels per sequence: tiles of the chunked three launches would be mostly padding
     ((19, 7, 20, 20, "f32"), LANES, LANES), ((7, 32, 20, 20, "bf16"), LANES, LANES), ((7, 32, 32, 32, "f32"), 9, 9),
+    # the scan alone, rows out of line
+    ((16, 32, 7, 29, "bf16"), FOUR, LANES), ((16, 32, 7, 29, "f32"), FOUR, LANES), ((110, 7, 7, 29, "f32"), FOUR, FOUR),
+    ((49, 400, 9, 9, "bf16"), ONE, PACKED), ((49, 400, 9, 9, "f32"), ONE, ONE), ((40, 400, 9, 9, "bf16"), ONE, ONE),
 ])
 def test_planner_of_short_sequences(case, map_shape, scan_shape, full_plan):
     B, D, H, W, dt = case
