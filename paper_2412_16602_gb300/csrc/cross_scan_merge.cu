@@ -430,17 +430,19 @@ __global__ void cross_merge_direct(const T* ys, T* out, int D, int H, int W, lon
 
 // Kernel of a cross-scan or cross-merge.  Below 1024 pixels whole planes are staged
 // with index tables.  From there on bands of rows, or, where a row is too long for a band,
-// whole planes with their indices computed, if there is a plane for every SM and whole vectors
-// can be copied (scanning fp32, also single elements of planes that leave room for two); and where neither fits, or a plane takes more
+// whole planes with their indices computed (merges: if there is a plane for every SM and whole
+// vectors can be copied; scans: for an eighth as many, or half as many element by element, as
+// the gather reads every element four times); and where neither fits, or a plane takes more
 // than kMaxSmem of staging (counted as two storage-type planes for the merge), bands only
 // where enough of them share an SM, else the gather of single elements.  GB300, us,
-// planes x H x W: scan 192x1x9000 fp32 staged 7.3, gather 34; 192x8x6000 72 and 170; out of
-// line 192x15x2999 187 and 160, 32x3x3297 34 and 13, 216x3x6803 32 and 62;
+// planes x H x W: scan, staged and gather, 40x1x9000 fp32 5.3 and 10.6, 16x1x9000 5.3 and 5.5,
+// 40x12x3760 18.6 and 35, 192x8x6000 72 and 170; out of line 80x3x7001 bf16 22 and 33, 80x9x5001 fp32 45 and 66,
+// 152x7x7743 bf16 54 and 145, 152x9x5001 99 and 125;
 // merge 192x2x8000 12 and 18, 16x2x8000 8.7 and 3.9, 192x4x6000 (117 KB staged) 41 and 29.  Merge in bands and
 // gather: 192x256x256 fp32 (64 KB a band) 92 and 104, bf16 30 and 102; 192x64x800 fp32
 // (100 KB) 99 and 80; 16x512x512 fp32 (128 KB) 60 and 36; rows out of line 192x201x201 fp32
 // (50 KB) 127 and 61, 16x401x399 bf16 (25 KB) 17 and 22, 192x7001x12 bf16 166 and 91.
-// Scan 192x15x2999 fp32 out of line (94 KB) 188 and 160, 192x61x997 (31 KB) 123 and 219.
+// Scan in bands and gather 192x15x2999 fp32 out of line (94 KB) 188 and 160, 192x61x997 (31 KB) 123 and 219.
 CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, bool aligned, int sms) {
     const long long L = (long long)H * W, es = dt == VMB_BF16 ? 2 : 4;
     if (planes >= (1ll << 31) || L * 4 >= (1ll << 31)) return CsmKernel::kGather;
@@ -450,7 +452,8 @@ CsmKernel csm_kernel(bool merge, vmb_dtype dt, long long planes, int H, int W, b
     const long long staged = merge ? 2ll * W * (H + 1) * es : (long long)H * (W + 1) * es;
     if (!band_fits) {
         const bool vec = aligned && L * es % 16 == 0;
-        const bool whole = staged <= (vec ? (long long)kMaxSmem : !merge && es == 4 ? 96 * 1024 : 0) && planes >= sms;
+        const bool whole = staged <= (long long)kMaxSmem &&
+                           (merge ? vec && planes >= sms : vec ? 8 * planes >= sms : 2 * planes >= sms);
         return whole ? CsmKernel::kPlane : CsmKernel::kGather;
     }
     if (staged <= (long long)kMaxSmem) return CsmKernel::kBand;

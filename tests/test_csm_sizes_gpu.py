@@ -18,7 +18,9 @@ CASES = [(1, 1, 1, 1), (2, 3, 1, 9), (3, 2, 31, 33), (1, 3, 33, 31), (2, 2, 1, 1
          (5, 130, 3, 5), (1, 2, 230, 232), (1, 1, 3, 3300),
          # long rows and tall planes: whole planes without index tables, bands, single elements
          (1, 3, 1, 9000), (2, 2, 7, 3201), (1, 2, 2, 8001), (1, 2, 3, 8793), (1, 1, 201, 201), (1, 2, 14, 1948),
-         (1, 1, 300, 256), (1, 1, 7001, 12), (1, 1, 128, 800)]
+         (1, 1, 300, 256), (1, 1, 7001, 12), (1, 1, 128, 800),
+         # enough planes of long rows: whole planes, in line and not
+         (2, 10, 1, 9000), (1, 80, 3, 6401), (2, 40, 7, 6999), (2, 80, 2, 7000), (1, 160, 1, 6403)]
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])

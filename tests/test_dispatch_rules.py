@@ -26,8 +26,8 @@ def lib():
     (0, F32, 32, 32, 1, BAND), (1, F32, 56, 56, 1, BAND),
     # rows too long for a band: whole planes while they fit shared memory
     (0, F32, 1, 9000, 1, PLANE), (0, F32, 8, 6000, 1, PLANE), (1, F32, 2, 8000, 1, PLANE), (0, BF16, 8, 8793, 1, PLANE),
-    (0, F32, 8, 6000, 0, GATHER), (0, F32, 7, 6418, 1, GATHER), (0, F32, 3, 6803, 1, PLANE), (1, F32, 3, 3297, 1, GATHER),
-    (0, BF16, 3, 8349, 1, GATHER),
+    (0, F32, 8, 6000, 0, PLANE), (0, F32, 7, 6418, 1, PLANE), (0, F32, 3, 6803, 1, PLANE), (1, F32, 3, 3297, 1, GATHER),
+    (0, BF16, 3, 8349, 1, PLANE), (0, F32, 9, 6000, 1, GATHER), (1, F32, 1, 9001, 1, GATHER),
     (0, F32, 16, 4000, 1, GATHER), (1, F32, 4, 6000, 1, GATHER), (1, BF16, 16, 7000, 1, GATHER),
     # planes larger than shared memory: bands where several share an SM
     (1, F32, 256, 256, 1, BAND), (1, F32, 64, 800, 1, GATHER), (1, F32, 512, 512, 1, GATHER),
@@ -43,6 +43,9 @@ def test_csm_kernel_of_few_planes(lib):
     assert lib.vmb_testing_csm_kernel(1, F32, 16, 2, 8000, 1, SMS) == GATHER
     assert lib.vmb_testing_csm_kernel(0, F32, 6, 4, 7336, 1, SMS) == GATHER
     assert lib.vmb_testing_csm_kernel(0, F32, 32, 3, 3297, 1, SMS) == GATHER
+    assert lib.vmb_testing_csm_kernel(0, F32, 76, 3, 3297, 1, SMS) == PLANE
+    assert lib.vmb_testing_csm_kernel(0, F32, 19, 4, 4096, 1, SMS) == PLANE
+    assert lib.vmb_testing_csm_kernel(0, F32, 18, 4, 4096, 1, SMS) == GATHER
     assert lib.vmb_testing_csm_kernel(1, BF16, 16, 7001, 12, 1, SMS) == BAND
 
 
