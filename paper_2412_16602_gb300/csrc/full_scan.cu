@@ -1797,8 +1797,9 @@ double ws_estimate(int np, bool two, long long tiles, int L, int sms, int ts, in
         const long long per_sm = (tiles * P + sms - 1) / sms;
         const long long waves = (per_sm + 2) / 3;
         const double step = c[per_sm > 2 ? 2 : per_sm - 1] * waves;
-        // two launches, and the second one folds up to P - 1 aggregates
-        const double t = P == 1 ? L * step : 2.0 * L / (P + 1) * step + 6000.0 + 300.0 * P;
+        // two launches, and the second one folds up to P - 1 aggregates (8 states, 4 batches of
+        // 192 channels, 288 steps: 13.9 us in one pass, 10.9 in four chunks)
+        const double t = P == 1 ? L * step : 2.0 * L / (P + 1) * step + (np == 8 ? 2500.0 : 6000.0) + 300.0 * P;
         if (P == 1 || t < best) {
             best = t;
             *chunks = P == 1 ? 1 : P + 1;

@@ -95,6 +95,13 @@ def test_planner_of_eight_states(case, shape, full_plan):
     assert full_plan(B, 4, D, N, H, W, dt, map=True)[0] == shape
 
 
+@pytest.mark.parametrize("case,chunks", [((4, 192, 8, 16, 18, "f32"), 4), ((8, 192, 8, 16, 18, "bf16"), 1),
+                                         ((4, 192, 8, 8, 16, "f32"), 1)])
+def test_planner_cuts_eight_states_into_chunks(case, chunks, full_plan):
+    B, D, N, H, W, dt = case
+    assert full_plan(B, 4, D, N, H, W, dt)[:2] == (3, chunks)
+
+
 @pytest.mark.parametrize("case,early", [
     # (B, D, N, H, W, dtype, off, flags beyond softplus): barrier-staged plans; a grid of less than one wave
     # of long-lived CTAs is not launched early, tiny sequences and full waves are
