@@ -890,6 +890,10 @@ bool transpose_by_planes(const void* x, const void* xt, int H, int W, vmb_dtype 
            (size_t)W * transpose_stride(H, VE, vec) * es <= kTrSmem;
 }
 
+bool transpose_whole_vectors(const void* x, const void* xt, int H, int W, vmb_dtype dt) {
+    return transpose_vec(x, xt, H, W, dt == VMB_BF16 ? 2 : 4);
+}
+
 vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, bool planes,
                                 cudaStream_t stream) {
     if (planes)

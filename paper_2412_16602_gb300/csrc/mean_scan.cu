@@ -941,14 +941,21 @@ bool mean_two_steps(long long n, int D, long long res1, long long res2, int sms,
 // fp32 out of line 58, after the transpose by tiles 47; one of 88x16x1536 54 and 45).  Planes that
 // leave most of a tile empty, maps of less than 2.5 MB and more than 8192 tiles are not cut into
 // tiles all the same (1 map of 10x10x1536 62 us by planes, 85 by tiles; of 24x24x768 23.8 and 25.8; 16
-// of 28x20x576 57 and 61).
+// of 28x20x576 57 and 61).  Nor, while every CTA has an SM of its own, with 16 states (fp32, 1 map of
+// 32x32x1536 70 by planes, 89 by tiles, of 28x20x1536 54 and 87, in line or not), up to 1024 channels (8 states,
+// 32x32x1024 39 and 45; 32x32x1536 with four 42 and 34) or with 8 states in bf16 (32x32x1536 55 and 66);
+// nor, in line, from two CTAs per SM on (1 map of 48x72x1024 fp32 49 and 54, 2 of 88x16x577 bf16 35 and 39;
+// out of line 4 of 56x56x192 44 and 41).
 bool mean_beside_transpose(const ScanArgs& a, const ScanPlan& plan, int H, int W) {
     if (!transpose_by_planes(a.u, a.u_t, H, W, a.dtype)) return false;
     const long long tiles = (long long)a.B * a.D * ((H + 31) / 32) * ((W + 31) / 32);
     const long long pixels = (long long)a.B * a.D * H * W;
     if (tiles > 8192 || 20 * pixels < 9 * 1024 * tiles || pixels * (a.dtype == VMB_BF16 ? 2 : 4) < 2500000) return true;
+    const long long grid = (long long)plan.n_seq * plan.n_chunks, sms = device_sm_count();
+    if (grid <= sms && (plan.np == 16 || a.D <= 1024 || (plan.np == 8 && a.dtype == VMB_BF16))) return true;
+    if (grid > 2 * sms && transpose_whole_vectors(a.u, a.u_t, H, W, a.dtype)) return true;
     const KInfo ki = mpick(a.dtype, plan.np, plan.chunk_len, (a.flags & VMB_FLAG_B_ZOH) != 0, false);
-    return ki.fn && (long long)plan.n_seq * plan.n_chunks >= resident_ctas(ki.fn, ki.threads, ki.smem);
+    return ki.fn && grid >= resident_ctas(ki.fn, ki.threads, ki.smem);
 }
 
 vmb_status plan_mean(const ScanArgs& a, ScanPlan* plan) {

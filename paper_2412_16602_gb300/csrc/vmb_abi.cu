@@ -728,6 +728,22 @@ int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned fla
     return s;
 }
 
+int vmb_testing_mean_beside(int B, int D, int N, int H, int W, vmb_dtype dtype, int off) {
+    ScanArgs a{};
+    a.B = B;
+    a.K = 4;
+    a.D = D;
+    a.N = N;
+    a.L = H * W;
+    a.dtype = dtype;
+    alignas(16) static const float dummy[8] = {};
+    a.u = reinterpret_cast<const char*>(dummy) + (off ? esize(dtype) : 0);
+    a.u_t = dummy;
+    a.gather_h = H;
+    ScanPlan plan{};
+    return plan_mean(a, &plan) == VMB_OK ? mean_beside_transpose(a, plan, H, W) : -1;
+}
+
 int vmb_testing_force_full_plan(int shape, int chunks) {
     g_force_chunks.store(chunks, std::memory_order_relaxed);
     g_force_shape.store(shape < 0 ? -1 : shape, std::memory_order_relaxed);

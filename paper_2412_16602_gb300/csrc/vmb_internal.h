@@ -201,6 +201,7 @@ vmb_status launch_cross_merge(const void* ys, void* out, int B, int D, int H, in
 // otherwise 32 x 32 tiles.
 constexpr size_t kTransposeSmem = 33 * 1024;
 bool transpose_by_planes(const void* x, const void* xt, int H, int W, vmb_dtype dt);
+bool transpose_whole_vectors(const void* x, const void* xt, int H, int W, vmb_dtype dt);
 vmb_status launch_map_transpose(const void* x, void* xt, int B, int D, int H, int W, vmb_dtype dt, bool planes,
                                 cudaStream_t stream);
 // Whether the channel-mean scan of this plan runs beside the transpose by planes.

@@ -25,12 +25,15 @@ extern "C" {
  * vmb_testing_selection_buffers: operand buffers of a selection grid.
  * vmb_testing_full_plan: out = {tile shape, L-chunks, launched early} of a full scan
  *   (map 1: as vmb_ss2d_full_fwd), with u or x (off & 1) or delta (off & 2) one element
- *   past 16-byte alignment.  Returns the status. */
+ *   past 16-byte alignment.  Returns the status.
+ * vmb_testing_mean_beside: 1 if the channel-mean scan of a block from the map runs beside
+ *   the transpose by planes, with x one element past 16-byte alignment (off 1); -1: no plan. */
 int vmb_testing_csm_kernel(int merge, vmb_dtype dtype, long long planes, int H, int W, int aligned, int sms);
 int vmb_testing_mean_two_steps(long long ctas, int D, long long res_one, long long res_two, int sms, int with_y);
 int vmb_testing_selection_buffers(long long grid, int D, int sms);
 int vmb_testing_full_plan(int B, int K, int D, int N, int H, int W, unsigned flags, vmb_dtype dtype, int map, int off,
                           int* out);
+int vmb_testing_mean_beside(int B, int D, int N, int H, int W, vmb_dtype dtype, int off);
 
 /* Force the full scan's tile shape (0..23 for 16 states; taken modulo the
  * number of shapes of the padded state count) and, for the look-back and

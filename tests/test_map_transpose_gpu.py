@@ -88,6 +88,22 @@ def test_calls_in_a_row_on_the_same_buffers(case, plan, force_plan):
         assert all(torch.equal(a, b) for a, b in zip(outs, want[rep % 4])), rep
 
 
+@pytest.mark.parametrize("case,beside", [
+    # (B, D, N, H, W, dtype, x out of line): 16 states in at most a CTA per SM, four states, two CTAs per SM
+    ((1, 1536, 16, 32, 32, "f32", 0), 1), ((1, 1536, 16, 28, 20, "bf16", 1), 1), ((1, 1536, 4, 32, 32, "f32", 0), 0),
+    ((2, 1024, 16, 30, 30, "f32", 0), 0), ((1, 1024, 4, 48, 72, "f32", 0), 1), ((1, 1024, 4, 48, 72, "f32", 1), 0),
+    ((1, 1024, 8, 28, 28, "f32", 0), 1), ((1, 1536, 8, 30, 30, "f32", 0), 0), ((1, 1536, 8, 32, 32, "bf16", 0), 1),
+    ((2, 1024, 16, 22, 48, "f32", 1), 0), ((8, 1024, 16, 28, 28, "f32", 0), 1), ((1, 1536, 16, 10, 10, "f32", 0), 1),
+])
+def test_mean_scan_beside_the_transpose(case, beside):
+    import ctypes
+
+    i = ctypes.c_int
+    vmb.lib.vmb_testing_mean_beside.argtypes = [i] * 7
+    B, D, N, H, W, dt, off = case
+    assert vmb.lib.vmb_testing_mean_beside(B, D, N, H, W, vmb.VMB_F32 if dt == "f32" else vmb.VMB_BF16, off) == beside
+
+
 def test_mean_block_of_many_maps_in_a_row():
     """Enough CTAs that the channel-mean scan starts beside the transpose by planes."""
     B, D, H, W = 40, 24, 24, 28
