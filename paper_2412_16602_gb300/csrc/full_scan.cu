@@ -1866,10 +1866,11 @@ vmb_status plan_full(const ScanArgs& a, ScanPlan* plan) {
     // Up to 1024 steps the lane-per-state kernel takes 3.2 us and 33.5 ns a step whatever the
     // rows (few enough), the three launches about 8 us and 42 ns a CTA on 152 SMs, and their
     // tiles of 64 channels are mostly padding where a sequence has few (fp32, us: 19 maps
-    // of 20x20x7 16.2 and 29.0; 7 of 32x32x32 37.2 and 25.5)
+    // of 20x20x7 16.2 and 29.0; 7 of 32x32x32 37.2 and 25.5; one direction of 21
+    // of 20x20x24 bf16, 147 CTAs, 14.6 and 12.9)
     auto chunk_beats_lanes = [&]() -> bool {
         const long long n = chunk_ctas();
-        return n >= 0 && (a.L > 1024 || 15200 * n <= (86LL * a.L - 20000) * sms);
+        return n >= 0 && (a.L > 1024 || 15200 * n <= (83LL * a.L - 16000) * sms);
     };
     int shape = 0, n_chunks = 1, forced_chunks = 0, forced_shape = 0;
     KernelInfo ki{};

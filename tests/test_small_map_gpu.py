@@ -100,6 +100,7 @@ LANES, PACKED, ONE, FOUR, SIXTEEN = 7, 16, 20, 21, 22
     ((71, 32, 7, 29, "f32"), LANES, LANES), ((44, 32, 13, 23, "bf16"), LANES, LANES),
     # few channels per sequence: tiles of the chunked three launches would be mostly padding
     ((19, 7, 20, 20, "f32"), LANES, LANES), ((7, 32, 20, 20, "bf16"), LANES, LANES), ((7, 32, 32, 32, "f32"), 9, 9),
+    ((6, 24, 20, 20, "bf16"), 9, 9),
     # the scan alone, rows out of line
     ((16, 32, 7, 29, "bf16"), FOUR, LANES), ((16, 32, 7, 29, "f32"), FOUR, LANES), ((110, 7, 7, 29, "f32"), FOUR, FOUR),
     ((49, 400, 9, 9, "bf16"), ONE, PACKED), ((49, 400, 9, 9, "f32"), ONE, ONE), ((40, 400, 9, 9, "bf16"), ONE, ONE),
