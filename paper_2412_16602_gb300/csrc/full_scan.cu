@@ -1756,14 +1756,15 @@ int small_rule(const ScanArgs& a, bool map, bool seq_ok, int sms) {
 // 6.5 and 5.4, of 96 steps 7.0 and 9.9; 64 of 128 steps 18.0 and 15.5.  bf16: 16 rows per SM of
 // 224 steps 9.5 and 27.5, 52 of 80 steps 11.2 and 15.9.  Element by element (rows counted with the
 // padding to CTAs of 16 channels), fp32: 5 rows per SM of 143 steps 8.5 and 7.1; 10 of 143 8.6 and
-// 10.0, of 203 11.4 and 18.7; 20 of 35 steps 5.9 and 5.2, of 203 16.1 and 18.7; 46 of 203 21.4 and 18.9.
+// 10.0, of 203 11.4 and 18.7; 20 of 35 steps 5.9 and 5.2, of 203 16.1 and 18.7; 21 of 176, more than
+// half of them padding (7 channels), 12.9 and 10.9; 46 of 203 21.4 and 18.9.
 // bf16: 5 of 143 steps 8.7 and 10.9, 20 of 203 15.4 and 31.0, 46 20.3 and 29.9; 60 of 35 9.5 and 8.2.
 bool lanes_beat_small(const ScanArgs& a, bool seq_ok, int sms) {
     const int L = a.L, staged = (L + 31) / 32 * 32;
     if (!seq_ok) {
         const long long rows = (long long)a.B * a.K * ((a.D + 15) / 16 * 16);
         if (a.dtype == VMB_BF16) return L >= 16 && rows <= 48LL * sms;
-        return rows > 8LL * sms && rows <= 24LL * sms && L >= 16 && 8 * staged <= 13 * L;
+        return rows > 8LL * sms && rows <= 24LL * sms && 3 * rows <= 4LL * a.B * a.K * a.D && L >= 16 && 8 * staged <= 13 * L;
     }
     const long long rows = (long long)a.B * a.K * a.D;
     if (a.dtype == VMB_BF16) return L >= 16;

@@ -103,6 +103,7 @@ LANES, PACKED, ONE, FOUR, SIXTEEN = 7, 16, 20, 21, 22
     ((6, 24, 20, 20, "bf16"), 9, 9),
     # the scan alone, rows out of line
     ((16, 32, 7, 29, "bf16"), FOUR, LANES), ((16, 32, 7, 29, "f32"), FOUR, LANES), ((110, 7, 7, 29, "f32"), FOUR, FOUR),
+    ((51, 7, 13, 13, "f32"), SIXTEEN, SIXTEEN), ((51, 7, 13, 13, "bf16"), SIXTEEN, LANES),
     ((49, 400, 9, 9, "bf16"), ONE, PACKED), ((49, 400, 9, 9, "f32"), ONE, ONE), ((40, 400, 9, 9, "bf16"), ONE, ONE),
 ])
 def test_planner_of_short_sequences(case, map_shape, scan_shape, full_plan):
